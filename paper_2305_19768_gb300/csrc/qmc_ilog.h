@@ -8,7 +8,8 @@
 //   x = 2^e m, m in [1, 2); F = 1 + j/1024 nearest to m (j = 0..1024);
 //   f = (m - F)/F, |f| <= 2^-11, held as f 2^74 in an int64;
 //   log1p(f) = f (1 - f c(f)),  c(f) = 1/2 - f/3 + f^2/4 - f^3/5 + f^4/6
-//     (truncation below 2^-79 relative), c by Horner in Q63;
+//     (truncation below 2^-58 relative), c by Horner, each coefficient to
+//     the bits that its weight leaves visible (Q32 inside, Q63 outside);
 //   ln x = e ln2 + ln F + log1p(f), summed in a signed 128-bit Q116 number
 //     (|ln x| < 745 < 2^9.6, and the smallest nonzero result, near x = 1,
 //     still has 64 significant bits), and rounded once to nearest-even.
@@ -32,11 +33,11 @@
 
 #define QMC_ILOG_LN2_LO 0x9abc9e3b39803f2fULL   // RN(2^116 ln 2), low word
 #define QMC_ILOG_LN2_HI 0xb17217f7d1cf7ULL      //                  high word
-#define QMC_ILOG_C2 0x4000000000000000LL        // RN(2^63 / k), k = 2..6
-#define QMC_ILOG_C3 0x2aaaaaaaaaaaaaabLL
-#define QMC_ILOG_C4 0x2000000000000000LL
-#define QMC_ILOG_C5 0x199999999999999aLL
-#define QMC_ILOG_C6 0x1555555555555555LL
+#define QMC_ILOG_C2 0x4000000000000000ULL       // RN(2^63 / k), k = 2, 3
+#define QMC_ILOG_C3 0x2aaaaaaaaaaaaaabULL
+#define QMC_ILOG_C4_32 0x40000000u              // RN(2^32 / k), k = 4, 5, 6
+#define QMC_ILOG_C5_32 0x33333333u
+#define QMC_ILOG_C6_32 0x2aaaaaabu
 
 typedef unsigned __int128 qmc_u128;
 
@@ -65,6 +66,22 @@ QMC_HD int qmc_clz64(uint64_t x) {
     return x ? __builtin_clzll(x) : 64;
 #endif
 }
+// high words of the unsigned 32- and 64-bit products (about 4 and 16 issue
+// cycles per warp on this GPU; the signed 64-bit form takes 27)
+QMC_HD uint32_t qmc_umulhi32(uint32_t a, uint32_t b) {
+#if defined(__CUDA_ARCH__)
+    return __umulhi(a, b);
+#else
+    return (uint32_t)(((uint64_t)a * b) >> 32);
+#endif
+}
+QMC_HD uint64_t qmc_umulhi64(uint64_t a, uint64_t b) {
+#if defined(__CUDA_ARCH__)
+    return __umul64hi(a, b);
+#else
+    return (uint64_t)(((qmc_u128)a * b) >> 64);
+#endif
+}
 // high 64 bits of the signed 128-bit product
 QMC_HD int64_t qmc_smulhi(int64_t a, int64_t b) {
 #if defined(__CUDA_ARCH__)
@@ -84,17 +101,30 @@ QMC_HD double qmc_ilog_core(int e, uint64_t frac63, const uint64_t *tab) {
     const uint64_t ra = fneg ? (uint64_t)(-ri) : (uint64_t)ri;
     // |f| 2^74 = |m - F| 2^63 RN(2^63/F) 2^-52 (truncated; exact for F = 1, 2)
     const uint64_t fm = (uint64_t)(((qmc_u128)ra * tab[3 * j]) >> 52);
-    const int64_t fq = fneg ? -(int64_t)fm : (int64_t)fm;
-    // c(f) in Q63: each step c <- C_k - f c, with f c = (f 2^74)(c 2^63) 2^-74
-    int64_t c = QMC_ILOG_C6;
-    c = QMC_ILOG_C5 - (qmc_smulhi(fq, c) >> 10);
-    c = QMC_ILOG_C4 - (qmc_smulhi(fq, c) >> 10);
-    c = QMC_ILOG_C3 - (qmc_smulhi(fq, c) >> 10);
-    c = QMC_ILOG_C2 - (qmc_smulhi(fq, c) >> 10);
-    const uint64_t h = (1ULL << 63) - (uint64_t)(qmc_smulhi(fq, c) >> 10);   // (1 - f c) 2^63
+    // c(f) by Horner on |f| with the sign of f carried into each sum. c enters
+    // log1p with weight f^2 <= 2^-22 relative, and each inner coefficient with
+    // one more factor 2^-11, so the inner two run in Q32 (c4 within 2^-30),
+    // 1/3 - f c4 in Q63 from a 32 x 32 product (within 2^-42: 2^-64 of
+    // log1p), and only the outer two products take 64 x 64 bits.
+    const uint32_t f32 = (uint32_t)(fm >> 31);                    // |f| 2^43
+    const uint32_t t6 = qmc_umulhi32(f32, QMC_ILOG_C6_32) >> 11;
+    const uint32_t c5 = fneg ? QMC_ILOG_C5_32 + t6 : QMC_ILOG_C5_32 - t6;
+    const uint32_t t5 = qmc_umulhi32(f32, c5) >> 11;
+    const uint32_t c4 = fneg ? QMC_ILOG_C4_32 + t5 : QMC_ILOG_C4_32 - t5;
+    const uint64_t t4 = ((uint64_t)f32 * c4) >> 12;
+    const uint64_t c3 = fneg ? QMC_ILOG_C3 + t4 : QMC_ILOG_C3 - t4;
+    const uint64_t t3 = qmc_umulhi64(fm, c3) >> 10;
+    const uint64_t c = fneg ? QMC_ILOG_C2 + t3 : QMC_ILOG_C2 - t3;
+    const uint64_t t2 = qmc_umulhi64(fm, c) >> 10;
+    const uint64_t h = fneg ? (1ULL << 63) + t2 : (1ULL << 63) - t2;   // (1 - f c) 2^63
     const qmc_u128 lp = ((qmc_u128)fm * h) >> 21;     // |log1p f| 2^116
-    const uint64_t ea = (uint64_t)(e < 0 ? -e : e);
-    const qmc_u128 el = (qmc_u128)ea * QMC_ILOG_LN2_LO + ((qmc_u128)(ea * QMC_ILOG_LN2_HI) << 64);
+    // |e| RN(2^116 ln 2): |e| < 2^11, four 32-bit words
+    const uint32_t ea = (uint32_t)(e < 0 ? -e : e);
+    const uint64_t p0 = (uint64_t)ea * (uint32_t)QMC_ILOG_LN2_LO;
+    const uint64_t p1 = (uint64_t)ea * (uint32_t)(QMC_ILOG_LN2_LO >> 32) + (p0 >> 32);
+    const uint64_t p2 = (uint64_t)ea * (uint32_t)QMC_ILOG_LN2_HI + (p1 >> 32);
+    const uint64_t elh = (((uint64_t)ea * (uint32_t)(QMC_ILOG_LN2_HI >> 32)) << 32) + p2;
+    const qmc_u128 el = ((qmc_u128)elh << 64) | ((p1 << 32) | (uint32_t)p0);
     const qmc_u128 lf = ((qmc_u128)tab[3 * j + 2] << 64) | tab[3 * j + 1];
     qmc_u128 S = lf + (fneg ? (qmc_u128)0 - lp : lp) + (e < 0 ? (qmc_u128)0 - el : el);   // mod 2^128
     const bool neg = (uint64_t)(S >> 127) != 0;

@@ -28,14 +28,6 @@ struct qmc_xf {
 
 #define QMC_XF_ZERO_E (-(1 << 20))   // exponent of a zero (below every nonzero value's)
 
-QMC_HD uint64_t qmc_umulhi(uint64_t a, uint64_t b) {
-#if defined(__CUDA_ARCH__)
-    return __umul64hi(a, b);
-#else
-    return (uint64_t)(((qmc_u128)a * b) >> 64);
-#endif
-}
-
 QMC_HD qmc_xf qmc_xf_one() { return qmc_xf{1ULL << 63, 0, 0}; }
 
 // x (finite double) as xf: exact
@@ -51,7 +43,7 @@ QMC_HD qmc_xf qmc_xf_of(double x) {
 }
 
 QMC_HD qmc_xf qmc_xf_mul(qmc_xf a, qmc_xf b) {
-    const uint64_t h = qmc_umulhi(a.m, b.m);
+    const uint64_t h = qmc_umulhi64(a.m, b.m);
     const int top = (int)(h >> 63);
     qmc_xf r;
     r.m = top ? h : (h << 1);
@@ -95,10 +87,12 @@ QMC_HD qmc_xf qmc_xf_neg(qmc_xf a) {
     return a;
 }
 
-// 1/a (a nonzero): Newton-Raphson y <- y + y (1 - m y) on m = a.m 2^-64 in
-// [1/2, 1), y in Q62, from an FP32 reciprocal of the top 24 bits (error
-// about 2^-22), two steps (2^-44, then the Q62 resolution). Relative error
-// below 2^-59.
+// 1/a (a nonzero): with m = a.m 2^-64 in [1/2, 1) and the hardware's FP32
+// reciprocal y0 of its top 24 bits (24 bits itself, m y0 = 1 - e with
+// |e| < 2^-21), 1/m = y0 (1 + e + e^2) within e^3 < 2^-63: one step of third
+// order. y0 has 24 bits, so m y0 takes two 32 x 32 products and is exact, and
+// y0 (e + e^2) two more (a second-order pair of steps in 64 x 64
+// bits took four high products). Relative error below 2^-61.
 QMC_HD qmc_xf qmc_xf_rcp(qmc_xf a) {
     qmc_xf r;
     r.neg = a.neg;
@@ -119,17 +113,20 @@ QMC_HD qmc_xf qmc_xf_rcp(qmc_xf a) {
     uint32_t yb;
     memcpy(&yb, &y0, 4);
 #endif
-    // y0 in (1, 2]: Q62 from its bits (2.0 clamps just below 2^63)
-    int64_t Y = ((yb >> 23) & 0xFF) >= 128 ? (int64_t)0x7FFFFFFFFFFFFFFFLL
-                                           : (int64_t)((1ULL << 62) | ((uint64_t)(yb & 0x7FFFFFu) << 39));
-    for (int it = 0; it < 2; ++it) {
-        const int64_t P = (int64_t)qmc_umulhi(a.m, (uint64_t)Y);    // m y 2^62
-        const int64_t E = (int64_t)(1ULL << 62) - P;                 // (1 - m y) 2^62
-        Y += qmc_smulhi(Y, E) << 2;
-        if (Y < 0) Y = 0x7FFFFFFFFFFFFFFFLL;            // (never: y < 2)
-    }
-    // 1/|a| = y 2^(-a.e - 1) with y = Y 2^-62 in (1, 2)
-    r.m = (uint64_t)Y << 1;
+    // y0 in (1, 2]: Q23
+    const uint32_t Y0 = yb >= 0x40000000u ? (1u << 24) : ((yb & 0x7FFFFFu) | (1u << 23));
+    const uint64_t p0 = (uint64_t)(uint32_t)a.m * Y0;
+    const uint64_t p1 = (uint64_t)(uint32_t)(a.m >> 32) * Y0 + (p0 >> 32);       // m y0 in Q55
+    // e in Q63 (rounded down), |e| < 2^42
+    const int64_t E = (int64_t)(((1ULL << 55) - p1) << 8) - (int64_t)((uint32_t)p0 >> 24);
+    const int32_t eh = (int32_t)(E >> 12);                                     // Q51
+    const int64_t T = E + (((int64_t)eh * eh) >> 39);                          // e + e^2 in Q63
+    // y = y0 + y0 (e + e^2) in Q63, exact products of the two words of T (mod
+    // 2^64: y0 = 2 wraps and y0 T < 0 brings it back below 2)
+    const uint64_t Y = ((uint64_t)Y0 << 40) + ((uint64_t)((int64_t)(int32_t)(T >> 32) * (int64_t)Y0) << 9) +
+                       (((uint64_t)(uint32_t)T * Y0) >> 23);
+    // 1/|a| = y 2^(-a.e - 1) with y in (1, 2)
+    r.m = Y;
     r.e = -a.e - 1;
     return r;
 }
