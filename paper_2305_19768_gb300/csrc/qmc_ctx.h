@@ -73,6 +73,7 @@ struct qmc_ctx {
     int tuned_ppt[QMC_NCLASS] = {};
     double presample_evals = 0.0;       // lattice points x shifts spent in qmc_presample_lambda
     bool host_only = false;             // QMC_DEVICE_NONE: no GPU, caller-supplied evaluator only
+    uint64_t kin_version = 0;           // counts qmc_set_kinematics calls
     std::vector<double> h_kin;          // host copy of the kinematics [npoints][ninv]
     // coefficients of qmc_set_coefficients: [npoints][namp][nint][ncoef]
     int coef_namp = 0, coef_npoints = 0, coef_nint = 0, coef_lo = 0, coef_n = 0;
@@ -95,11 +96,19 @@ struct ClassLaunch {
     unsigned int *d_jobfail = nullptr;   // per-job sign-check failures
     std::vector<int> orig;               // caller's index of each class-local job
     int block = 128, ppt = 16, grid = 0;
+    // jobs for the integer evaluator (qmc_real.cuh); `general`: the kinematics
+    // set since no longer qualify, the general kernel runs instead
+    bool fx = false, general = false;
+    struct FxJob {
+        int integral, sector, point;
+    };
+    std::vector<FxJob> fx_jobs;          // per class-local job
 };
 
 struct qmc_plan {
     qmc_ctx *ctx = nullptr;
     int lo = 0, norders = 0, njobs = 0;
+    uint64_t kin_version = 0;            // the kinematics its launches were chosen for
     double evals = 0.0;                  // lattice points x shifts of one run
     size_t out_size = 0;
     double *d_out = nullptr;

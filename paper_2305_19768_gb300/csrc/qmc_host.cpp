@@ -331,6 +331,8 @@ int pack_sector(qmc_ctx *ctx, const HostSector &S, int si, int ninv, std::vector
     }
     if ((int)local.size() > QMC_MAXMONO)
         return fail(ctx, QMC_E_INVAL, "sector %d: %zu monomials > %d", si, local.size(), QMC_MAXMONO);
+    H.weight_b = S.weight;
+    for (int qq = 0; qq < S.ns; ++qq) H.weight_b /= S.b[H.sing[qq]];
     H.pad0 = std::max(emax, 1);
     for (int j = 0; j < S.d; ++j)
         if (S.a[j] > 0) H.pad0 = std::max(H.pad0, S.a[j]);
@@ -369,6 +371,61 @@ int upload_tables(qmc_ctx *ctx) {
                              cudaMemcpyHostToDevice));
     ctx->nsectors_dev = (int)secs.size();
     return QMC_OK;
+}
+
+// Whether a job qualifies for the integer evaluator (qmc_real.cuh): a real
+// class, small integer exponents, and U and F with coefficients >= 0 at its
+// kinematic point and a constant term of at least 1/128 of their sum (fixed
+// point then holds every corner value to FP64's precision).
+bool fx_job_ok(const qmc_ctx *ctx, const HostSector &S, int cls, int point) {
+    if (cls != QMC_CLASS_REAL3 && cls != QMC_CLASS_REAL3M && cls != QMC_CLASS_REAL6 && cls != QMC_CLASS_REAL6M)
+        return false;
+    for (double x : {S.u0, S.u1, S.f0, S.f1})
+        if (x != (double)(int)x || std::abs(x) > QMC_EMAX) return false;
+    for (int j = 0; j < S.d; ++j)
+        if (S.a[j] > QMC_EMAX || (S.a[j] <= -1 && S.b[j] == 0.0)) return false;
+    const size_t ninv = (size_t)ctx->ninv;
+    if ((size_t)point * ninv + ninv > ctx->h_kin.size() && ninv > 0) return false;
+    const double *kin = ctx->h_kin.data() + (size_t)point * ninv;
+    for (const std::vector<Term> *P : {&S.U, &S.F}) {
+        double sum = 0.0, c0 = 0.0;
+        for (const Term &T : *P) {
+            double v = T.c[0];
+            for (size_t i = 0; i < ninv && i + 1 < QMC_NCOEF; ++i) v = std::fma(T.c[i + 1], kin[i], v);
+            if (!(v >= 0.0)) return false;
+            sum += v;
+            bool constant = true;
+            for (int j = 0; j < S.d; ++j) constant = constant && T.e[j] == 0;
+            if (constant) c0 += v;
+        }
+        if (!(c0 > 1e-100) || !(sum < 1e100) || !(sum <= 128.0 * c0)) return false;
+    }
+    return true;
+}
+
+// Points per thread of a launch by qmc_real.cuh or qmc_deformed.cuh: the
+// estimate (waves of `resident` tiles) x (points + 3), the 3 for a tile's
+// staging and lattice set-up, over the tiles that the lattices' sizes give.
+// Few tiles: small ones, so that every SM works (one shift of a pilot lattice
+// would otherwise keep a few blocks busy for 16 points a thread); many: the
+// size that leaves the fewest threads of the last tile of a lattice idle.
+int fx_points_per_thread(const std::vector<QmcJobDev> &jobs, int block, uint64_t resident) {
+    std::map<uint64_t, uint64_t> shifts;             // lattice size -> shifts
+    for (const QmcJobDev &D : jobs) shifts[D.n] += (uint64_t)D.shifts;
+    int best = 1;
+    double best_cost = 0.0;
+    for (int ppt = 1; ppt <= 32; ++ppt) {
+        const uint64_t tile = (uint64_t)block * ppt;
+        double tiles = 0.0;
+        for (const auto &x : shifts) tiles += (double)((x.first + tile - 1) / tile) * (double)x.second;
+        const double waves = tiles <= (double)resident ? 1.0 : tiles / (double)resident + 0.5;
+        const double cost = waves * (ppt + 3.0);
+        if (ppt == 1 || cost < best_cost) {
+            best = ppt;
+            best_cost = cost;
+        }
+    }
+    return best;
 }
 
 void free_plan_buffers(qmc_plan *p) {
@@ -539,6 +596,7 @@ int qmc_set_kinematics(qmc_ctx *ctx, const double *inv, int npoints, int ninv) {
     for (size_t i = 0; i < (size_t)npoints * ninv; ++i)
         if (!std::isfinite(inv[i])) return fail(ctx, QMC_E_INVAL, "non-finite invariant at %zu", i);
     ctx->h_kin.assign(inv, inv + (size_t)npoints * ninv);
+    ++ctx->kin_version;
     if (ctx->host_only) {
         ctx->npoints = npoints;
         ctx->ninv = ninv;
@@ -565,8 +623,10 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
     if (ctx->host_only) return fail(ctx, QMC_E_CUDA, "qmc_plan_create: host-only context (no GPU)");
     cudaSetDevice(ctx->device);
     const int hi = lo + norders - 1;
-    std::vector<std::vector<QmcJobDev>> per(QMC_NCLASS);
-    std::vector<std::vector<int>> per_orig(QMC_NCLASS);
+    // launches: per class, the jobs of the general kernels and (odd slots)
+    // those of the integer evaluator
+    std::vector<std::vector<QmcJobDev>> per(2 * QMC_NCLASS);
+    std::vector<std::vector<int>> per_orig(2 * QMC_NCLASS);
     uint64_t out_off = 0;
     double evals = 0.0;
     for (int i = 0; i < njobs; ++i) {
@@ -619,8 +679,9 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         D.flags = J.flags & QMC_JOB_UNSHIFTED;
         out_off += (uint64_t)J.shifts * norders * 2;
         evals += (double)J.n * J.shifts;
-        per[cls].push_back(D);
-        per_orig[cls].push_back(i);
+        const int slot = 2 * cls + (hi == 0 && fx_job_ok(ctx, S, cls, J.point) ? 1 : 0);
+        per[slot].push_back(D);
+        per_orig[slot].push_back(i);
     }
     qmc_plan *p = new qmc_plan();
     p->ctx = ctx;
@@ -645,8 +706,9 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
     PLAN_TRY(cudaMemset(p->d_status, 0, 2 * sizeof(unsigned long long)));
     PLAN_TRY(cudaEventCreate(&p->ev0));
     PLAN_TRY(cudaEventCreate(&p->ev1));
-    for (int cls = 0; cls < QMC_NCLASS; ++cls) {
-        std::vector<QmcJobDev> &v = per[cls];
+    for (int slot = 0; slot < 2 * QMC_NCLASS; ++slot) {
+        const int cls = slot / 2;
+        std::vector<QmcJobDev> &v = per[slot];
         if (v.empty()) continue;
         // the tile queue hands out tiles in job order: costly jobs first (more
         // singular variables, larger lattices) shortens the tail of the launch,
@@ -655,7 +717,7 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
             std::vector<int> ord(v.size());
             for (size_t u = 0; u < ord.size(); ++u) ord[u] = (int)u;
             auto key = [&](int u) {
-                const qmc_job &J = jobs[per_orig[cls][u]];
+                const qmc_job &J = jobs[per_orig[slot][u]];
                 const int ns = ctx->integrals[J.integral_id].sectors[J.sector].ns;
                 return std::make_pair(ns, (double)v[u].n * v[u].shifts);
             };
@@ -664,14 +726,17 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
             std::vector<int> o2;
             for (int u : ord) {
                 v2.push_back(v[u]);
-                o2.push_back(per_orig[cls][u]);
+                o2.push_back(per_orig[slot][u]);
             }
             v.swap(v2);
-            per_orig[cls].swap(o2);
+            per_orig[slot].swap(o2);
         }
         ClassLaunch c;
         c.cls = cls;
-        c.orig = per_orig[cls];
+        c.orig = per_orig[slot];
+        c.fx = (slot & 1) != 0;
+        if (c.fx)
+            for (int u : c.orig) c.fx_jobs.push_back({jobs[u].integral_id, jobs[u].sector, jobs[u].point});
         c.block = ctx->opt.block == 256 ? 256 : (ctx->opt.block == 128 ? 128 : (ctx->tuned_block[cls] ? ctx->tuned_block[cls] : 128));
         if (qmc_class_dmax(cls) > 3) c.block = 128;   // the d <= 6 classes exist with 128-thread blocks only
         c.ppt = ctx->opt.ppt > 0 ? ctx->opt.ppt : (ctx->tuned_ppt[cls] ? ctx->tuned_ppt[cls] : 16);
@@ -681,6 +746,22 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
             uint64_t nmax = 0;
             for (const QmcJobDev &D : v) nmax = std::max<uint64_t>(nmax, D.n);
             if (nmax < 16384) c.ppt = 4;
+        }
+        // power-table rows: the largest exponent among the launch's sectors
+        // (fewer rows, less shared memory per block, more resident blocks)
+        int prow = 1, occ = 1;
+        for (int u : c.orig) {
+            const qmc_job &J = jobs[u];
+            prow = std::max(prow, ctx->integrals[J.integral_id].sectors[J.sector].prow);
+        }
+        if (c.fx) {
+            if (qmc_class_dmax(cls) > 3) c.block = QMC_FX6_BLOCK;
+            else if (ctx->opt.block != 128 && ctx->opt.block != 256 && !ctx->tuned_block[cls]) c.block = 256;
+            occ = std::max(1, qmc_k_occupancy_real(cls, c.block, prow));
+            if (ctx->opt.ppt <= 0 && !ctx->tuned_ppt[cls])
+                c.ppt = fx_points_per_thread(v, c.block, (uint64_t)ctx->sm_count * occ);
+        } else {
+            occ = std::max(1, qmc_k_occupancy(cls, c.block, prow));
         }
         const uint64_t tile_k = (uint64_t)c.block * c.ppt;
         uint64_t tiles = 0;
@@ -696,17 +777,7 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         PLAN_TRY(cudaMemset(c.d_queue, 0, sizeof(unsigned long long)));
         PLAN_TRY(cudaMalloc(&c.d_jobfail, v.size() * sizeof(unsigned int)));
         PLAN_TRY(cudaMemset(c.d_jobfail, 0, v.size() * sizeof(unsigned int)));
-        // power-table rows: the largest exponent among the launch's sectors
-        // (fewer rows, less shared memory per block, more resident blocks)
-        int prow = 1;
-        for (int u : c.orig) {
-            const qmc_job &J = jobs[u];
-            prow = std::max(prow, ctx->integrals[J.integral_id].sectors[J.sector].prow);
-        }
-        int occ = qmc_k_occupancy(cls, c.block, prow);
-        if (occ < 1) occ = 1;
-        c.grid = (int)std::min<uint64_t>(tiles, (uint64_t)ctx->sm_count * occ);
-        if (c.grid < 1) c.grid = 1;
+        c.grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(tiles, (uint64_t)ctx->sm_count * occ));
         QmcLaunch &L = c.L;
         L.sectors = ctx->d_sectors;
         L.monos = ctx->d_monos;
@@ -720,6 +791,8 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         L.tile_k = (uint32_t)tile_k;
         L.transform = ctx->opt.transform;
         L.prow = prow;
+        L.mone = -1.0;
+        L.nzero = -0.0;
         L.partials = c.d_partials;
         L.queue = c.d_queue;
         L.status = p->d_status;
@@ -748,6 +821,7 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         }
     }
 #undef PLAN_TRY
+    p->kin_version = ctx->kin_version;
     ctx->plans.push_back(p);
     *out = p;
     return QMC_OK;
@@ -777,7 +851,14 @@ int plan_enqueue(qmc_plan *plan, double *out, cudaStream_t st, bool capturing) {
         CUDA_TRY(ctx, cudaMemsetAsync(c.d_jobfail, 0, c.orig.size() * sizeof(unsigned int), cs));
         CUDA_TRY(ctx, cudaEventRecordWithFlags(plan->kev[2 * i], cs, evflags));
         if (c.L.ntiles > 0) {
-            if (qmc_k_launch_eval(c.cls, &c.L, c.block, c.ppt, c.grid, cs))
+            const bool fx = c.fx && !c.general;
+            // the general d <= 6 kernels exist with 128 threads only
+            const int gblock = c.fx && qmc_class_dmax(c.cls) > 3 ? 128 : c.block;
+            const int ggrid = fx || !c.fx ? c.grid
+                                    : (int)std::min<uint64_t>(c.L.ntiles, (uint64_t)ctx->sm_count *
+                                                                std::max(1, qmc_k_occupancy(c.cls, gblock, c.L.prow)));
+            if (fx ? qmc_k_launch_real(c.cls, &c.L, c.block, c.ppt, c.grid, cs)
+                   : qmc_k_launch_eval(c.cls, &c.L, gblock, (int)(c.L.tile_k / gblock), ggrid, cs))
                 return fail(ctx, QMC_E_CUDA, "evaluator launch failed: %s", cudaGetErrorString(cudaGetLastError()));
             ++launches;
         }
@@ -804,6 +885,18 @@ int qmc_plan_run(qmc_plan *plan, double *out_dev, void *stream) {
     cudaSetDevice(ctx->device);
     cudaStream_t st = stream ? (cudaStream_t)stream : ctx->stream;
     double *out = out_dev ? out_dev : plan->d_out;
+    if (plan->kin_version != ctx->kin_version) {
+        // new kinematics: the integer evaluator's jobs must still qualify, and
+        // a captured graph holds the old table's address
+        for (ClassLaunch &c : plan->launches) {
+            c.general = false;
+            for (const ClassLaunch::FxJob &J : c.fx_jobs)
+                c.general = c.general || !fx_job_ok(ctx, ctx->integrals[J.integral].sectors[J.sector], c.cls, J.point);
+        }
+        if (plan->gexec) cudaGraphExecDestroy(plan->gexec);
+        plan->gexec = nullptr;
+        plan->kin_version = ctx->kin_version;
+    }
     if (plan->use_graph) {
         if (!plan->gexec || plan->graph_out != out) {
             if (plan->gexec) cudaGraphExecDestroy(plan->gexec);
@@ -1120,6 +1213,7 @@ extern "C" int qmc_eval_jobs_noalloc(qmc_ctx *ctx, const qmc_job *jobs, int njob
     const uint64_t tile_k = (uint64_t)block * ppt;
     const int hi = lo + norders - 1;
     int cls = -1;
+    bool fx = hi == 0;   // every job qualifies for the integer evaluator
     uint64_t tiles = 0, out_off = 0;
     for (int i = 0; i < njobs; ++i) {
         const qmc_job &J = jobs[i];
@@ -1147,6 +1241,7 @@ extern "C" int qmc_eval_jobs_noalloc(qmc_ctx *ctx, const qmc_job *jobs, int njob
             return fail(ctx, QMC_E_INVAL, "qmc_eval_jobs_noalloc: all jobs must use one evaluator class");
         if (qmc_class_big(cls) || norders > qmc_class_lmax(cls) || hi + S.ns + 1 > qmc_class_lmax(cls))
             return fail(ctx, QMC_E_INVAL, "job %d: orders %d..%d not supported by the evaluator", i, lo, hi);
+        fx = fx && fx_job_ok(ctx, S, cls, J.point);
         QmcJobDev &D = recs[i];
         memset(&D, 0, sizeof D);
         D.sector = S.global_index;
@@ -1182,11 +1277,13 @@ extern "C" int qmc_eval_jobs_noalloc(qmc_ctx *ctx, const qmc_job *jobs, int njob
     L.ntiles = tiles;
     L.tile_k = (uint32_t)tile_k;
     L.transform = ctx->opt.transform;
+    L.mone = -1.0;
+    L.nzero = -0.0;
     L.prow = QMC_EMAX;   // the fixed launch shape: a table for every exponent
     L.out = out_dev;
     cudaStream_t st = stream ? (cudaStream_t)stream : ctx->stream;
     unsigned long long status[2] = {0, 0};
-    int rc = qmc_k_noalloc_eval(ctx->device, cls, recs, njobs, &L, block, ppt, ctx->sm_count, status, st);
+    int rc = qmc_k_noalloc_eval(ctx->device, cls, fx ? 1 : 0, recs, njobs, &L, block, ppt, ctx->sm_count, status, st);
     if (rc == -2) return fail(ctx, QMC_E_INVAL, "qmc_eval_jobs_noalloc: size beyond the fixed scratch");
     if (rc) return fail(ctx, QMC_E_CUDA, "qmc_eval_jobs_noalloc: %s", cudaGetErrorString(cudaGetLastError()));
     CUDA_TRY(ctx, cudaStreamSynchronize(st));

@@ -44,6 +44,7 @@ struct QmcSectorDev {
     double b[QMC_DMAX];
     double u0, u1, f0, f1;
     double weight;                          // constant factor of the sector
+    double weight_b;                        // weight times prod 1/b_j over the singular variables
 };
 
 // One evaluation job: (sector, kinematic point) with its lattice and shifts.
@@ -80,8 +81,14 @@ struct QmcLaunch {
     unsigned long long *queue;   // tile counter (reset by the finish kernel)
     unsigned long long *status;  // [0]: sign-check failures, [1]: non-finite partials
     double *out;           // per-shift sums
+    double mone, nzero;          // -1 and -0 (the integer evaluator adds and multiplies by FMA)
     unsigned int *job_fail;      // per-job sign-check failures (class-local job index) or null
 };
+
+// Threads per block of the d <= 6 integer evaluator
+#ifndef QMC_FX6_BLOCK
+#define QMC_FX6_BLOCK 384
+#endif
 
 // Fixed scratch of the no-allocation entry point (qmc_eval_jobs_noalloc).
 #define QMC_NOALLOC_BYTES (4u << 20)   // 4 MiB per device
@@ -135,8 +142,11 @@ int qmc_k_fp64_probe(double *out_dev, int iters, int grid, int block, void *stre
 int qmc_k_fp32_probe(float *out_dev, int iters, int grid, int block, void *stream);
 int qmc_k_sm_count(int device);
 int qmc_k_occupancy(int cls, int block, int prow);
+// the integer evaluator of the real classes (qmc_real.cuh), for jobs that qualify
+int qmc_k_launch_real(int cls, const QmcLaunch *L, int block, int ppt, int grid, void *stream);
+int qmc_k_occupancy_real(int cls, int block, int prow);
 size_t qmc_k_noalloc_partial_capacity(void);
 int qmc_k_noalloc_setup(int device, void **ptr);
-int qmc_k_noalloc_eval(int device, int cls, const QmcJobDev *jobs_host, int njobs, const QmcLaunch *tmpl,
+int qmc_k_noalloc_eval(int device, int cls, int fx, const QmcJobDev *jobs_host, int njobs, const QmcLaunch *tmpl,
                        int block, int ppt, int sm_count, unsigned long long *status_host, void *stream);
 }

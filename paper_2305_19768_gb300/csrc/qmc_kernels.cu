@@ -2841,16 +2841,55 @@ int occupancy_cls(int block, int prow) {
     return v;
 }
 
+#if QMC_PART >= 4
+#include "qmc_real.cuh"
+#endif
 }  // namespace
 
 // Per translation unit: the launcher and occupancy query of the classes it
 // instantiates (-2 / 0 for the others). The evaluator classes are compiled in
-// four translation units in parallel: part 0 the real d <= 3 classes (and
+// six translation units in parallel: part 0 the real d <= 3 classes (and
 // everything that is not an evaluator), part 1 the deformed classes, part 2
-// the d <= 6 classes, part 3 the Taylor-subtraction classes.
+// the d <= 6 classes, part 3 the Taylor-subtraction classes, parts 4 and 5
+// the integer evaluator (qmc_real.cuh) for d <= 3 and d <= 6.
 #define QMC_PART_FN2(name, part) name##_part##part
 #define QMC_PART_FN(name, part) QMC_PART_FN2(name, part)
 
+#if QMC_PART >= 4
+extern "C" int QMC_PART_FN(qmc_k_launch_real, QMC_PART)(int cls, const QmcLaunch *L, int block, int ppt, int grid,
+                                                         void *stream) {
+    cudaStream_t st = (cudaStream_t)stream;
+    switch (cls) {
+#if QMC_PART == 4
+        case QMC_CLASS_REAL3:
+            return block == 256 ? fx_launch<3, 2, 4, false, 256>(L, ppt, grid, st)
+                                : fx_launch<3, 2, 4, false, 128>(L, ppt, grid, st);
+        case QMC_CLASS_REAL3M:
+            return block == 256 ? fx_launch<3, 2, 4, true, 256>(L, ppt, grid, st)
+                                : fx_launch<3, 2, 4, true, 128>(L, ppt, grid, st);
+#else
+        case QMC_CLASS_REAL6: return fx_launch<6, 4, 6, false, QMC_FX6_BLOCK>(L, ppt, grid, st);
+        case QMC_CLASS_REAL6M: return fx_launch<6, 4, 6, true, QMC_FX6_BLOCK>(L, ppt, grid, st);
+#endif
+        default: return -2;
+    }
+}
+
+extern "C" int QMC_PART_FN(qmc_k_occupancy_real, QMC_PART)(int cls, int block, int prow) {
+    switch (cls) {
+#if QMC_PART == 4
+        case QMC_CLASS_REAL3:
+            return block == 256 ? fx_occupancy<3, 2, 4, false, 256>(prow) : fx_occupancy<3, 2, 4, false, 128>(prow);
+        case QMC_CLASS_REAL3M:
+            return block == 256 ? fx_occupancy<3, 2, 4, true, 256>(prow) : fx_occupancy<3, 2, 4, true, 128>(prow);
+#else
+        case QMC_CLASS_REAL6: return fx_occupancy<6, 4, 6, false, QMC_FX6_BLOCK>(prow);
+        case QMC_CLASS_REAL6M: return fx_occupancy<6, 4, 6, true, QMC_FX6_BLOCK>(prow);
+#endif
+        default: return 0;
+    }
+}
+#else
 extern "C" int QMC_PART_FN(qmc_k_launch_eval, QMC_PART)(int cls, const QmcLaunch *L, int block, int ppt, int grid,
                                                          void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
@@ -2902,6 +2941,7 @@ extern "C" int QMC_PART_FN(qmc_k_occupancy, QMC_PART)(int cls, int block, int pr
         default: return 0;
     }
 }
+#endif
 
 #if QMC_PART == 0
 extern "C" int qmc_k_launch_eval_part1(int, const QmcLaunch *, int, int, int, void *);
@@ -2910,6 +2950,21 @@ extern "C" int qmc_k_launch_eval_part3(int, const QmcLaunch *, int, int, int, vo
 extern "C" int qmc_k_occupancy_part1(int, int, int);
 extern "C" int qmc_k_occupancy_part2(int, int, int);
 extern "C" int qmc_k_occupancy_part3(int, int, int);
+
+extern "C" int qmc_k_launch_real_part4(int, const QmcLaunch *, int, int, int, void *);
+extern "C" int qmc_k_launch_real_part5(int, const QmcLaunch *, int, int, int, void *);
+extern "C" int qmc_k_occupancy_real_part4(int, int, int);
+extern "C" int qmc_k_occupancy_real_part5(int, int, int);
+
+extern "C" int qmc_k_launch_real(int cls, const QmcLaunch *L, int block, int ppt, int grid, void *stream) {
+    const int rc = qmc_k_launch_real_part4(cls, L, block, ppt, grid, stream);
+    return rc != -2 ? rc : qmc_k_launch_real_part5(cls, L, block, ppt, grid, stream);
+}
+
+extern "C" int qmc_k_occupancy_real(int cls, int block, int prow) {
+    const int v = qmc_k_occupancy_real_part4(cls, block, prow);
+    return v ? v : qmc_k_occupancy_real_part5(cls, block, prow);
+}
 
 extern "C" int qmc_k_launch_eval(int cls, const QmcLaunch *L, int block, int ppt, int grid, void *stream) {
     int (*const parts[4])(int, const QmcLaunch *, int, int, int, void *) = {
@@ -3026,10 +3081,11 @@ extern "C" int qmc_k_noalloc_setup(int device, void **ptr) {
     return 0;
 }
 
-// Queue the evaluation of `njobs` host job records of one kernel class into
+// Queue the evaluation of `njobs` host job records of one kernel class (fx:
+// all of them by the integer evaluator) into
 // the fixed scratch, then copy the status words to `status_host`. The caller
 // synchronises the stream before reading `status_host`.
-extern "C" int qmc_k_noalloc_eval(int device, int cls, const QmcJobDev *jobs_host, int njobs,
+extern "C" int qmc_k_noalloc_eval(int device, int cls, int fx, const QmcJobDev *jobs_host, int njobs,
                                   const QmcLaunch *tmpl, int block, int ppt, int sm_count,
                                   unsigned long long *status_host, void *stream) {
     void *base = nullptr;
@@ -3049,12 +3105,14 @@ extern "C" int qmc_k_noalloc_eval(int device, int cls, const QmcJobDev *jobs_hos
     if (cudaMemcpyAsync(b + kNoallocJobOff, jobs_host, (size_t)njobs * sizeof(QmcJobDev),
                         cudaMemcpyHostToDevice, st) != cudaSuccess)
         return -1;
-    int occ = qmc_k_occupancy(cls, block, L.prow);
+    int occ = fx ? qmc_k_occupancy_real(cls, block, L.prow) : qmc_k_occupancy(cls, block, L.prow);
     if (occ < 1) occ = 1;
     uint64_t g = (uint64_t)sm_count * occ;
     if (L.ntiles < g) g = L.ntiles;
     const int grid = g < 1 ? 1 : (int)g;
-    if (L.ntiles > 0 && qmc_k_launch_eval(cls, &L, block, ppt, grid, stream)) return -1;
+    if (L.ntiles > 0 && (fx ? qmc_k_launch_real(cls, &L, block, ppt, grid, stream)
+                            : qmc_k_launch_eval(cls, &L, block, ppt, grid, stream)))
+        return -1;
     if (qmc_k_launch_finish(&L, stream)) return -1;
     if (cudaMemcpyAsync(status_host, b + 64, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st) !=
         cudaSuccess)
