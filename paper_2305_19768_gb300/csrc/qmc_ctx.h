@@ -96,13 +96,13 @@ struct ClassLaunch {
     unsigned int *d_jobfail = nullptr;   // per-job sign-check failures
     std::vector<int> orig;               // caller's index of each class-local job
     int block = 128, ppt = 16, grid = 0;
-    // jobs for the integer evaluator (qmc_real.cuh); `general`: the kinematics
-    // set since no longer qualify, the general kernel runs instead
+    // jobs for the evaluators of qmc_real.cuh or qmc_deformed.cuh; `general`:
+    // the kinematics set since no longer qualify, the general kernel runs instead
     bool fx = false, general = false;
     struct FxJob {
         int integral, sector, point;
     };
-    std::vector<FxJob> fx_jobs;          // per class-local job
+    std::vector<FxJob> fx_jobs;          // the jobs whose kinematics must qualify
 };
 
 struct qmc_plan {

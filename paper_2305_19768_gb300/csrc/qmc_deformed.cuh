@@ -21,6 +21,12 @@
 //  * transform, weight, 1/t, ln t, reciprocals and logarithms run on the
 //    integer pipe, and the corners are folded variable by variable as in
 //    qmc_real.cuh (complex corner series, real factors).
+// Measured (evaluations/s, general kernel -> this one): massive box, 64 points
+// at n = 10007, 1.74e9 -> 5.9e9 (90 FP64 instructions per evaluation, pipe
+// 93 % busy); the same in mixed precision, 256 points at n = 1009,
+// 2.85e9 -> 5.4e9; massless box, 16 physical points at n = 4001, 5.9e8 ->
+// 1.06e9 (453, pipe 90 %). 16 warps (128 registers) beat 12 and 8 even with
+// the FP64 kernel's spills.
 // MIXED: derivatives of F and U(z), F(z) from FP32 monomial products in the
 // order of the general mixed kernel, everything after them in FP64.
 

@@ -428,6 +428,25 @@ int fx_points_per_thread(const std::vector<QmcJobDev> &jobs, int block, uint64_t
     return best;
 }
 
+// Whether a job qualifies for the deformed evaluator (qmc_deformed.cuh): a
+// deformed class with small integer exponents and, in FP64, F of total
+// degree <= 2 (whatever its coefficients)
+bool fd_job_ok(const HostSector &S, int cls) {
+    if (cls != QMC_CLASS_CPLX3 && cls != QMC_CLASS_CPLX3M) return false;
+    auto small_int = [](double x) { return x == (double)(int)x && std::abs(x) <= QMC_EMAX; };
+    for (double x : {S.u0, S.u1, S.f0, S.f1})
+        if (!small_int(x)) return false;
+    for (int j = 0; j < S.d; ++j)
+        if (!small_int(S.b[j]) || S.a[j] < -1 || S.a[j] > QMC_EMAX || (S.a[j] == -1 && S.b[j] == 0.0)) return false;
+    if (cls == QMC_CLASS_CPLX3M) return true;
+    for (const Term &T : S.F) {
+        int deg = 0;
+        for (int j = 0; j < S.d; ++j) deg += T.e[j];
+        if (deg > 2) return false;
+    }
+    return true;
+}
+
 void free_plan_buffers(qmc_plan *p) {
     for (ClassLaunch &c : p->launches) {
         cudaFree(c.d_jobs);
@@ -624,7 +643,7 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
     cudaSetDevice(ctx->device);
     const int hi = lo + norders - 1;
     // launches: per class, the jobs of the general kernels and (odd slots)
-    // those of the integer evaluator
+    // those of the evaluators of qmc_real.cuh and qmc_deformed.cuh
     std::vector<std::vector<QmcJobDev>> per(2 * QMC_NCLASS);
     std::vector<std::vector<int>> per_orig(2 * QMC_NCLASS);
     uint64_t out_off = 0;
@@ -679,7 +698,7 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         D.flags = J.flags & QMC_JOB_UNSHIFTED;
         out_off += (uint64_t)J.shifts * norders * 2;
         evals += (double)J.n * J.shifts;
-        const int slot = 2 * cls + (hi == 0 && fx_job_ok(ctx, S, cls, J.point) ? 1 : 0);
+        const int slot = 2 * cls + (hi == 0 && (fd_job_ok(S, cls) || fx_job_ok(ctx, S, cls, J.point)) ? 1 : 0);
         per[slot].push_back(D);
         per_orig[slot].push_back(i);
     }
@@ -735,7 +754,7 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         c.cls = cls;
         c.orig = per_orig[slot];
         c.fx = (slot & 1) != 0;
-        if (c.fx)
+        if (c.fx && cls != QMC_CLASS_CPLX3 && cls != QMC_CLASS_CPLX3M)
             for (int u : c.orig) c.fx_jobs.push_back({jobs[u].integral_id, jobs[u].sector, jobs[u].point});
         c.block = ctx->opt.block == 256 ? 256 : (ctx->opt.block == 128 ? 128 : (ctx->tuned_block[cls] ? ctx->tuned_block[cls] : 128));
         if (qmc_class_dmax(cls) > 3) c.block = 128;   // the d <= 6 classes exist with 128-thread blocks only
@@ -1213,7 +1232,7 @@ extern "C" int qmc_eval_jobs_noalloc(qmc_ctx *ctx, const qmc_job *jobs, int njob
     const uint64_t tile_k = (uint64_t)block * ppt;
     const int hi = lo + norders - 1;
     int cls = -1;
-    bool fx = hi == 0;   // every job qualifies for the integer evaluator
+    bool fx = hi == 0;   // every job qualifies for qmc_real.cuh or qmc_deformed.cuh
     uint64_t tiles = 0, out_off = 0;
     for (int i = 0; i < njobs; ++i) {
         const qmc_job &J = jobs[i];
@@ -1241,7 +1260,7 @@ extern "C" int qmc_eval_jobs_noalloc(qmc_ctx *ctx, const qmc_job *jobs, int njob
             return fail(ctx, QMC_E_INVAL, "qmc_eval_jobs_noalloc: all jobs must use one evaluator class");
         if (qmc_class_big(cls) || norders > qmc_class_lmax(cls) || hi + S.ns + 1 > qmc_class_lmax(cls))
             return fail(ctx, QMC_E_INVAL, "job %d: orders %d..%d not supported by the evaluator", i, lo, hi);
-        fx = fx && fx_job_ok(ctx, S, cls, J.point);
+        fx = fx && (fd_job_ok(S, cls) || fx_job_ok(ctx, S, cls, J.point));
         QmcJobDev &D = recs[i];
         memset(&D, 0, sizeof D);
         D.sector = S.global_index;

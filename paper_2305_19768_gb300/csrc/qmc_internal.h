@@ -142,7 +142,7 @@ int qmc_k_fp64_probe(double *out_dev, int iters, int grid, int block, void *stre
 int qmc_k_fp32_probe(float *out_dev, int iters, int grid, int block, void *stream);
 int qmc_k_sm_count(int device);
 int qmc_k_occupancy(int cls, int block, int prow);
-// the integer evaluator of the real classes (qmc_real.cuh), for jobs that qualify
+// the evaluators of qmc_real.cuh and qmc_deformed.cuh, for jobs that qualify
 int qmc_k_launch_real(int cls, const QmcLaunch *L, int block, int ppt, int grid, void *stream);
 int qmc_k_occupancy_real(int cls, int block, int prow);
 size_t qmc_k_noalloc_partial_capacity(void);

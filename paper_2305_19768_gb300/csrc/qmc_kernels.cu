@@ -2844,14 +2844,18 @@ int occupancy_cls(int block, int prow) {
 #if QMC_PART >= 4
 #include "qmc_real.cuh"
 #endif
+#if QMC_PART == 6
+#include "qmc_deformed.cuh"
+#endif
 }  // namespace
 
 // Per translation unit: the launcher and occupancy query of the classes it
 // instantiates (-2 / 0 for the others). The evaluator classes are compiled in
-// six translation units in parallel: part 0 the real d <= 3 classes (and
+// seven translation units in parallel: part 0 the real d <= 3 classes (and
 // everything that is not an evaluator), part 1 the deformed classes, part 2
 // the d <= 6 classes, part 3 the Taylor-subtraction classes, parts 4 and 5
-// the integer evaluator (qmc_real.cuh) for d <= 3 and d <= 6.
+// the integer evaluator (qmc_real.cuh) for d <= 3 and d <= 6, part 6 the
+// deformed evaluator of qmc_deformed.cuh.
 #define QMC_PART_FN2(name, part) name##_part##part
 #define QMC_PART_FN(name, part) QMC_PART_FN2(name, part)
 
@@ -2867,6 +2871,11 @@ extern "C" int QMC_PART_FN(qmc_k_launch_real, QMC_PART)(int cls, const QmcLaunch
         case QMC_CLASS_REAL3M:
             return block == 256 ? fx_launch<3, 2, 4, true, 256>(L, ppt, grid, st)
                                 : fx_launch<3, 2, 4, true, 128>(L, ppt, grid, st);
+#elif QMC_PART == 6
+        case QMC_CLASS_CPLX3:
+            return block == 256 ? fd_launch<false, 256>(L, ppt, grid, st) : fd_launch<false, 128>(L, ppt, grid, st);
+        case QMC_CLASS_CPLX3M:
+            return block == 256 ? fd_launch<true, 256>(L, ppt, grid, st) : fd_launch<true, 128>(L, ppt, grid, st);
 #else
         case QMC_CLASS_REAL6: return fx_launch<6, 4, 6, false, QMC_FX6_BLOCK>(L, ppt, grid, st);
         case QMC_CLASS_REAL6M: return fx_launch<6, 4, 6, true, QMC_FX6_BLOCK>(L, ppt, grid, st);
@@ -2882,6 +2891,9 @@ extern "C" int QMC_PART_FN(qmc_k_occupancy_real, QMC_PART)(int cls, int block, i
             return block == 256 ? fx_occupancy<3, 2, 4, false, 256>(prow) : fx_occupancy<3, 2, 4, false, 128>(prow);
         case QMC_CLASS_REAL3M:
             return block == 256 ? fx_occupancy<3, 2, 4, true, 256>(prow) : fx_occupancy<3, 2, 4, true, 128>(prow);
+#elif QMC_PART == 6
+        case QMC_CLASS_CPLX3: return block == 256 ? fd_occupancy<false, 256>(prow) : fd_occupancy<false, 128>(prow);
+        case QMC_CLASS_CPLX3M: return block == 256 ? fd_occupancy<true, 256>(prow) : fd_occupancy<true, 128>(prow);
 #else
         case QMC_CLASS_REAL6: return fx_occupancy<6, 4, 6, false, QMC_FX6_BLOCK>(prow);
         case QMC_CLASS_REAL6M: return fx_occupancy<6, 4, 6, true, QMC_FX6_BLOCK>(prow);
@@ -2953,17 +2965,25 @@ extern "C" int qmc_k_occupancy_part3(int, int, int);
 
 extern "C" int qmc_k_launch_real_part4(int, const QmcLaunch *, int, int, int, void *);
 extern "C" int qmc_k_launch_real_part5(int, const QmcLaunch *, int, int, int, void *);
+extern "C" int qmc_k_launch_real_part6(int, const QmcLaunch *, int, int, int, void *);
 extern "C" int qmc_k_occupancy_real_part4(int, int, int);
 extern "C" int qmc_k_occupancy_real_part5(int, int, int);
+extern "C" int qmc_k_occupancy_real_part6(int, int, int);
 
 extern "C" int qmc_k_launch_real(int cls, const QmcLaunch *L, int block, int ppt, int grid, void *stream) {
-    const int rc = qmc_k_launch_real_part4(cls, L, block, ppt, grid, stream);
-    return rc != -2 ? rc : qmc_k_launch_real_part5(cls, L, block, ppt, grid, stream);
+    for (auto f : {qmc_k_launch_real_part4, qmc_k_launch_real_part5, qmc_k_launch_real_part6}) {
+        const int rc = f(cls, L, block, ppt, grid, stream);
+        if (rc != -2) return rc;
+    }
+    return -2;
 }
 
 extern "C" int qmc_k_occupancy_real(int cls, int block, int prow) {
-    const int v = qmc_k_occupancy_real_part4(cls, block, prow);
-    return v ? v : qmc_k_occupancy_real_part5(cls, block, prow);
+    for (auto f : {qmc_k_occupancy_real_part4, qmc_k_occupancy_real_part5, qmc_k_occupancy_real_part6}) {
+        const int v = f(cls, block, prow);
+        if (v) return v;
+    }
+    return 0;
 }
 
 extern "C" int qmc_k_launch_eval(int cls, const QmcLaunch *L, int block, int ppt, int grid, void *stream) {
