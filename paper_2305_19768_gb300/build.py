@@ -17,10 +17,10 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libqmc.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-# the evaluator's instantiations are split over seven translation units
-# (qmc_kernels.cu and the six part files that include it) compiled in parallel
+# the evaluator's instantiations are split over eight translation units
+# (qmc_kernels.cu and the seven part files that include it) compiled in parallel
 SOURCES = ["qmc_kernels_wide.cu", "qmc_kernels_cplx.cu", "qmc_kernels.cu", "qmc_kernels_h.cu", "qmc_kernels_fx6.cu",
-           "qmc_kernels_fx3.cu", "qmc_kernels_fd.cu", "qmc_mlp.cu", "qmc_host.cpp", "qmc_integrate.cpp"]
+           "qmc_kernels_fx3.cu", "qmc_kernels_fd.cu", "qmc_kernels_fdm.cu", "qmc_mlp.cu", "qmc_host.cpp", "qmc_integrate.cpp"]
 
 
 def _nvcc() -> str:

@@ -1,8 +1,8 @@
-// The deformed evaluator for sums ending at eps^0: contour-deformed sectors
+// The deformed evaluator for sums ending at eps^0 or eps^1: contour-deformed sectors
 // with d <= 3, at most two singular variables and exponents u0, u1, f0, f1,
 // b_j that are integers of magnitude <= 4; in FP64 also F of total degree <= 2
 // (every one-loop sector of the built-in integrals). Included by
-// qmc_kernels.cu (part 6) after qmc_real.cuh, whose front it shares.
+// qmc_kernels.cu (parts 6, FP64, and 7, mixed precision) after qmc_real.cuh, whose front it shares.
 //
 // What bounds it: the FP64 pipe (76 % busy in the general kernel, at 175
 // useful FP64 instructions per evaluation of the massive box and as many
@@ -61,13 +61,13 @@ __device__ __forceinline__ FdShared &fd_shared() { return *reinterpret_cast<FdSh
 __device__ __noinline__ double fd_half_log_ratio(double a, double b) {
     const qmc_xf x = qmc_xf_of(a), y = qmc_xf_of(b);
     if (x.m == 0 || y.m == 0) return a * (1.0 / b);      // (the integrand is singular there)
-    const FxM q = fx_norm(fx_mul(FxM{x.m, x.e}, FxM{qmc_xf_rcp(y).m, qmc_xf_rcp(y).e}));
+    const FxM q = fx_norm(fx_mul(FxM{x.m, x.e}, FxM{qmc_xf_rcp3(y).m, qmc_xf_rcp3(y).e}));
     return fx_half(qmc_ilog_xf(qmc_xf{q.m, q.e, 0}, fd_shared().logtab));
 }
 __device__ __noinline__ double fd_rcp(double x) {
     const qmc_xf a = qmc_xf_of(x);
     if (a.m == 0) return 1.0 / x;
-    return qmc_xf_to_double(qmc_xf_rcp(a));
+    return qmc_xf_to_double(qmc_xf_rcp3(a));
 }
 __device__ __noinline__ double fd_atan2(double y, double x) { return qatan2(y, x, fd_shared().atantab); }
 
@@ -185,10 +185,10 @@ struct FdCorner {
 };
 
 // The corner with the slots of V at t = 0 (D variables, NS of them singular)
-template <int D, int BLOCK, int NS, int V, bool MIXED>
+template <int D, int BLOCK, int NS, int HI, int V, bool MIXED>
 __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, int prow, int &signfail) {
     const FdShared &S = fd_shared();
-    constexpr bool lam = V != 0;                        // needs its eps exponent (sums end at eps^0)
+    constexpr bool lam = HI > 0 || V != 0;              // needs its eps exponent
     constexpr int NA = D - __builtin_popcount(V);       // variables left
     double g[D];                                        // dF/dt_j
     double Vd[D], Vo[D][D];                             // J = 1 - i V: diagonal, off-diagonal
@@ -439,23 +439,24 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
 }
 
 // Depth-first fold of the corners (see qmc_real.cuh), complex series
-template <int D, int BLOCK, int NS, bool MIXED> struct FdFold {
+template <int D, int BLOCK, int NS, int HI, bool MIXED> struct FdFold {
     const FdPoint &P;
     const FdOps &o;
-    const double (&h)[SlotArr<NS>::N][SlotArr<NS>::N];
+    const double (&h)[SlotArr<NS>::N][NS + HI + 1];
     int prow;
     int &signfail;
 
     template <int Q, int V>
-    __device__ __forceinline__ void run(dc (&out)[Q + __builtin_popcount(V) + 1]) const {
+    __device__ __forceinline__ void run(dc (&out)[Q + __builtin_popcount(V) + HI + 1]) const {
         constexpr int pv = __builtin_popcount(V);
         if constexpr (Q == 0) {
-            const FdCorner c = fd_corner<D, BLOCK, NS, V, MIXED>(P, o, prow, signfail);
+            const FdCorner c = fd_corner<D, BLOCK, NS, HI, V, MIXED>(P, o, prow, signfail);
             out[0] = c.B;
-            if constexpr (pv >= 1) out[1] = o.mul(c.B, c.L);
-            if constexpr (pv >= 2) out[2] = o.mul(out[1], dc{fx_half(c.L.re), fx_half(c.L.im)});
+            if constexpr (pv + HI >= 1) out[1] = o.mul(c.B, c.L);
+            if constexpr (pv + HI >= 2) out[2] = o.mul(out[1], dc{fx_half(c.L.re), fx_half(c.L.im)});
+            if constexpr (pv + HI >= 3) out[3] = o.mul(out[2], dc{c.L.re * (1.0 / 3), c.L.im * (1.0 / 3)});
         } else {
-            constexpr int n = Q + pv;
+            constexpr int n = Q + pv + HI;
             dc a[n], b[n + 1];
             run<Q - 1, V>(a);
             run<Q - 1, V | (1 << (Q - 1))>(b);
@@ -475,7 +476,7 @@ template <int D, int BLOCK, int NS, bool MIXED> struct FdFold {
     }
 };
 
-template <int D, int BLOCK, int NS, bool MIXED, int LMAX>
+template <int D, int BLOCK, int NS, int HI, bool MIXED, int LMAX>
 __device__ __forceinline__ void fd_points(const QmcLaunch &Lc, uint64_t k0, uint64_t kend, int lo, int nord,
                                           dc (&acc)[LMAX], int &signfail) {
     constexpr int NSA = SlotArr<NS>::N;
@@ -494,9 +495,10 @@ __device__ __forceinline__ void fd_points(const QmcLaunch &Lc, uint64_t k0, uint
         }
     }
     const FdOps o{S.mone, S.nzero};
-    dc accN[NS + 1];
+    constexpr int NO = NS + HI + 1;
+    dc accN[NO];
 #pragma unroll
-    for (int i = 0; i <= NS; ++i) accN[i] = dc{0.0, 0.0};
+    for (int i = 0; i < NO; ++i) accN[i] = dc{0.0, 0.0};
 #pragma unroll 1
     for (uint64_t k = k0; k < kend; ++k) {
         FxM w{1ULL << 63, 0};
@@ -541,24 +543,25 @@ __device__ __forceinline__ void fd_points(const QmcLaunch &Lc, uint64_t k0, uint
                 else P.tf[2] = f;
             }
             if (i < NS && u.y.m) {
-                const qmc_xf r = qmc_xf_rcp(qmc_xf{t.m, t.e, 0});
+                const qmc_xf r = qmc_xf_rcp3(qmc_xf{t.m, t.e, 0});
                 hb[i] = S.bd[i] * fx_pack(FxM{r.m, r.e});
-                if (NS > 1) bl[i] = S.bd[i] * qmc_ilog_core(t.e, t.m & 0x7FFFFFFFFFFFFFFFULL, S.logtab);
+                if (NS + HI > 1) bl[i] = S.bd[i] * qmc_ilog_core(t.e, t.m & 0x7FFFFFFFFFFFFFFFULL, S.logtab);
             }
         }
         if (zero) continue;
         double W = 1.0;
         if (Lc.transform == 0) W = fx_pack(fx_norm(fx_mul(fx_mul(w, w), w)));
-        double h[NSA][NSA];
+        double h[NSA][NO];
 #pragma unroll
         for (int q = 0; q < NS; ++q) {
             h[q][0] = hb[q];
-            if (NS > 1) h[q][1 % NSA] = o.mul(hb[q], bl[q]);
+            if constexpr (NS + HI > 1) h[q][1] = o.mul(hb[q], bl[q]);
+            if constexpr (NS + HI > 2) h[q][2] = o.mul(h[q][1], fx_half(bl[q]));
         }
-        dc res[NS + 1];
-        FdFold<D, BLOCK, NS, MIXED>{P, o, h, Lc.prow, signfail}.template run<NS, 0>(res);
+        dc res[NO];
+        FdFold<D, BLOCK, NS, HI, MIXED>{P, o, h, Lc.prow, signfail}.template run<NS, 0>(res);
 #pragma unroll
-        for (int i = 0; i <= NS; ++i) {
+        for (int i = 0; i < NO; ++i) {
             accN[i].re = fma(res[i].re, W, accN[i].re);
             accN[i].im = fma(res[i].im, W, accN[i].im);
         }
@@ -567,7 +570,7 @@ __device__ __forceinline__ void fd_points(const QmcLaunch &Lc, uint64_t k0, uint
     for (int q = 0; q < LMAX; ++q) {
         dc v{0.0, 0.0};
 #pragma unroll
-        for (int i = 0; i <= NS; ++i)
+        for (int i = 0; i < NO; ++i)
             if (i == lo + q + NS) v = accN[i];
         if (q < nord) acc[q] = v;
     }
@@ -681,7 +684,7 @@ __device__ __forceinline__ void fd_stage(FdShared &S, const QmcLaunch &Lc) {
 #ifndef QMC_FD_MINB
 #define QMC_FD_MINB 4
 #endif
-template <bool MIXED, int BLOCK>
+template <bool MIXED, int BLOCK, int HI>
 __global__ void __launch_bounds__(BLOCK, QMC_FD_MINB * 128 / BLOCK) qmc_deformed_kernel(QmcLaunch Lc, int ppt) {
     constexpr int LMAX = 4;
     FdShared &S = fd_shared();
@@ -751,16 +754,16 @@ __global__ void __launch_bounds__(BLOCK, QMC_FD_MINB * 128 / BLOCK) qmc_deformed
             const uint64_t kend = min(kt1, k0 + (uint64_t)ppt);
             const int ns = S.ns;
             if (S.d == 3) {
-                if (ns == 0) fd_points<3, BLOCK, 0, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
-                else if (ns == 1) fd_points<3, BLOCK, 1, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
-                else fd_points<3, BLOCK, 2, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
+                if (ns == 0) fd_points<3, BLOCK, 0, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
+                else if (ns == 1) fd_points<3, BLOCK, 1, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
+                else fd_points<3, BLOCK, 2, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
             } else if (S.d == 2) {
-                if (ns == 0) fd_points<2, BLOCK, 0, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
-                else if (ns == 1) fd_points<2, BLOCK, 1, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
-                else fd_points<2, BLOCK, 2, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
+                if (ns == 0) fd_points<2, BLOCK, 0, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
+                else if (ns == 1) fd_points<2, BLOCK, 1, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
+                else fd_points<2, BLOCK, 2, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
             } else {
-                if (ns == 0) fd_points<1, BLOCK, 0, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
-                else fd_points<1, BLOCK, 1, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
+                if (ns == 0) fd_points<1, BLOCK, 0, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
+                else fd_points<1, BLOCK, 1, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc, signfail);
             }
         }
         // sign-check failures of this tile: per job (if counted) and in total
@@ -802,24 +805,25 @@ template <bool MIXED, int BLOCK> constexpr int fd_dyn_smem(int prow) {
     return (int)sizeof(FdShared) + 16 * 3 * BLOCK + (MIXED ? 12 * 3 * prow * BLOCK : 0);
 }
 
-template <bool MIXED, int BLOCK> bool fd_allow() {
-    static const bool ok = cudaFuncSetAttribute(qmc_deformed_kernel<MIXED, BLOCK>,
+template <bool MIXED, int BLOCK, int HI> bool fd_allow() {
+    static const bool ok = cudaFuncSetAttribute(qmc_deformed_kernel<MIXED, BLOCK, HI>,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 fd_dyn_smem<MIXED, BLOCK>(QMC_EMAX)) == cudaSuccess;
     return ok;
 }
 
-template <bool MIXED, int BLOCK>
-int fd_launch(const QmcLaunch *L, int ppt, int grid, cudaStream_t st) {
-    if (L->prow < 1 || L->prow > QMC_EMAX || !fd_allow<MIXED, BLOCK>()) return -1;
-    qmc_deformed_kernel<MIXED, BLOCK><<<grid, BLOCK, fd_dyn_smem<MIXED, BLOCK>(L->prow), st>>>(*L, ppt);
+template <bool MIXED, int BLOCK, int HI>
+int fd_launch(const QmcLaunch *L, int grid, cudaStream_t st) {
+    if (L->prow < 1 || L->prow > QMC_EMAX || !fd_allow<MIXED, BLOCK, HI>()) return -1;
+    qmc_deformed_kernel<MIXED, BLOCK, HI><<<grid, BLOCK, fd_dyn_smem<MIXED, BLOCK>(L->prow), st>>>(
+        *L, (int)((L->tile_k + BLOCK - 1) / BLOCK));
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-template <bool MIXED, int BLOCK> int fd_occupancy(int prow) {
-    if (!fd_allow<MIXED, BLOCK>()) return 0;
+template <bool MIXED, int BLOCK, int HI> int fd_occupancy(int prow) {
+    if (!fd_allow<MIXED, BLOCK, HI>()) return 0;
     int v = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, qmc_deformed_kernel<MIXED, BLOCK>, BLOCK,
-                                                                        fd_dyn_smem<MIXED, BLOCK>(prow));
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &v, qmc_deformed_kernel<MIXED, BLOCK, HI>, BLOCK, fd_dyn_smem<MIXED, BLOCK>(prow));
     return e == cudaSuccess ? v : 0;
 }

@@ -373,6 +373,9 @@ int upload_tables(qmc_ctx *ctx) {
     return QMC_OK;
 }
 
+// The highest orders that qmc_real.cuh and qmc_deformed.cuh sum to
+bool fx_order_ok(int hi, int cls) { return hi == 0 || (hi == 1 && qmc_class_dmax(cls) <= 3); }
+
 // Whether a job qualifies for the integer evaluator (qmc_real.cuh): a real
 // class, small integer exponents, and U and F with coefficients >= 0 at its
 // kinematic point and a constant term of at least 1/128 of their sum (fixed
@@ -404,7 +407,7 @@ bool fx_job_ok(const qmc_ctx *ctx, const HostSector &S, int cls, int point) {
 }
 
 // Points per thread of a launch by qmc_real.cuh or qmc_deformed.cuh: the
-// estimate (waves of `resident` tiles) x (points + 3), the 3 for a tile's
+// estimate (waves of `resident` tiles) x (points + setup), for a tile's
 // staging and lattice set-up, over the tiles that the lattices' sizes give.
 // Few tiles: small ones, so that every SM works (one shift of a pilot lattice
 // would otherwise keep a few blocks busy for 16 points a thread); many: the
@@ -414,12 +417,17 @@ int fx_points_per_thread(const std::vector<QmcJobDev> &jobs, int block, uint64_t
     for (const QmcJobDev &D : jobs) shifts[D.n] += (uint64_t)D.shifts;
     int best = 1;
     double best_cost = 0.0;
-    for (int ppt = 1; ppt <= 32; ++ppt) {
+    // the d <= 6 blocks are large, and warps that finish a tile early wait for
+    // the others: small tiles (double box, n = 10007: 1.67e9 evaluations/s at
+    // 3 points a thread, 1.64e9 at 4, 1.58e9 at 6)
+    const int most = block > 256 ? 4 : 32;
+    const double setup = block > 256 ? 0.5 : 3.0;
+    for (int ppt = 1; ppt <= most; ++ppt) {
         const uint64_t tile = (uint64_t)block * ppt;
         double tiles = 0.0;
         for (const auto &x : shifts) tiles += (double)((x.first + tile - 1) / tile) * (double)x.second;
         const double waves = tiles <= (double)resident ? 1.0 : tiles / (double)resident + 0.5;
-        const double cost = waves * (ppt + 3.0);
+        const double cost = waves * (ppt + setup);
         if (ppt == 1 || cost < best_cost) {
             best = ppt;
             best_cost = cost;
@@ -698,7 +706,7 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         D.flags = J.flags & QMC_JOB_UNSHIFTED;
         out_off += (uint64_t)J.shifts * norders * 2;
         evals += (double)J.n * J.shifts;
-        const int slot = 2 * cls + (hi == 0 && (fd_job_ok(S, cls) || fx_job_ok(ctx, S, cls, J.point)) ? 1 : 0);
+        const int slot = 2 * cls + (fx_order_ok(hi, cls) && (fd_job_ok(S, cls) || fx_job_ok(ctx, S, cls, J.point)) ? 1 : 0);
         per[slot].push_back(D);
         per_orig[slot].push_back(i);
     }
@@ -774,9 +782,8 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
             prow = std::max(prow, ctx->integrals[J.integral_id].sectors[J.sector].prow);
         }
         if (c.fx) {
-            if (qmc_class_dmax(cls) > 3) c.block = QMC_FX6_BLOCK;
-            else if (ctx->opt.block != 128 && ctx->opt.block != 256 && !ctx->tuned_block[cls]) c.block = 256;
-            occ = std::max(1, qmc_k_occupancy_real(cls, c.block, prow));
+            c.block = qmc_class_dmax(cls) > 3 ? QMC_FX6_BLOCK : QMC_FX3_BLOCK;   // their one block size
+            occ = std::max(1, qmc_k_occupancy_real(cls, hi, prow));
             if (ctx->opt.ppt <= 0 && !ctx->tuned_ppt[cls])
                 c.ppt = fx_points_per_thread(v, c.block, (uint64_t)ctx->sm_count * occ);
         } else {
@@ -876,7 +883,7 @@ int plan_enqueue(qmc_plan *plan, double *out, cudaStream_t st, bool capturing) {
             const int ggrid = fx || !c.fx ? c.grid
                                     : (int)std::min<uint64_t>(c.L.ntiles, (uint64_t)ctx->sm_count *
                                                                 std::max(1, qmc_k_occupancy(c.cls, gblock, c.L.prow)));
-            if (fx ? qmc_k_launch_real(c.cls, &c.L, c.block, c.ppt, c.grid, cs)
+            if (fx ? qmc_k_launch_real(c.cls, &c.L, c.grid, cs)
                    : qmc_k_launch_eval(c.cls, &c.L, gblock, (int)(c.L.tile_k / gblock), ggrid, cs))
                 return fail(ctx, QMC_E_CUDA, "evaluator launch failed: %s", cudaGetErrorString(cudaGetLastError()));
             ++launches;
@@ -1232,7 +1239,7 @@ extern "C" int qmc_eval_jobs_noalloc(qmc_ctx *ctx, const qmc_job *jobs, int njob
     const uint64_t tile_k = (uint64_t)block * ppt;
     const int hi = lo + norders - 1;
     int cls = -1;
-    bool fx = hi == 0;   // every job qualifies for qmc_real.cuh or qmc_deformed.cuh
+    bool fx = true;   // every job qualifies for qmc_real.cuh or qmc_deformed.cuh
     uint64_t tiles = 0, out_off = 0;
     for (int i = 0; i < njobs; ++i) {
         const qmc_job &J = jobs[i];
@@ -1260,7 +1267,7 @@ extern "C" int qmc_eval_jobs_noalloc(qmc_ctx *ctx, const qmc_job *jobs, int njob
             return fail(ctx, QMC_E_INVAL, "qmc_eval_jobs_noalloc: all jobs must use one evaluator class");
         if (qmc_class_big(cls) || norders > qmc_class_lmax(cls) || hi + S.ns + 1 > qmc_class_lmax(cls))
             return fail(ctx, QMC_E_INVAL, "job %d: orders %d..%d not supported by the evaluator", i, lo, hi);
-        fx = fx && (fd_job_ok(S, cls) || fx_job_ok(ctx, S, cls, J.point));
+        fx = fx && fx_order_ok(hi, cls) && (fd_job_ok(S, cls) || fx_job_ok(ctx, S, cls, J.point));
         QmcJobDev &D = recs[i];
         memset(&D, 0, sizeof D);
         D.sector = S.global_index;

@@ -85,9 +85,13 @@ struct QmcLaunch {
     unsigned int *job_fail;      // per-job sign-check failures (class-local job index) or null
 };
 
-// Threads per block of the d <= 6 integer evaluator
+// Threads per block of qmc_real.cuh for d <= 6, and of qmc_real.cuh and
+// qmc_deformed.cuh for d <= 3
 #ifndef QMC_FX6_BLOCK
 #define QMC_FX6_BLOCK 384
+#endif
+#ifndef QMC_FX3_BLOCK
+#define QMC_FX3_BLOCK 256
 #endif
 
 // Fixed scratch of the no-allocation entry point (qmc_eval_jobs_noalloc).
@@ -143,8 +147,8 @@ int qmc_k_fp32_probe(float *out_dev, int iters, int grid, int block, void *strea
 int qmc_k_sm_count(int device);
 int qmc_k_occupancy(int cls, int block, int prow);
 // the evaluators of qmc_real.cuh and qmc_deformed.cuh, for jobs that qualify
-int qmc_k_launch_real(int cls, const QmcLaunch *L, int block, int ppt, int grid, void *stream);
-int qmc_k_occupancy_real(int cls, int block, int prow);
+int qmc_k_launch_real(int cls, const QmcLaunch *L, int grid, void *stream);
+int qmc_k_occupancy_real(int cls, int hi, int prow);
 size_t qmc_k_noalloc_partial_capacity(void);
 int qmc_k_noalloc_setup(int device, void **ptr);
 int qmc_k_noalloc_eval(int device, int cls, int fx, const QmcJobDev *jobs_host, int njobs, const QmcLaunch *tmpl,

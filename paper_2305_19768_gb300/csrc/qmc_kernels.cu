@@ -2844,62 +2844,56 @@ int occupancy_cls(int block, int prow) {
 #if QMC_PART >= 4
 #include "qmc_real.cuh"
 #endif
-#if QMC_PART == 6
+#if QMC_PART >= 6
 #include "qmc_deformed.cuh"
 #endif
 }  // namespace
 
 // Per translation unit: the launcher and occupancy query of the classes it
 // instantiates (-2 / 0 for the others). The evaluator classes are compiled in
-// seven translation units in parallel: part 0 the real d <= 3 classes (and
+// eight translation units in parallel: part 0 the real d <= 3 classes (and
 // everything that is not an evaluator), part 1 the deformed classes, part 2
 // the d <= 6 classes, part 3 the Taylor-subtraction classes, parts 4 and 5
-// the integer evaluator (qmc_real.cuh) for d <= 3 and d <= 6, part 6 the
-// deformed evaluator of qmc_deformed.cuh.
+// the integer evaluator (qmc_real.cuh) for d <= 3 and d <= 6, parts 6 and
+// 7 the deformed evaluator of qmc_deformed.cuh, FP64 and mixed.
 #define QMC_PART_FN2(name, part) name##_part##part
 #define QMC_PART_FN(name, part) QMC_PART_FN2(name, part)
 
 #if QMC_PART >= 4
-extern "C" int QMC_PART_FN(qmc_k_launch_real, QMC_PART)(int cls, const QmcLaunch *L, int block, int ppt, int grid,
-                                                         void *stream) {
-    cudaStream_t st = (cudaStream_t)stream;
-    switch (cls) {
-#if QMC_PART == 4
-        case QMC_CLASS_REAL3:
-            return block == 256 ? fx_launch<3, 2, 4, false, 256>(L, ppt, grid, st)
-                                : fx_launch<3, 2, 4, false, 128>(L, ppt, grid, st);
-        case QMC_CLASS_REAL3M:
-            return block == 256 ? fx_launch<3, 2, 4, true, 256>(L, ppt, grid, st)
-                                : fx_launch<3, 2, 4, true, 128>(L, ppt, grid, st);
+// hi: the highest order of the sums (0, or 1 for d <= 3)
+#if QMC_PART == 5
+#define QMC_FX_CLASS(cls, fn, ...) (cls) == QMC_CLASS_REAL6 ? fn<6, 4, 6, false, QMC_FX6_BLOCK, 0>(__VA_ARGS__) : \
+                                   (cls) == QMC_CLASS_REAL6M ? fn<6, 4, 6, true, QMC_FX6_BLOCK, 0>(__VA_ARGS__) :
+#elif QMC_PART == 4
+#define QMC_FX_CLASS(cls, fn, ...) (cls) == QMC_CLASS_REAL3 ? (hi ? fn<3, 2, 4, false, QMC_FX3_BLOCK, 1>(__VA_ARGS__) \
+                                                             : fn<3, 2, 4, false, QMC_FX3_BLOCK, 0>(__VA_ARGS__)) : \
+                                   (cls) == QMC_CLASS_REAL3M ? (hi ? fn<3, 2, 4, true, QMC_FX3_BLOCK, 1>(__VA_ARGS__) \
+                                                              : fn<3, 2, 4, true, QMC_FX3_BLOCK, 0>(__VA_ARGS__)) :
 #elif QMC_PART == 6
-        case QMC_CLASS_CPLX3:
-            return block == 256 ? fd_launch<false, 256>(L, ppt, grid, st) : fd_launch<false, 128>(L, ppt, grid, st);
-        case QMC_CLASS_CPLX3M:
-            return block == 256 ? fd_launch<true, 256>(L, ppt, grid, st) : fd_launch<true, 128>(L, ppt, grid, st);
+#define QMC_FD_CLASS(cls, fn, ...) (cls) == QMC_CLASS_CPLX3 ? (hi ? fn<false, QMC_FX3_BLOCK, 1>(__VA_ARGS__) \
+                                                             : fn<false, QMC_FX3_BLOCK, 0>(__VA_ARGS__)) :
 #else
-        case QMC_CLASS_REAL6: return fx_launch<6, 4, 6, false, QMC_FX6_BLOCK>(L, ppt, grid, st);
-        case QMC_CLASS_REAL6M: return fx_launch<6, 4, 6, true, QMC_FX6_BLOCK>(L, ppt, grid, st);
+#define QMC_FD_CLASS(cls, fn, ...) (cls) == QMC_CLASS_CPLX3M ? (hi ? fn<true, QMC_FX3_BLOCK, 1>(__VA_ARGS__) \
+                                                              : fn<true, QMC_FX3_BLOCK, 0>(__VA_ARGS__)) :
 #endif
-        default: return -2;
-    }
+extern "C" int QMC_PART_FN(qmc_k_launch_real, QMC_PART)(int cls, const QmcLaunch *L, int grid, void *stream) {
+    cudaStream_t st = (cudaStream_t)stream;
+    const int hi = L->lo + L->norders - 1;
+    (void)hi;
+#if QMC_PART <= 5
+    return QMC_FX_CLASS(cls, fx_launch, L, grid, st) - 2;
+#else
+    return QMC_FD_CLASS(cls, fd_launch, L, grid, st) - 2;
+#endif
 }
 
-extern "C" int QMC_PART_FN(qmc_k_occupancy_real, QMC_PART)(int cls, int block, int prow) {
-    switch (cls) {
-#if QMC_PART == 4
-        case QMC_CLASS_REAL3:
-            return block == 256 ? fx_occupancy<3, 2, 4, false, 256>(prow) : fx_occupancy<3, 2, 4, false, 128>(prow);
-        case QMC_CLASS_REAL3M:
-            return block == 256 ? fx_occupancy<3, 2, 4, true, 256>(prow) : fx_occupancy<3, 2, 4, true, 128>(prow);
-#elif QMC_PART == 6
-        case QMC_CLASS_CPLX3: return block == 256 ? fd_occupancy<false, 256>(prow) : fd_occupancy<false, 128>(prow);
-        case QMC_CLASS_CPLX3M: return block == 256 ? fd_occupancy<true, 256>(prow) : fd_occupancy<true, 128>(prow);
+extern "C" int QMC_PART_FN(qmc_k_occupancy_real, QMC_PART)(int cls, int hi, int prow) {
+    (void)hi;
+#if QMC_PART <= 5
+    return QMC_FX_CLASS(cls, fx_occupancy, prow) 0;
 #else
-        case QMC_CLASS_REAL6: return fx_occupancy<6, 4, 6, false, QMC_FX6_BLOCK>(prow);
-        case QMC_CLASS_REAL6M: return fx_occupancy<6, 4, 6, true, QMC_FX6_BLOCK>(prow);
+    return QMC_FD_CLASS(cls, fd_occupancy, prow) 0;
 #endif
-        default: return 0;
-    }
 }
 #else
 extern "C" int QMC_PART_FN(qmc_k_launch_eval, QMC_PART)(int cls, const QmcLaunch *L, int block, int ppt, int grid,
@@ -2963,24 +2957,26 @@ extern "C" int qmc_k_occupancy_part1(int, int, int);
 extern "C" int qmc_k_occupancy_part2(int, int, int);
 extern "C" int qmc_k_occupancy_part3(int, int, int);
 
-extern "C" int qmc_k_launch_real_part4(int, const QmcLaunch *, int, int, int, void *);
-extern "C" int qmc_k_launch_real_part5(int, const QmcLaunch *, int, int, int, void *);
-extern "C" int qmc_k_launch_real_part6(int, const QmcLaunch *, int, int, int, void *);
-extern "C" int qmc_k_occupancy_real_part4(int, int, int);
-extern "C" int qmc_k_occupancy_real_part5(int, int, int);
-extern "C" int qmc_k_occupancy_real_part6(int, int, int);
+#define QMC_REAL_PART(part)                                                      \
+    extern "C" int qmc_k_launch_real_part##part(int, const QmcLaunch *, int, void *); \
+    extern "C" int qmc_k_occupancy_real_part##part(int, int, int);
+QMC_REAL_PART(4)
+QMC_REAL_PART(5)
+QMC_REAL_PART(6)
+QMC_REAL_PART(7)
 
-extern "C" int qmc_k_launch_real(int cls, const QmcLaunch *L, int block, int ppt, int grid, void *stream) {
-    for (auto f : {qmc_k_launch_real_part4, qmc_k_launch_real_part5, qmc_k_launch_real_part6}) {
-        const int rc = f(cls, L, block, ppt, grid, stream);
+extern "C" int qmc_k_launch_real(int cls, const QmcLaunch *L, int grid, void *stream) {
+    for (auto f : {qmc_k_launch_real_part4, qmc_k_launch_real_part5, qmc_k_launch_real_part6, qmc_k_launch_real_part7}) {
+        const int rc = f(cls, L, grid, stream);
         if (rc != -2) return rc;
     }
     return -2;
 }
 
-extern "C" int qmc_k_occupancy_real(int cls, int block, int prow) {
-    for (auto f : {qmc_k_occupancy_real_part4, qmc_k_occupancy_real_part5, qmc_k_occupancy_real_part6}) {
-        const int v = f(cls, block, prow);
+extern "C" int qmc_k_occupancy_real(int cls, int hi, int prow) {
+    for (auto f : {qmc_k_occupancy_real_part4, qmc_k_occupancy_real_part5, qmc_k_occupancy_real_part6,
+                   qmc_k_occupancy_real_part7}) {
+        const int v = f(cls, hi, prow);
         if (v) return v;
     }
     return 0;
@@ -3125,12 +3121,12 @@ extern "C" int qmc_k_noalloc_eval(int device, int cls, int fx, const QmcJobDev *
     if (cudaMemcpyAsync(b + kNoallocJobOff, jobs_host, (size_t)njobs * sizeof(QmcJobDev),
                         cudaMemcpyHostToDevice, st) != cudaSuccess)
         return -1;
-    int occ = fx ? qmc_k_occupancy_real(cls, block, L.prow) : qmc_k_occupancy(cls, block, L.prow);
+    int occ = fx ? qmc_k_occupancy_real(cls, L.lo + L.norders - 1, L.prow) : qmc_k_occupancy(cls, block, L.prow);
     if (occ < 1) occ = 1;
     uint64_t g = (uint64_t)sm_count * occ;
     if (L.ntiles < g) g = L.ntiles;
     const int grid = g < 1 ? 1 : (int)g;
-    if (L.ntiles > 0 && (fx ? qmc_k_launch_real(cls, &L, block, ppt, grid, stream)
+    if (L.ntiles > 0 && (fx ? qmc_k_launch_real(cls, &L, grid, stream)
                             : qmc_k_launch_eval(cls, &L, block, ppt, grid, stream)))
         return -1;
     if (qmc_k_launch_finish(&L, stream)) return -1;

@@ -1,5 +1,5 @@
-// The real evaluator on integers: undeformed sectors whose sums end at eps^0,
-// whose exponents u0, u1, f0, f1 are integers of magnitude <= 4 and whose U
+// The real evaluator on integers: undeformed sectors whose sums end at eps^0
+// (d <= 3: or eps^1), whose exponents u0, u1, f0, f1 are integers of magnitude <= 4 and whose U
 // and F have non-negative coefficients at the job's kinematic point with a
 // constant term c0 >= (sum of coefficients) / 128 (the host checks this per
 // job; see fx_job_ok in qmc_host.cpp). Every Euclidean sector of the built-in
@@ -18,10 +18,14 @@
 //    coefficients, below 2^-53 of any corner value (all are >= c0);
 //  * a corner's powers and logarithm follow from those integers directly.
 // FP64 is left with each corner's series (B L^i / i!), their combination and
-// the accumulation. Sectors with four singular variables keep the monomials
-// in FP64 and their corner values rounded to 53 bits: their eps^0 sums cancel
-// by up to 1e8, so the rounding of each U and F shows in the result at 1e-9,
-// and results stay comparable with the general kernel's there.
+// the accumulation. Sectors with three or four singular variables (EX below)
+// take the general kernel's roundings up to the corner values instead: t to
+// FP64, monomials and group sums in FP64, subset sums and corner products in
+// 64-bit mantissas in the same order, and the Moebius transform before the
+// fold. Their eps^0 sums cancel by up to 1e8, so that the last bit of one
+// corner of one point near the border shows in a shift's sum at 1e-7: with
+// other roundings, each as good, results would not be comparable between the
+// kernels (with these they agree to 1e-15).
 //
 // The combination folds one singular variable at a time instead of forming
 // the Moebius transform of all corners and then every pole set:
@@ -57,8 +61,8 @@ struct alignas(16) FxShared {
     uint64_t logtab[3 * QMC_LOG_TABLE_ROWS + 1];
     // a monomial's factors as offsets of the power-table rows (4-byte units, 16
     // bits each, in x, y, z) and their count (w); its coefficient times 2^sh
-    // (mixed precision: its FP32 value in the low word; four singular
-    // variables: the FP64 value)
+    // (mixed precision: its FP32 value in the low word; three or four
+    // singular variables: the FP64 value)
     uint4 mdesc[QMC_MAXMONO];
     uint64_t cfix[QMC_MAXMONO];
     int32_t gs[2][QMC_NGROUP + 1];   // first monomial of each singular-mask group of U, F
@@ -187,6 +191,25 @@ __device__ __forceinline__ FxM fx_korobov(const FxCoord &u) {
     const int c = __clzll((long long)hi);               // hi >= 2^56
     return FxM{(hi << c) | ((lo >> 1) >> (63 - c)), 10 - c + 4 * u.y.e};
 }
+// korobov3 of u in the general kernel's roundings (korobov_phi_fix: P by
+// Horner on the smaller of u and 1 - u), the bits below the mantissa or-ed
+// into its last one, so that it rounds to the same FP64 value
+__device__ __forceinline__ FxM fx_korobov_ex(const FxCoord &u) {
+    const uint64_t sm = u.lower ? ~0ULL : 0ULL;
+    const uint64_t y = u.lower ? u.Y >> 2 : u.Y;
+    const uint32_t ylo = (uint32_t)y;
+    const uint64_t y20 = (y >> 1) + (y >> 3) + ((((ylo & 1u) << 2) + (ylo & 7u)) >> 3);   // 20 Y in Q57 / Q59
+    const uint64_t a1 = (u.lower ? 70ULL << 57 : 10ULL << 59) + ((y20 ^ sm) - sm);
+    const uint64_t a2 = (u.lower ? 84ULL << 57 : 4ULL << 59) + ((__umul64hi(u.Y, a1) ^ sm) - sm);
+    const uint64_t P = (u.lower ? 35ULL << 57 : 1ULL << 59) + ((__umul64hi(u.Y, a2) ^ sm) - sm);
+    const uint64_t M = u.lower ? u.y.m : u.big;
+    const int e = u.lower ? u.y.e : -1;
+    const uint64_t p2 = __umul64hi(M, M);
+    const uint64_t p4 = __umul64hi(p2, p2);
+    const uint64_t hi = __umul64hi(p4, P), lo = p4 * P;
+    const int c = __clzll((long long)hi);
+    return FxM{(hi << c) | ((lo >> 1) >> (63 - c)) | ((lo << c) ? 1ULL : 0ULL), 67 - c + 4 * e - (u.lower ? 57 : 59)};
+}
 // 1 - s for 0 < s <= 1/2 (2^-64 below 1 where s < 2^-64)
 __device__ __forceinline__ FxM fx_one_minus(FxM s) {
     const uint64_t S = s.e >= -64 ? s.m >> (-1 - s.e) : 0;
@@ -209,8 +232,8 @@ __device__ __forceinline__ double fx_half(double x) {
 // One group's sum of monomials [m0, m1): out of line, one copy for every
 // group of both polynomials. FP32 products in the order of the table for the
 // mixed precision.
-// P64: FP64 products and sums.
-template <int DMAX, int BLOCK, bool MIXED, bool P64>
+// EX: the sum in FP64, in the general kernel's order (its bits).
+template <int DMAX, int BLOCK, bool MIXED, bool EX>
 __device__ __noinline__ uint64_t fx_group(int m0, int m1, int sh) {
     const FxShared &S = fx_shared();
     if constexpr (MIXED) {
@@ -238,12 +261,13 @@ __device__ __noinline__ uint64_t fx_group(int m0, int m1, int sh) {
             }
             s = m == m0 ? __fmul_rn(v, c) : __fmaf_rn(v, c, s);
         }
+        if constexpr (EX) return (uint64_t)__double_as_longlong((double)s);
         // s 2^sh (s >= 0), rounded
         const uint32_t b = __float_as_uint(s);
         const uint64_t mant = (b & 0x7FFFFFu) | (b >= 0x800000u ? 0x800000u : 0u);
         const int x = (int)(b >> 23) - 150 + sh;
         return x >= 0 ? mant << x : (x > -26 ? (mant + (1ULL << (-x - 1))) >> -x : 0);
-    } else if constexpr (P64) {
+    } else if constexpr (EX) {
         const unsigned char *pt = fx_pt<DMAX, BLOCK>(8);
         auto ld = [&](uint32_t off) { return *reinterpret_cast<const double *>(pt + 4 * off); };
         double s = 0.0;
@@ -268,11 +292,7 @@ __device__ __noinline__ uint64_t fx_group(int m0, int m1, int sh) {
             }
             s = fma(v, c, m == m0 ? S.nzero : s);
         }
-        // s 2^sh (s >= 0), rounded
-        const uint64_t b = (uint64_t)__double_as_longlong(s);
-        const uint64_t mant = (b & 0x000FFFFFFFFFFFFFULL) | (b >> 52 ? 1ULL << 52 : 0);
-        const int x = (int)(b >> 52) - 1075 + sh;
-        return x >= 0 ? mant << x : (x > -55 ? (mant + (1ULL << (-x - 1))) >> -x : 0);
+        return (uint64_t)__double_as_longlong(s);
     } else {
         const unsigned char *pt = fx_pt<DMAX, BLOCK>(8);
         auto ld = [&](uint32_t off) { return *reinterpret_cast<const uint64_t *>(pt + 4 * off); };
@@ -320,27 +340,18 @@ __device__ __forceinline__ FxM fx_pow(FxM x, FxM r, int k) {
     }
     return p;
 }
-// x to 53 bits (nearest even)
-__device__ __forceinline__ FxM fx_round53(FxM a) {
-    const uint64_t m = (a.m + 0x3FFULL + ((a.m >> 11) & 1ULL)) & ~0x7FFULL;
-    return m ? FxM{m, a.e} : FxM{1ULL << 63, a.e + 1};
-}
-__device__ __noinline__ FxCorner fx_corner(uint64_t U, uint64_t F, FxM Cc, double Lc, bool lam, bool round53) {
+__device__ __noinline__ FxCorner fx_corner(uint64_t U, uint64_t F, FxM Cc, double Lc, bool lam) {
     const FxShared &S = fx_shared();
     const uint32_t ex = S.ex;
     const int u0 = (int8_t)ex, f0 = (int8_t)(ex >> 8), u1 = (int8_t)(ex >> 16), f1 = (int8_t)(ex >> 24);
-    FxM u = fx_norm(FxM{U, 63 - S.sh[0]}), f = fx_norm(FxM{F, 63 - S.sh[1]});
-    if (round53) {
-        u = fx_round53(u);
-        f = fx_round53(f);
-    }
+    const FxM u = fx_norm(FxM{U, 63 - S.sh[0]}), f = fx_norm(FxM{F, 63 - S.sh[1]});
     FxM ru = u, rf = f;
     if (u0 < 0 || (lam && u1 < 0)) {
-        const qmc_xf r = qmc_xf_rcp(qmc_xf{u.m, u.e, 0});
+        const qmc_xf r = qmc_xf_rcp3(qmc_xf{u.m, u.e, 0});
         ru = FxM{r.m, r.e};
     }
     if (f0 < 0 || (lam && f1 < 0)) {
-        const qmc_xf r = qmc_xf_rcp(qmc_xf{f.m, f.e, 0});
+        const qmc_xf r = qmc_xf_rcp3(qmc_xf{f.m, f.e, 0});
         rf = FxM{r.m, r.e};
     }
     FxCorner out{1.0, 0.0};
@@ -361,26 +372,107 @@ __device__ __noinline__ FxCorner fx_corner(uint64_t U, uint64_t F, FxM Cc, doubl
     return out;
 }
 
+// The same for the EX sectors: FP64 values of U and F (positive), and the
+// products of qmc_xf_mul in the order of corner_xf
+__device__ __forceinline__ FxM fx_mulx(FxM a, FxM b) {
+    const uint64_t h = __umul64hi(a.m, b.m);
+    const int top = (int)(h >> 63);
+    return FxM{top ? h : h << 1, a.e + b.e + top};
+}
+// x^k0 and x^k1 by repeated products of x or 1/x
+__device__ __forceinline__ void fx_powx(FxM x, FxM r, int k0, int k1, FxM &p0, FxM &p1) {
+    p0 = p1 = FxM{1ULL << 63, 0};
+    const int n = max(max(k0, k1), 0), m = max(max(-k0, -k1), 0);
+    FxM p = x;
+    for (int i = 1; i <= n; ++i) {
+        if (i > 1) p = fx_mulx(p, x);
+        if (i == k0) p0 = p;
+        if (i == k1) p1 = p;
+    }
+    p = r;
+    for (int i = 1; i <= m; ++i) {
+        if (i > 1) p = fx_mulx(p, r);
+        if (i == -k0) p0 = p;
+        if (i == -k1) p1 = p;
+    }
+}
+__device__ __forceinline__ FxM fx_of(double x) {
+    const qmc_xf a = qmc_xf_of(x);
+    return FxM{a.m, a.e};
+}
+__device__ __noinline__ FxCorner fx_corner_ex(double U, double F, double Cc, double Lc, bool lam) {
+    const FxShared &S = fx_shared();
+    const uint32_t ex = S.ex;
+    const int u0 = (int8_t)ex, f0 = (int8_t)(ex >> 8), u1 = (int8_t)(ex >> 16), f1 = (int8_t)(ex >> 24);
+    const FxM u = fx_of(U), f = fx_of(F);
+    FxM ru = u, rf = f;
+    if (u0 < 0 || (lam && u1 < 0)) {
+        const qmc_xf r = qmc_xf_rcp(qmc_xf{u.m, u.e, 0});
+        ru = FxM{r.m, r.e};
+    }
+    if (f0 < 0 || (lam && f1 < 0)) {
+        const qmc_xf r = qmc_xf_rcp(qmc_xf{f.m, f.e, 0});
+        rf = FxM{r.m, r.e};
+    }
+    FxM pu0, pu1, pf0, pf1;
+    fx_powx(u, ru, u0, lam ? u1 : 0, pu0, pu1);
+    fx_powx(f, rf, f0, lam ? f1 : 0, pf0, pf1);
+    const FxM b = fx_mulx(S.hasC ? fx_of(Cc) : FxM{1ULL << 63, 0}, fx_mulx(pu0, pf0));
+    FxCorner out{qmc_xf_to_double(qmc_xf{b.m, b.e, 0}), 0.0};
+    if (lam) {
+        const FxM x = fx_mulx(pu1, pf1);
+        out.L = qmc_ilog_xf(qmc_xf{x.m, x.e, 0}, S.logtab);
+        if (S.hasL) out.L += Lc;
+    }
+    return out;
+}
+// Their subset sums over the singular variables, of non-negative FP64 values
+// (subset_sums_xf without signs), rounded to FP64 in place
+template <int NS> __device__ __noinline__ void fx_subset_ex(double *h) {
+    constexpr int NG = 1 << NS;
+    FxM x[NG];
+#pragma unroll
+    for (int g = 0; g < NG; ++g) x[g] = fx_of(h[g]);
+#pragma unroll
+    for (int q = 0; q < NS; ++q)
+#pragma unroll
+        for (int g = 0; g < NG; ++g)
+            if (g & (1 << q)) {
+                const FxM a = x[g], b = x[g ^ (1 << q)];
+                const bool sw = b.e > a.e;
+                const uint64_t big = sw ? b.m : a.m, small = sw ? a.m : b.m;
+                const int e = sw ? b.e : a.e, d = sw ? b.e - a.e : a.e - b.e;
+                const uint64_t s = big + (d < 64 ? small >> d : 0ULL);
+                const bool c = s < big;
+                x[g] = FxM{c ? (s >> 1) | (1ULL << 63) : s, e + (c ? 1 : 0)};
+            }
+#pragma unroll
+    for (int g = 0; g < NG; ++g) h[g] = qmc_xf_to_double(qmc_xf{x[g].m, x[g].e, 0});
+}
+
 // Depth-first fold over the singular variables (see the top): out receives
-// the orders eps^-Q .. eps^|V|, V the corner bits at and above Q.
-template <int NS> struct FxFold {
+// the orders eps^-Q .. eps^(|V| + HI), V the corner bits at and above Q and
+// eps^HI the last order of the sums.
+template <int NS, int HI> struct FxFold {
     const double (&B)[1 << NS];   // corner values and exponents
     const double (&L)[1 << NS];
-    const double (&h)[SlotArr<NS>::N][SlotArr<NS>::N];   // (b/t) (b ln t)^j / j! per slot
+    const double (&h)[SlotArr<NS>::N][NS + HI + 1];   // (b/t) (b ln t)^j / j! per slot
     double mone, nzero;
 
     template <int Q, int V>
-    __device__ __forceinline__ void run(double (&out)[Q + __builtin_popcount(V) + 1]) const {
+    __device__ __forceinline__ void run(double (&out)[Q + __builtin_popcount(V) + HI + 1]) const {
         constexpr int pv = __builtin_popcount(V);
         if constexpr (Q == 0) {
-            const double l = L[V];
+            // B L^i / i!
+            constexpr int N = pv + HI;
+            const double l = N > 0 ? L[V] : 0.0;
             out[0] = B[V];
-            if constexpr (pv >= 1) out[1] = fma(out[0], l, nzero);
-            if constexpr (pv >= 2) out[2] = fma(out[1], fx_half(l), nzero);
-            if constexpr (pv >= 3) out[3] = fma(out[2], l * (1.0 / 3), nzero);
-            if constexpr (pv >= 4) out[4] = fma(out[3], fx_half(fx_half(l)), nzero);
+            if constexpr (N >= 1) out[1] = fma(out[0], l, nzero);
+            if constexpr (N >= 2) out[2] = fma(out[1], fx_half(l), nzero);
+            if constexpr (N >= 3) out[3] = fma(out[2], l * (1.0 / 3), nzero);
+            if constexpr (N >= 4) out[4] = fma(out[3], fx_half(fx_half(l)), nzero);
         } else {
-            constexpr int n = Q + pv;
+            constexpr int n = Q + pv + HI;
             double a[n], b[n + 1];
             run<Q - 1, V>(a);
             run<Q - 1, V | (1 << (Q - 1))>(b);
@@ -397,14 +489,44 @@ template <int NS> struct FxFold {
     }
 };
 
+// EX: the fold over the Moebius-transformed corner series D (series_fp64 and
+// moebius_fp64 of the general kernel):
+//   S(Q, P) = (b/t) e^{eps b ln t} S(Q-1, P) + S(Q-1, P + q) / eps
+template <int NS, int HI> struct FxFoldD {
+    const double (&D)[1 << NS][NS + HI + 1];
+    const double (&h)[SlotArr<NS>::N][NS + HI + 1];
+
+    template <int Q, int P>
+    __device__ __forceinline__ void run(double (&out)[Q + __builtin_popcount(P) + HI + 1]) const {
+        constexpr int n = Q + __builtin_popcount(P) + HI;
+        if constexpr (Q == 0) {
+#pragma unroll
+            for (int i = 0; i <= n; ++i) out[i] = D[P][i];
+        } else {
+            double a[n], b[n + 1];
+            run<Q - 1, P>(a);
+            run<Q - 1, P | (1 << (Q - 1))>(b);
+            out[0] = b[0];
+#pragma unroll
+            for (int k = 0; k < n; ++k) {
+                double s = b[k + 1];
+#pragma unroll
+                for (int i = 0; i <= k; ++i) s = fma(h[Q - 1][k - i], a[i], s);
+                out[k + 1] = s;
+            }
+        }
+    }
+};
+
 // The thread's points [k0, kend) of the tile: acc[o] is the sum of W f_o,
 // order eps^(lo + o).
-template <int DMAX, int BLOCK, int NS, bool MIXED, int LMAX>
+template <int DMAX, int BLOCK, int NS, int HI, bool MIXED, int LMAX>
 __device__ __forceinline__ void fx_points(const QmcLaunch &Lc, uint64_t k0, uint64_t kend, int lo, int nord,
                                           double (&acc)[LMAX]) {
     constexpr int NSA = SlotArr<NS>::N;
     constexpr int NG = 1 << NS;
-    constexpr bool P64 = !MIXED && NS == 4;   // FP64 monomials (see the top)
+    constexpr bool EX = NS >= 3;              // the general kernel's roundings (see the top)
+    constexpr bool P64 = !MIXED && EX;        // FP64 monomials
     const FxShared &S = fx_shared();
     const int d = S.d;
     const uint64_t n = S.job.n;
@@ -421,9 +543,10 @@ __device__ __forceinline__ void fx_points(const QmcLaunch &Lc, uint64_t k0, uint
             walk[i * BLOCK] = make_uint4((uint32_t)Q, (uint32_t)(Q >> 32), (uint32_t)r0, (uint32_t)R);
         }
     }
-    double accN[NS + 1];
+    constexpr int NO = NS + HI + 1;
+    double accN[NO];
 #pragma unroll
-    for (int i = 0; i <= NS; ++i) accN[i] = 0.0;
+    for (int i = 0; i < NO; ++i) accN[i] = 0.0;
 #pragma unroll 1
     for (uint64_t k = k0; k < kend; ++k) {
         FxM w{1ULL << 63, 0}, Cc{1ULL << 63, 0};
@@ -441,8 +564,12 @@ __device__ __forceinline__ void fx_points(const QmcLaunch &Lc, uint64_t k0, uint
             }
             FxM t;
             if (Lc.transform == 0) {
-                const FxM s = fx_korobov(u);
-                t = u.lower ? s : fx_one_minus(s);
+                if constexpr (EX) {
+                    t = fx_korobov_ex(u);
+                } else {
+                    const FxM s = fx_korobov(u);
+                    t = u.lower ? s : fx_one_minus(s);
+                }
                 // the weight: prod u (1 - u), cubed below
                 w = fx_norm(fx_mul(w, FxM{__umul64hi(u.y.m, u.big), u.y.e}));
             } else if (Lc.transform == 1) {             // baker: 1 - |2u - 1|
@@ -491,9 +618,9 @@ __device__ __forceinline__ void fx_points(const QmcLaunch &Lc, uint64_t k0, uint
             const bool reg = (S.regular >> i) & 1;
             if (i < NS || reg) {
                 double l = 0.0;
-                if (NS > 1 || (NS > 0 && reg)) l = qmc_ilog_core(t.e, t.m & 0x7FFFFFFFFFFFFFFFULL, S.logtab);
+                if (NS + HI > 1 || (NS + HI > 0 && reg)) l = qmc_ilog_core(t.e, t.m & 0x7FFFFFFFFFFFFFFFULL, S.logtab);
                 if (i < NS) {
-                    const qmc_xf r = qmc_xf_rcp(qmc_xf{t.m, t.e, 0});
+                    const qmc_xf r = qmc_xf_rcp3(qmc_xf{t.m, t.e, 0});
                     hb[i] = S.bvar[i] * fx_pack(FxM{r.m, r.e});
                     bl[i] = S.bvar[i] * l;
                 } else {
@@ -508,50 +635,78 @@ __device__ __forceinline__ void fx_points(const QmcLaunch &Lc, uint64_t k0, uint
         if (Lc.transform == 0) W = fx_pack(fx_norm(fx_mul(fx_mul(w, w), w)));
         // the polynomials: group sums, then subset sums over the singular
         // variables; the value at corner V (t_V = 0) is h[(NG-1) ^ V]
-        uint64_t hU[NG], hF[NG];
-#pragma unroll
-        for (int g = 0; g < NG; ++g) {
-            const int u0 = S.gs[0][g], u1 = S.gs[0][g + 1], f0 = S.gs[1][g], f1 = S.gs[1][g + 1];
-            hU[g] = 0;
-            hF[g] = 0;
-            if (u1 > u0) hU[g] = fx_group<DMAX, BLOCK, MIXED, P64>(u0, u1, S.sh[0]);
-            if (f1 > f0) hF[g] = fx_group<DMAX, BLOCK, MIXED, P64>(f0, f1, S.sh[1]);
-        }
-#pragma unroll
-        for (int q = 0; q < NS; ++q)
-#pragma unroll
-            for (int g = 0; g < NG; ++g)
-                if (g & (1 << q)) {
-                    hU[g] += hU[g ^ (1 << q)];
-                    hF[g] += hF[g ^ (1 << q)];
-                }
         double B[NG], L[NG];
+        if constexpr (EX) {
+            double hU[NG], hF[NG];
 #pragma unroll 1
-        for (int V = 0; V < NG; ++V) {
-            const FxCorner c = fx_corner(hU[(NG - 1) ^ V], hF[(NG - 1) ^ V], Cc, Lr, V != 0, NS == 4);
-            B[V] = c.B;
-            L[V] = c.L;
+            for (int g = 0; g < NG; ++g) {
+                const int u0 = S.gs[0][g], u1 = S.gs[0][g + 1], f0 = S.gs[1][g], f1 = S.gs[1][g + 1];
+                hU[g] = 0.0;
+                hF[g] = 0.0;
+                if (u1 > u0) hU[g] = __longlong_as_double((long long)fx_group<DMAX, BLOCK, MIXED, EX>(u0, u1, 0));
+                if (f1 > f0) hF[g] = __longlong_as_double((long long)fx_group<DMAX, BLOCK, MIXED, EX>(f0, f1, 0));
+            }
+            fx_subset_ex<NS>(hU);
+            fx_subset_ex<NS>(hF);
+            const double Cd = S.hasC ? fx_pack(Cc) : 1.0;
+#pragma unroll 1
+            for (int V = 0; V < NG; ++V) {
+                const FxCorner c = fx_corner_ex(hU[(NG - 1) ^ V], hF[(NG - 1) ^ V], Cd, Lr, HI > 0 || V != 0);
+                B[V] = c.B;
+                L[V] = c.L;
+            }
+        } else {
+            uint64_t hU[NG], hF[NG];
+#pragma unroll
+            for (int g = 0; g < NG; ++g) {
+                const int u0 = S.gs[0][g], u1 = S.gs[0][g + 1], f0 = S.gs[1][g], f1 = S.gs[1][g + 1];
+                hU[g] = 0;
+                hF[g] = 0;
+                if (u1 > u0) hU[g] = fx_group<DMAX, BLOCK, MIXED, EX>(u0, u1, S.sh[0]);
+                if (f1 > f0) hF[g] = fx_group<DMAX, BLOCK, MIXED, EX>(f0, f1, S.sh[1]);
+            }
+#pragma unroll
+            for (int q = 0; q < NS; ++q)
+#pragma unroll
+                for (int g = 0; g < NG; ++g)
+                    if (g & (1 << q)) {
+                        hU[g] += hU[g ^ (1 << q)];
+                        hF[g] += hF[g ^ (1 << q)];
+                    }
+#pragma unroll 1
+            for (int V = 0; V < NG; ++V) {
+                const FxCorner c = fx_corner(hU[(NG - 1) ^ V], hF[(NG - 1) ^ V], Cc, Lr, HI > 0 || V != 0);
+                B[V] = c.B;
+                L[V] = c.L;
+            }
         }
-        double h[NSA][NSA];
+        double h[NSA][NO];
         const double mone = S.mone, nzero = S.nzero;
 #pragma unroll
         for (int q = 0; q < NS; ++q) {
             h[q][0] = hb[q];
-            if (NS > 1) h[q][1 % NSA] = fma(hb[q], bl[q], nzero);
-            if (NS > 2) h[q][2 % NSA] = fma(h[q][1 % NSA], fx_half(bl[q]), nzero);
-            if (NS > 3) h[q][3 % NSA] = fma(h[q][2 % NSA], bl[q] * (1.0 / 3), nzero);
+            if constexpr (NS + HI > 1) h[q][1] = fma(hb[q], bl[q], nzero);
+            if constexpr (NS + HI > 2) h[q][2] = fma(h[q][1], fx_half(bl[q]), nzero);
+            if constexpr (NS + HI > 3) h[q][3] = fma(h[q][2], bl[q] * (1.0 / 3), nzero);
         }
-        double res[NS + 1];
-        FxFold<NS>{B, L, h, mone, nzero}.template run<NS, 0>(res);
+        double res[NO];
+        if constexpr (EX) {
+            double D[NG][NO];
+            series_fp64<NS, HI>(B, L, D);
+            moebius_fp64<NS, HI>(D);
+            FxFoldD<NS, HI>{D, h}.template run<NS, 0>(res);
+        } else {
+            FxFold<NS, HI>{B, L, h, mone, nzero}.template run<NS, 0>(res);
+        }
 #pragma unroll
-        for (int i = 0; i <= NS; ++i) accN[i] = fma(res[i], W, accN[i]);
+        for (int i = 0; i < NO; ++i) accN[i] = fma(res[i], W, accN[i]);
     }
     // output order o is eps^(lo+o), i.e. index lo + o + NS of accN
 #pragma unroll
     for (int o = 0; o < LMAX; ++o) {
         double v = 0.0;
 #pragma unroll
-        for (int i = 0; i <= NS; ++i)
+        for (int i = 0; i < NO; ++i)
             if (i == lo + o + NS) v = accN[i];
         if (o < nord) acc[o] = v;
     }
@@ -671,7 +826,7 @@ __device__ __forceinline__ void fx_stage(FxShared &S, const QmcLaunch &Lc) {
         const uint64_t b = S.cfix[m];
         if constexpr (MIXED) {
             S.cfix[m] = __float_as_uint((float)__longlong_as_double((long long)b));
-        } else if (ns < 4) {                     // (four: the double itself)
+        } else if (ns < 3) {                     // (three and more: the double itself)
             const int be = (int)(b >> 52);
             const uint64_t mant = (b & 0x000FFFFFFFFFFFFFULL) | (be ? 1ULL << 52 : 0);
             const int x = be - 1075 + sh[m < nU ? 0 : 1];            // c 2^sh = mant 2^x
@@ -687,7 +842,7 @@ __device__ __forceinline__ void fx_stage(FxShared &S, const QmcLaunch &Lc) {
 #ifndef QMC_FX6_MINB
 #define QMC_FX6_MINB 6
 #endif
-template <int DMAX, int SMAX, int LMAX, bool MIXED, int BLOCK>
+template <int DMAX, int SMAX, int LMAX, bool MIXED, int BLOCK, int HI>
 __global__ void __launch_bounds__(BLOCK, (DMAX > 3 ? QMC_FX6_MINB : QMC_FX_MINB) * 128 / BLOCK) qmc_real_kernel(QmcLaunch Lc, int ppt) {
     FxShared &S = fx_shared();
     const int lo = Lc.lo, nord = Lc.norders;
@@ -753,12 +908,12 @@ __global__ void __launch_bounds__(BLOCK, (DMAX > 3 ? QMC_FX6_MINB : QMC_FX_MINB)
         if (k0 < kt1) {
             const uint64_t kend = min(kt1, k0 + (uint64_t)ppt);
             const int ns = S.ns;
-            if (ns == 0) fx_points<DMAX, BLOCK, 0, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc);
-            else if (ns == 1) fx_points<DMAX, BLOCK, 1, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc);
-            else if (ns == 2 || SMAX < 3) fx_points<DMAX, BLOCK, 2, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc);
+            if (ns == 0) fx_points<DMAX, BLOCK, 0, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc);
+            else if (ns == 1) fx_points<DMAX, BLOCK, 1, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc);
+            else if (ns == 2 || SMAX < 3) fx_points<DMAX, BLOCK, 2, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc);
             else if constexpr (SMAX >= 3) {
-                if (ns == 3) fx_points<DMAX, BLOCK, 3, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc);
-                else fx_points<DMAX, BLOCK, 4, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc);
+                if (ns == 3) fx_points<DMAX, BLOCK, 3, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc);
+                else fx_points<DMAX, BLOCK, 4, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc);
             }
         }
         // block reduction: warp shuffles, then warps in index order
@@ -789,27 +944,29 @@ constexpr int fx_dyn_smem(int prow, bool mixed) {
     return (int)sizeof(FxShared) + 16 * DMAX * BLOCK + (mixed ? 4 : 8) * prow * DMAX * BLOCK;
 }
 
-template <int DMAX, int SMAX, int LMAX, bool MIXED, int BLOCK>
+template <int DMAX, int SMAX, int LMAX, bool MIXED, int BLOCK, int HI>
 bool fx_allow() {
-    static const bool ok = cudaFuncSetAttribute(qmc_real_kernel<DMAX, SMAX, LMAX, MIXED, BLOCK>,
+    static const bool ok = cudaFuncSetAttribute(qmc_real_kernel<DMAX, SMAX, LMAX, MIXED, BLOCK, HI>,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 fx_dyn_smem<DMAX, BLOCK>(QMC_EMAX, MIXED)) == cudaSuccess;
     return ok;
 }
 
-template <int DMAX, int SMAX, int LMAX, bool MIXED, int BLOCK>
-int fx_launch(const QmcLaunch *L, int ppt, int grid, cudaStream_t st) {
-    if (L->prow < 1 || L->prow > QMC_EMAX || !fx_allow<DMAX, SMAX, LMAX, MIXED, BLOCK>()) return -1;
-    qmc_real_kernel<DMAX, SMAX, LMAX, MIXED, BLOCK>
-        <<<grid, BLOCK, fx_dyn_smem<DMAX, BLOCK>(L->prow, MIXED), st>>>(*L, ppt);
+// One block size per kernel: the tile's points over its threads, whatever
+// block and points per thread made the tile
+template <int DMAX, int SMAX, int LMAX, bool MIXED, int BLOCK, int HI>
+int fx_launch(const QmcLaunch *L, int grid, cudaStream_t st) {
+    if (L->prow < 1 || L->prow > QMC_EMAX || !fx_allow<DMAX, SMAX, LMAX, MIXED, BLOCK, HI>()) return -1;
+    qmc_real_kernel<DMAX, SMAX, LMAX, MIXED, BLOCK, HI>
+        <<<grid, BLOCK, fx_dyn_smem<DMAX, BLOCK>(L->prow, MIXED), st>>>(*L, (int)((L->tile_k + BLOCK - 1) / BLOCK));
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-template <int DMAX, int SMAX, int LMAX, bool MIXED, int BLOCK>
+template <int DMAX, int SMAX, int LMAX, bool MIXED, int BLOCK, int HI>
 int fx_occupancy(int prow) {
-    if (!fx_allow<DMAX, SMAX, LMAX, MIXED, BLOCK>()) return 0;
+    if (!fx_allow<DMAX, SMAX, LMAX, MIXED, BLOCK, HI>()) return 0;
     int v = 0;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &v, qmc_real_kernel<DMAX, SMAX, LMAX, MIXED, BLOCK>, BLOCK, fx_dyn_smem<DMAX, BLOCK>(prow, MIXED));
+        &v, qmc_real_kernel<DMAX, SMAX, LMAX, MIXED, BLOCK, HI>, BLOCK, fx_dyn_smem<DMAX, BLOCK>(prow, MIXED));
     return e == cudaSuccess ? v : 0;
 }

@@ -87,13 +87,52 @@ QMC_HD qmc_xf qmc_xf_neg(qmc_xf a) {
     return a;
 }
 
-// 1/a (a nonzero): with m = a.m 2^-64 in [1/2, 1) and the hardware's FP32
+// 1/a (a nonzero): Newton-Raphson y <- y + y (1 - m y) on m = a.m 2^-64 in
+// [1/2, 1), y in Q62, from an FP32 reciprocal of the top 24 bits (error
+// about 2^-22), two steps (2^-44, then the Q62 resolution). Relative error
+// below 2^-59.
+QMC_HD qmc_xf qmc_xf_rcp(qmc_xf a) {
+    qmc_xf r;
+    r.neg = a.neg;
+    if (a.m == (1ULL << 63)) {                         // a power of two: exact
+        r.m = a.m;
+        r.e = -a.e;
+        return r;
+    }
+    uint32_t fb = (126u << 23) | (uint32_t)((a.m >> 40) & 0x7FFFFFu);   // m rounded down to float
+    float f, y0;
+#if defined(__CUDA_ARCH__)
+    f = __int_as_float((int)fb);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(f));
+    const uint32_t yb = (uint32_t)__float_as_int(y0);
+#else
+    memcpy(&f, &fb, 4);
+    y0 = 1.0f / f;
+    uint32_t yb;
+    memcpy(&yb, &y0, 4);
+#endif
+    // y0 in (1, 2]: Q62 from its bits (2.0 clamps just below 2^63)
+    int64_t Y = ((yb >> 23) & 0xFF) >= 128 ? (int64_t)0x7FFFFFFFFFFFFFFFLL
+                                           : (int64_t)((1ULL << 62) | ((uint64_t)(yb & 0x7FFFFFu) << 39));
+    for (int it = 0; it < 2; ++it) {
+        const int64_t P = (int64_t)qmc_umulhi64(a.m, (uint64_t)Y);    // m y 2^62
+        const int64_t E = (int64_t)(1ULL << 62) - P;                 // (1 - m y) 2^62
+        Y += qmc_smulhi(Y, E) << 2;
+        if (Y < 0) Y = 0x7FFFFFFFFFFFFFFFLL;            // (never: y < 2)
+    }
+    // 1/|a| = y 2^(-a.e - 1) with y = Y 2^-62 in (1, 2)
+    r.m = (uint64_t)Y << 1;
+    r.e = -a.e - 1;
+    return r;
+}
+
+// The same in about half the instructions: with m = a.m 2^-64 in [1/2, 1) and the hardware's FP32
 // reciprocal y0 of its top 24 bits (24 bits itself, m y0 = 1 - e with
 // |e| < 2^-21), 1/m = y0 (1 + e + e^2) within e^3 < 2^-63: one step of third
 // order. y0 has 24 bits, so m y0 takes two 32 x 32 products and is exact, and
 // y0 (e + e^2) two more (a second-order pair of steps in 64 x 64
 // bits took four high products). Relative error below 2^-61.
-QMC_HD qmc_xf qmc_xf_rcp(qmc_xf a) {
+QMC_HD qmc_xf qmc_xf_rcp3(qmc_xf a) {
     qmc_xf r;
     r.neg = a.neg;
     if (a.m == (1ULL << 63)) {                         // a power of two: exact

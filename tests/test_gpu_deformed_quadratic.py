@@ -1,9 +1,11 @@
 """The deformed evaluator for quadratic F (csrc/qmc_deformed.cuh, GPU) against
-the general deformed kernel, which runs when the requested orders go beyond
-eps^0, on everything it accepts: one to three variables, zero to two of them
-singular, FP64 and mixed precision, every transform and block size; and
+the general deformed kernel, which takes F of higher degree, on everything it
+accepts: one to three variables, zero to two of them singular, FP64 and (sums
+to eps^1 against sums to eps^0) mixed precision, every transform; and
 sectors it does not accept (F of higher degree), which stay on the general
 kernel and still match the oracle."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -14,6 +16,7 @@ from paper_2305_19768_gb300.inputs.integral import Integral
 from paper_2305_19768_gb300.inputs.lattice import lattice_for
 
 from parity import Gpu, assert_close
+from test_gpu_real_integer import general
 
 pytestmark = pytest.mark.gpu
 
@@ -49,18 +52,28 @@ def test_same_sums_as_the_general_kernel(name, transform, mixed, n, block, flags
     try:
         iid = g.load(I)
         qmc.qmc_set_kinematics(g.ctx, np.array(kin))
-        m, nord = (1 if flags else 2), -lo + 1
+        m = 1 if flags else 2
         specs = [dict(integral_id=iid, sector=s, point=p, shifts=m, n=n, seed=11, stream=p * 20 + s, flags=flags,
                       **{"lambda": 0.6}) for p in range(len(kin)) for s in range(len(I.sectors))]
-        a, fa, _ = g.eval(iid, specs, lo, nord)
-        b, fb, _ = g.eval(iid, specs, lo, nord + 1)
-        assert fa == fb
-        a = a.reshape(len(specs), m, nord, 2)
-        b = b.reshape(len(specs), m, nord + 1, 2)[:, :, :nord]
-        for i, sp in enumerate(specs):
-            o, A, C = _oracle(I, sp, kin[sp["point"]], m, lo, nord, transform)
-            bar = 2e-12 * np.maximum(np.abs(o), A[..., None]) + 6e-16 * C[..., None]
-            assert np.all(np.abs(a[i] - b[i]) <= bar), (sp, float(np.max(np.abs(a[i] - b[i]) / bar)))
+        gid = g.load(general(I, Fraction(1, 10 ** 250)))
+        for hi in (0, 1):
+            nord = hi - lo + 1
+            a, fa, _ = g.eval(iid, specs, lo, nord)
+            if mixed:
+                b, fb, _ = g.eval(iid, specs, lo, 2 - lo if hi == 0 else 1 - lo)
+                nb = 2 - lo if hi == 0 else 1 - lo
+            else:
+                b, fb, _ = g.eval(gid, [dict(sp, integral_id=gid) for sp in specs], lo, nord)
+                nb = nord
+            assert fa == fb
+            a = a.reshape(len(specs), m, nord, 2)
+            b = b.reshape(len(specs), m, nb, 2)
+            for i, sp in enumerate(specs):
+                o, A, C = _oracle(I, sp, kin[sp["point"]], m, lo, nord, transform)
+                bar = 2e-12 * np.maximum(np.abs(o), A[..., None]) + 6e-16 * C[..., None]
+                k = min(nb, nord)
+                err, bar = np.abs(a[i][:, :k] - b[i][:, :k]), bar[:, :k]
+                assert np.all(err <= bar), (sp, hi, float(np.max(err / bar)))
     finally:
         g.close()
 
