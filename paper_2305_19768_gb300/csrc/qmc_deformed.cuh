@@ -18,32 +18,45 @@
 //  * at a corner t_V = 0 the rows of the Jacobian of the zeroed variables are
 //    diagonal with entries rho_j, which cancel the 1 / rho_j of the integrand:
 //    determinant and products are formed over the other variables only;
-//  * transform, weight, 1/t, ln t, reciprocals and logarithms run on the
-//    integer pipe, and the corners are folded variable by variable as in
+//  * the Jacobian is 1 - i diag(p) M with p = lambda t (1 - t) and M symmetric,
+//    M_jj = A_jj + (1 - 2t) / (t (1 - t)) g_j: its minors take one FMA each;
+//  * x^-e enters as conj(x)^e / |x|^2e: the complex products collect in FP64,
+//    the norms as mantissas, whose logarithm is also the corner's Re L; its
+//    Im L is the sum of the factors' principal arguments in fixed point (an
+//    integer arctangent), so that no branch has to be restored;
+//  * transform, weight, the real factors of the deformation, 1/t, ln t,
+//    reciprocals, logarithms and arguments run on the integer pipe (an FP64
+//    negation or doubling by itself takes the FP64 pipe too: both go through
+//    the bits), and the corners are folded variable by variable as in
 //    qmc_real.cuh (complex corner series, real factors).
-// Measured (evaluations/s, general kernel -> this one): massive box, 64 points
-// at n = 10007, 1.74e9 -> 5.9e9 (90 FP64 instructions per evaluation, pipe
-// 93 % busy); the same in mixed precision, 256 points at n = 1009,
-// 2.85e9 -> 5.4e9; massless box, 16 physical points at n = 4001, 5.9e8 ->
-// 1.06e9 (453, pipe 90 %). 16 warps (128 registers) beat 12 and 8 even with
-// the FP64 kernel's spills.
+// Measured (evaluations/s, general kernel -> this one; FP64 instructions per
+// evaluation): massive box, 64 points at n = 10007, 1.74e9 (175, and as many
+// switched off) -> 5.9e9 (90) with the Jacobian entry by entry -> 7.4e9 (68,
+// pipe 87 % busy); massless box, 16 physical points at n = 4001, 5.9e8 (555)
+// -> 1.06e9 (453) with complex logarithms of the factors' product -> 1.86e9
+// (204, 78 %); the massive box in mixed precision, 256 points at n = 1009,
+// 2.85e9 -> 6.1e9. 24 warps per SM (85 registers) are as good as 16 for the
+// massless box and better for the others (6.7e9 -> 7.4e9; 5.4e9 -> 6.1e9).
 // MIXED: derivatives of F and U(z), F(z) from FP32 monomial products in the
 // order of the general mixed kernel, everything after them in FP64.
 
 struct alignas(16) FdShared {
     uint64_t logtab[3 * QMC_LOG_TABLE_ROWS + 1];
-    double atantab[2 * QMC_ATAN_TABLE_ROWS];
+    int64_t atan60[QMC_ATAN_TABLE_ROWS];   // atan(j / 64) 2^60
     uint32_t exps[QMC_MAXMONO];      // FP64: variables in slot order (singular first)
     uint4 mdesc[QMC_MAXMONO];        // MIXED: factors as in FxShared, original variable order
     double cval[QMC_MAXMONO];
     float cvalf[QMC_MAXMONO];
     // F(t) = qc[0] + sum_j t_j (qc[1+j] + qc[4+j] t_j) + qc[7] t_0 t_1 + qc[8] t_0 t_2 + qc[9] t_1 t_2 (slots)
     double qc[10];
-    int32_t qmask;                   // bits 0..2: qc[7..9] present
+    double qa[3];                    // 2 qc[4..6]
+    int32_t qmask;                   // bits 0..2: qc[7..9] present; 3..5: qc[4..6]
     int32_t d, ns, nU, nF, dbase, prow;
     int32_t dFoff[3], dFn[3], Hoff[QMC_NHESS], Hn[QMC_NHESS];
     int32_t perm[QMC_DMAX], slotof[QMC_DMAX], avar[QMC_DMAX], bvar[QMC_DMAX];
     double bd[QMC_DMAX], lam[QMC_DMAX];
+    uint64_t lamm[QMC_DMAX];         // lambda as mantissa, exponent and sign
+    int32_t lame[QMC_DMAX], lamneg[QMC_DMAX];
     int32_t regular, u0, f0, u1, f1;
     double delta[QMC_DMAX];
     uint64_t dfix[QMC_DMAX], qz[QMC_DMAX];
@@ -57,19 +70,66 @@ struct alignas(16) FdShared {
 };
 __device__ __forceinline__ FdShared &fd_shared() { return *reinterpret_cast<FdShared *>(qmc_fx_raw); }
 
-// 0.5 ln(a / b) of positive finite a, b, and 1 / x: integer pipe, out of line
-__device__ __noinline__ double fd_half_log_ratio(double a, double b) {
-    const qmc_xf x = qmc_xf_of(a), y = qmc_xf_of(b);
-    if (x.m == 0 || y.m == 0) return a * (1.0 / b);      // (the integrand is singular there)
-    const FxM q = fx_norm(fx_mul(FxM{x.m, x.e}, FxM{qmc_xf_rcp3(y).m, qmc_xf_rcp3(y).e}));
-    return fx_half(qmc_ilog_xf(qmc_xf{q.m, q.e, 0}, fd_shared().logtab));
-}
-__device__ __noinline__ double fd_rcp(double x) {
+// Positive FP64 values as mantissa and exponent; zero (or worse) gives a tiny
+// one: the integrand is singular there and the sum not finite
+__device__ __forceinline__ FxM fd_of(double x) {
     const qmc_xf a = qmc_xf_of(x);
-    if (a.m == 0) return 1.0 / x;
-    return qmc_xf_to_double(qmc_xf_rcp3(a));
+    return a.m ? FxM{a.m, a.e} : FxM{1ULL << 63, -1022};
 }
-__device__ __noinline__ double fd_atan2(double y, double x) { return qatan2(y, x, fd_shared().atantab); }
+__device__ __forceinline__ FxM fd_rcp(FxM a) {
+    const qmc_xf r = qmc_xf_rcp3(qmc_xf{a.m, a.e, 0});
+    return FxM{r.m, r.e};
+}
+__device__ __noinline__ double fd_half_log(FxM x) {
+    return fx_half(qmc_ilog_xf(qmc_xf{x.m, x.e, 0}, fd_shared().logtab));
+}
+
+// Argument of x + i y times 2^60 in fixed point, in (-pi, pi]; with m0 a zero
+// y counts as -0 (the prescription F - i0). The reduction of qatan2: with
+// mn <= mx the smaller and larger of |x|, |y| and c = j/64 nearest mn/mx,
+// atan(mn/mx) = atan(c) + atan(d), d = (mn - c mx) / (mx + c mn), |d| <= 2^-7,
+// and atan(d) = d - d^3 (1/3 - d^2 (1/5 - d^2 / 7)) (truncation below 2^-66);
+// the inner coefficients in 32 bits. Absolute error a few 2^-60. Out of line.
+__device__ __noinline__ int64_t fd_arg(double y, double x, bool m0) {
+    const qmc_xf ax = qmc_xf_of(x), ay = qmc_xf_of(y);
+    const bool sw = ay.e > ax.e || (ay.e == ax.e && ay.m > ax.m);
+    const uint64_t mx = sw ? ay.m : ax.m, ms = sw ? ax.m : ay.m;
+    const int dd = sw ? ay.e - ax.e : ax.e - ay.e;
+    int64_t r = 0;
+    if (mx != 0 && ms != 0 && dd < 64) {
+        const uint64_t mn = ms >> dd;                  // both in units of mx's last place
+        int j = 0;
+        if (dd <= 7) {
+            const float fs = __int_as_float(0x3F800000 | (int)((ms >> 40) & 0x7FFFFFu));
+            const float fx = __int_as_float(0x3F800000 | (int)((mx >> 40) & 0x7FFFFFu));
+            j = min(__float2int_rn(__fdividef(fs, fx) * __int_as_float((133 - dd) << 23)), 64);
+        }
+        const int64_t num = (int64_t)((mn << 6) - (uint64_t)j * mx);      // 64 (mn - c mx)
+        const uint64_t an = (uint64_t)(num < 0 ? -num : num);
+        const FxM den = fx_norm(FxM{(mx >> 1) + __umul64hi(mn, (uint64_t)j << 57), 0});   // (mx + c mn) / 2
+        const FxM q = fd_rcp(FxM{den.m, 0});           // 2^63 / den.m
+        const uint64_t d = __umul64hi(an, q.m) << (q.e + 1 - den.e);      // |d| 2^70
+        const uint64_t z = __umul64hi(d, d);           // d^2 2^76
+        const uint32_t z45 = (uint32_t)(z >> 31);
+        const uint32_t c5 = 0x33333333u - (__umulhi(z45, 0x24924925u) >> 13);
+        const uint64_t c3 = 0x2AAAAAAAAAAAAAABULL - (((uint64_t)z45 * c5) >> 14);
+        const uint64_t at = (d >> 10) - (__umul64hi(__umul64hi(d, z), c3) >> 21);
+        r = fd_shared().atan60[j] + (num < 0 ? -(int64_t)at : (int64_t)at);
+    }
+    if (sw) r = 0x1921FB54442D1847LL - r;
+    if (ax.neg) r = 0x3243F6A8885A308DLL - r;
+    return (ay.neg || (m0 && ay.m == 0)) ? -r : r;
+}
+// -x or x on the sign bit (a negation by itself takes the FP64 pipe)
+__device__ __forceinline__ double fd_signed(double x, bool neg) {
+    return __hiloint2double(__double2hiint(x) ^ (neg ? (int)0x80000000 : 0), __double2loint(x));
+}
+// a 2^-57 as FP64
+__device__ __forceinline__ double fd_from57(int64_t a) {
+    const uint64_t u = (uint64_t)(a < 0 ? -a : a);
+    if (u == 0) return 0.0;
+    return fd_signed(fx_pack(fx_norm(FxM{u, 6})), a < 0);
+}
 
 // FP32 <-> FP64 conversions on the integer pipe (normal range; below it 0)
 __device__ __forceinline__ float fd_to_float(double x) {
@@ -93,31 +153,26 @@ __device__ __forceinline__ double fd_to_double(float x) {
 
 // complex arithmetic in FMAs (an FP64 multiply holds the pipe longer than an FMA)
 struct FdOps {
-    double mone, nzero;
+    double mone, nzero, one;
     __device__ __forceinline__ double mul(double a, double b) const { return fma(a, b, nzero); }
-    __device__ __forceinline__ double add(double a, double b) const { return fma(b, -mone, a); }
+    __device__ __forceinline__ double add(double a, double b) const { return fma(b, one, a); }
+    // 2 a on the exponent (a normal, or 0 for anything below)
+    __device__ __forceinline__ double dbl(double a) const {
+        const int h = __double2hiint(a);
+        return (h & 0x7FF00000) ? __hiloint2double(h + 0x00100000, __double2loint(a)) : 0.0;
+    }
     __device__ __forceinline__ double sub(double a, double b) const { return fma(b, mone, a); }
     __device__ __forceinline__ dc mul(dc a, dc b) const {
         return dc{fma(a.re, b.re, mul(-a.im, b.im)), fma(a.re, b.im, mul(a.im, b.re))};
     }
     __device__ __forceinline__ dc sub(dc a, dc b) const { return dc{sub(a.re, b.re), sub(a.im, b.im)}; }
-    // num *= x^e or den *= x^-e
-    __device__ __forceinline__ void ipow(dc x, int e, dc &num, bool &hn, dc &den, bool &hd) const {
-        if (e == 0) return;
-        const int a = e > 0 ? e : -e;
-        dc p = x;
-        if (a > 1) {
-            const dc x2 = dc{fma(x.re, x.re, mul(-x.im, x.im)), mul(x.re + x.re, x.im)};
-            p = a == 3 ? mul(x2, x) : x2;
-            if (a == 4) p = dc{fma(x2.re, x2.re, mul(-x2.im, x2.im)), mul(x2.re + x2.re, x2.im)};
-        }
-        if (e > 0) {
-            num = hn ? mul(num, p) : p;
-            hn = true;
-        } else {
-            den = hd ? mul(den, p) : p;
-            hd = true;
-        }
+    // x^a, 1 <= a <= 4
+    __device__ __forceinline__ dc pow(dc x, int a) const {
+        if (a == 1) return x;
+        const dc x2 = dc{fma(x.re, x.re, mul(-x.im, x.im)), mul(dbl(x.re), x.im)};
+        if (a == 2) return x2;
+        if (a == 3) return mul(x2, x);
+        return dc{fma(x2.re, x2.re, mul(-x2.im, x2.im)), mul(dbl(x2.re), x2.im)};
     }
 };
 
@@ -177,11 +232,13 @@ template <int BLOCK> __device__ __noinline__ fc fd_polyc(int m0, int count) {
 }
 
 struct FdPoint {
-    double t[3], s[3], p[3], r[3];   // t; lambda (1 - t); lambda t (1 - t); lambda (1 - 2t)  (slots)
+    // per slot: t, lambda t (1 - t), (1 - 2t) / (t (1 - t)), and lambda (1 - t) of the singular ones
+    double t[3], p[3], k[3], s[3];
     float tf[3];                     // FP32 t, original variable order (MIXED)
 };
 struct FdCorner {
-    dc B, L;
+    dc B, L;                         // the corner value is B q
+    FxM q;
 };
 
 // The corner with the slots of V at t = 0 (D variables, NS of them singular)
@@ -191,37 +248,28 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
     constexpr bool lam = HI > 0 || V != 0;              // needs its eps exponent
     constexpr int NA = D - __builtin_popcount(V);       // variables left
     double g[D];                                        // dF/dt_j
-    double Vd[D], Vo[D][D];                             // J = 1 - i V: diagonal, off-diagonal
-    double y[D];
+    double e[D];                                        // F(t) = c + sum t_j e_j
+    double Ad[D], Ao[3];                                // d2F: diagonal (MIXED), off-diagonal (01, 02, 12)
     dc F, U{1.0, 0.0};
     const bool needU = S.u0 != 0 || (lam && S.u1 != 0);
-#pragma unroll
-    for (int j = 0; j < D; ++j)
-#pragma unroll
-        for (int k = 0; k < D; ++k) Vo[j][k] = 0.0;
-    const int qm = MIXED ? 7 : S.qmask;
+    const int qm = MIXED ? 63 : S.qmask;
     if constexpr (!MIXED) {
 #pragma unroll
         for (int j = 0; j < D; ++j) {
-            g[j] = S.qc[1 + j];
-            if (!(V >> j & 1)) g[j] = fma(S.qc[4 + j], P.t[j] + P.t[j], g[j]);
+            e[j] = S.qc[1 + j];
+            if (!(V >> j & 1)) {
+                if (qm >> (3 + j) & 1) e[j] = fma(S.qc[4 + j], P.t[j], e[j]);
+#pragma unroll
+                for (int k = j + 1; k < D; ++k)
+                    if (!(V >> k & 1) && (qm >> (j + k - 1) & 1)) e[j] = fma(S.qc[6 + j + k], P.t[k], e[j]);
+            }
+            g[j] = e[j];
+            if (!(V >> j & 1) && (qm >> (3 + j) & 1)) g[j] = fma(S.qc[4 + j], P.t[j], g[j]);
+#pragma unroll
+            for (int k = 0; k < D; ++k)
+                if (k != j && (k < j || (V >> j & 1)) && !(V >> k & 1) && (qm >> (j + k - 1) & 1))
+                    g[j] = fma(S.qc[6 + j + k], P.t[k], g[j]);
         }
-#pragma unroll
-        for (int j = 0; j < D; ++j)
-#pragma unroll
-            for (int k = j + 1; k < D; ++k)
-                if (qm >> (j + k - 1) & 1) {
-                    const double A = S.qc[6 + j + k];
-                    if (!(V >> k & 1)) g[j] = fma(A, P.t[k], g[j]);
-                    if (!(V >> j & 1)) g[k] = fma(A, P.t[j], g[k]);
-                    if (!(V >> j & 1) && !(V >> k & 1)) {
-                        Vo[j][k] = o.mul(A, P.p[j]);
-                        Vo[k][j] = o.mul(A, P.p[k]);
-                    }
-                }
-#pragma unroll
-        for (int j = 0; j < D; ++j)
-            if (!(V >> j & 1)) Vd[j] = fma(S.qc[4 + j], P.p[j] + P.p[j], o.mul(P.r[j], g[j]));
     } else {
         // FP32 derivatives, original variable order
 #pragma unroll
@@ -258,73 +306,79 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
 #pragma unroll
                     for (int b = 0; b < 3; ++b)
                         if (pi == a && pk == b) h = Hf[a][b];
-                const double H = fd_to_double(h);
-                if (i == k) Vd[i] = fma(H, P.p[i], o.mul(P.r[i], g[i]));
-                else {
-                    Vo[i][k] = o.mul(H, P.p[i]);
-                    Vo[k][i] = o.mul(H, P.p[k]);
-                }
+                if (i == k) Ad[i] = fd_to_double(h);
+                else Ao[i + k - 1] = fd_to_double(h);
             }
         }
     }
-    // rho_j = 1 - i g_j lambda_j (1 - t_j), z_j = t_j rho_j
-    double gl[D];
+    // y_j = lambda t (1 - t) g_j (z = t - i y); the Jacobian J = 1 - i V with
+    // V = diag(p) M, M_jj = A_jj + k_j g_j, M_jk = A_jk: symmetric, so its
+    // minors take one FMA each with the squares of the couplings
+    double y[D], M[D];
 #pragma unroll
     for (int j = 0; j < D; ++j) {
-        gl[j] = 0.0;
-        y[j] = 0.0;
-        if (V >> j & 1) gl[j] = o.mul(S.lam[j], g[j]);
-        else {
-            if (j < NS || needU || MIXED || (S.regular >> j & 1)) gl[j] = o.mul(P.s[j], g[j]);
-            y[j] = o.mul(P.p[j], g[j]);
-        }
+        y[j] = M[j] = 0.0;
+        if (V >> j & 1) continue;
+        y[j] = o.mul(P.p[j], g[j]);
+        M[j] = fma(P.k[j], g[j], MIXED ? Ad[j] : S.qa[j]);
     }
-    // det J over the remaining variables
     dc J{1.0, 0.0};
     {
         int a[3] = {0, 0, 0}, na = 0;
 #pragma unroll
         for (int j = 0; j < D; ++j)
             if (!(V >> j & 1)) a[na++] = j;
+        // M_x M_z - A_xz^2
+        auto minor2 = [&](int x, int z) {
+            if (!(qm >> (x + z - 1) & 1)) return o.mul(M[x], M[z]);
+            const double A = MIXED ? Ao[x + z - 1] : S.qc[6 + x + z];
+            return fma(M[x], M[z], o.mul(-A, A));
+        };
         if constexpr (NA == 1) {
-            J = dc{1.0, -Vd[a[0]]};
+            J = dc{1.0, o.mul(-P.p[a[0]], M[a[0]])};
         } else if constexpr (NA == 2) {
             const int x = a[0], z = a[1];
-            const double det = fma(Vd[x], Vd[z], o.mul(-Vo[x][z], Vo[z][x]));
-            J = dc{1.0 - det, -(Vd[x] + Vd[z])};
+            J.re = fma(o.mul(-P.p[x], P.p[z]), minor2(x, z), o.one);
+            J.im = fma(-P.p[x], M[x], o.mul(-P.p[z], M[z]));
         } else if constexpr (NA == 3) {
-            double m01 = o.mul(Vd[0], Vd[1]), m02 = o.mul(Vd[0], Vd[2]), m12 = o.mul(Vd[1], Vd[2]);
-            if (qm & 1) m01 = fma(-Vo[0][1], Vo[1][0], m01);
-            if (qm & 2) m02 = fma(-Vo[0][2], Vo[2][0], m02);
-            if (qm & 4) m12 = fma(-Vo[1][2], Vo[2][1], m12);
-            double det = o.mul(Vd[0], m12);
-            if (qm & 1) {
-                double c = o.mul(Vo[1][0], Vd[2]);
-                if ((qm & 6) == 6) c = fma(-Vo[1][2], Vo[2][0], c);
-                det = fma(-Vo[0][1], c, det);
+            const double c01 = minor2(0, 1), c02 = minor2(0, 2), c12 = minor2(1, 2);
+            double det = o.mul(M[0], c12);
+            if (qm & 3) {
+                // - A01^2 M2 - A02^2 M1 + 2 A01 A02 A12
+                const double a01 = MIXED ? Ao[0] : S.qc[7], a02 = MIXED ? Ao[1] : S.qc[8], a12 = MIXED ? Ao[2] : S.qc[9];
+                if (qm & 1) det = fma(o.mul(-a01, M[2]), a01, det);
+                if (qm & 2) det = fma(o.mul(-a02, M[1]), a02, det);
+                if ((qm & 7) == 7) det = fma(o.mul(o.dbl(a01), a02), a12, det);
             }
-            if (qm & 2) {
-                double c = o.mul(-Vd[1], Vo[2][0]);
-                if ((qm & 5) == 5) c = fma(Vo[1][0], Vo[2][1], c);
-                det = fma(Vo[0][2], c, det);
-            }
-            J = dc{1.0 - o.add(o.add(m01, m02), m12), o.sub(det, o.add(o.add(Vd[0], Vd[1]), Vd[2]))};
+            const double p01 = o.mul(P.p[0], P.p[1]);
+            J.re = fma(-p01, c01, fma(o.mul(-P.p[0], P.p[2]), c02, fma(o.mul(-P.p[1], P.p[2]), c12, o.one)));
+            J.im = fma(-P.p[0], M[0], fma(-P.p[1], M[1], fma(-P.p[2], M[2], o.mul(o.mul(p01, P.p[2]), det))));
         }
     }
     // U and F on the contour
     if constexpr (!MIXED) {
         double re = S.qc[0], im = 0.0;
+        bool first = true;
 #pragma unroll
         for (int j = 0; j < D; ++j) {
             if (V >> j & 1) continue;
-            // t_j (b_j + g_j) / 2 - y_j (A_jj y_j / 2 + sum_{k > j} A_jk y_k);  -y_j g_j
-            re = fma(fx_half(P.t[j]), S.qc[1 + j] + g[j], re);
-            double q = o.mul(S.qc[4 + j], y[j]);
+            // t_j e_j - y_j (A_jj y_j / 2 + sum_{k > j} A_jk y_k);  -y_j g_j
+            re = fma(P.t[j], e[j], re);
+            double q = 0.0;
+            bool any = false;
+            if (qm >> (3 + j) & 1) {
+                q = o.mul(S.qc[4 + j], y[j]);
+                any = true;
+            }
 #pragma unroll
             for (int k = j + 1; k < D; ++k)
-                if (!(V >> k & 1) && (qm >> (j + k - 1) & 1)) q = fma(S.qc[6 + j + k], y[k], q);
-            re = fma(-y[j], q, re);
-            im = fma(-y[j], g[j], im);
+                if (!(V >> k & 1) && (qm >> (j + k - 1) & 1)) {
+                    q = fma(S.qc[6 + j + k], y[k], any ? q : o.nzero);
+                    any = true;
+                }
+            if (any) re = fma(-y[j], q, re);
+            im = fma(-y[j], g[j], first ? o.nzero : im);
+            first = false;
         }
         F = dc{re, im};
         if (needU) {
@@ -334,25 +388,23 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
 #pragma unroll
             for (int j = 0; j < D; ++j)
                 if (V >> j & 1) vm |= 15u << (4 * j);
-            dc z[D];
-#pragma unroll
-            for (int j = 0; j < D; ++j) z[j] = dc{P.t[j], -o.mul(P.t[j], gl[j])};
             for (int m = 0; m < S.nU; ++m) {
-                const uint32_t e = S.exps[m];
-                if (e & vm) continue;
+                const uint32_t ex = S.exps[m];
+                if (ex & vm) continue;
                 const double c = S.cval[m];
-                if (e == 0) {
+                if (ex == 0) {
                     U.re = o.add(U.re, c);
                     continue;
                 }
                 dc v{1.0, 0.0};
-                bool first = true;
+                bool one = true;
 #pragma unroll
                 for (int j = 0; j < D; ++j) {
                     if (V >> j & 1) continue;
-                    for (int q = (int)(e >> (4 * j) & 15u); q > 0; --q) {
-                        v = first ? z[j] : o.mul(v, z[j]);
-                        first = false;
+                    const dc z{P.t[j], -y[j]};
+                    for (int q = (int)(ex >> (4 * j) & 15u); q > 0; --q) {
+                        v = one ? z : o.mul(v, z);
+                        one = false;
                     }
                 }
                 U = dc{fma(c, v.re, U.re), fma(c, v.im, U.im)};
@@ -368,7 +420,7 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
             for (int i = 0; i < D; ++i)
                 if (sl == i) {
                     if (V >> i & 1) zeroed = true;
-                    else zi = o.mul(-P.t[i], gl[i]);
+                    else zi = -y[i];
                 }
             fd_putc<BLOCK>(j, prow, zeroed ? fc{0.0f, 0.0f} : fc{P.tf[j], fd_to_float(zi)});
         }
@@ -380,61 +432,51 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
         F = dc{fd_to_double(f.re), fd_to_double(f.im)};
     }
     if (__double_as_longlong(F.im) > 0) ++signfail;
-    // B = det J / prod rho (kept singular) prod z^a (regular) U^u0 F^f0 and
-    // the corner's exponent L = ln(prod rho^b prod z^b U^u1 F^f1), one complex
-    // logarithm whose argument is restored to the sum of the factors'
-    // principal arguments by an FP32 estimate
-    FdCorner out{dc{1.0, 0.0}, dc{0.0, 0.0}};
-    dc num = J, den{1.0, 0.0}, Xn{1.0, 0.0}, Xd{1.0, 0.0};
-    bool hn = NA > 0, hd = false, xn = false, xd = false;
-    float sarg = 0.0f;
+    // The corner value J / prod rho (kept singular) prod z^a (regular) U^u0
+    // F^f0, a factor x^-e as conj(x)^e / |x|^2e: B collects the complex
+    // products and q the real ones, in mantissas. Its exponent
+    // L = sum of e ln x over rho^b, z^b, U^u1, F^f1: ln |x|^2 of the product
+    // of norms in mantissas, and the principal arguments in fixed point.
+    FdCorner out;
+    dc B = J;
+    FxM den{1ULL << 63, 0}, np{1ULL << 63, 0}, nn{1ULL << 63, 0};
+    int64_t arg = 0;
+    auto factor = [&](dc x, FxM n, int e0, int e1, bool m0) {
+        if (e0) {
+            const int a = e0 < 0 ? -e0 : e0;
+            B = o.mul(B, o.pow(e0 < 0 ? conj_(x) : x, a));
+            if (e0 < 0) den = fx_norm(fx_mul(den, fx_pow(n, n, a)));
+        }
+        if (lam && e1) {
+            const int a = e1 < 0 ? -e1 : e1;
+            if (e1 > 0) np = fx_norm(fx_mul(np, fx_pow(n, n, a)));
+            else nn = fx_norm(fx_mul(nn, fx_pow(n, n, a)));
+            arg += (int64_t)e1 * (fd_arg(x.im, x.re, m0) >> 3);
+        }
+    };
 #pragma unroll
     for (int j = 0; j < D; ++j) {
         if (j < NS) {
-            const dc rho{1.0, -gl[j]};
+            // rho = 1 - i gl
+            if ((V >> j & 1) && !lam) continue;
+            const double gl = o.mul((V >> j & 1) ? S.lam[j] : P.s[j], g[j]);
+            const FxM n = fd_of(fma(gl, gl, o.one));
             if (!(V >> j & 1)) {
-                den = hd ? o.mul(den, rho) : rho;
-                hd = true;
+                B = dc{fma(-gl, B.im, B.re), fma(gl, B.re, B.im)};
+                den = fx_norm(fx_mul(den, n));
             }
-            if constexpr (lam) {
-                o.ipow(rho, S.bvar[j], Xn, xn, Xd, xd);
-                sarg = fmaf((float)S.bvar[j], arg32(rho, false), sarg);
-            }
+            factor(dc{1.0, -gl}, n, 0, S.bvar[j], false);
         } else if (S.regular >> j & 1) {
-            const dc z{P.t[j], -o.mul(P.t[j], gl[j])};
-            o.ipow(z, S.avar[j], num, hn, den, hd);
-            if constexpr (lam)
-                if (S.bvar[j] != 0) {
-                    o.ipow(z, S.bvar[j], Xn, xn, Xd, xd);
-                    sarg = fmaf((float)S.bvar[j], arg32(z, false), sarg);
-                }
+            const dc z{P.t[j], -y[j]};
+            factor(z, fd_of(fma(z.re, z.re, o.mul(z.im, z.im))), S.avar[j], S.bvar[j], false);
         }
     }
-    o.ipow(U, S.u0, num, hn, den, hd);
-    o.ipow(F, S.f0, num, hn, den, hd);
-    if (hd) {
-        const double q = fd_rcp(fma(den.re, den.re, o.mul(den.im, den.im)));
-        const dc di{o.mul(den.re, q), o.mul(-den.im, q)};
-        out.B = hn ? o.mul(num, di) : di;
-    } else {
-        out.B = num;
-    }
-    if constexpr (lam) {
-        if (S.u1 != 0) {
-            o.ipow(U, S.u1, Xn, xn, Xd, xd);
-            sarg = fmaf((float)S.u1, arg32(U, false), sarg);
-        }
-        if (S.f1 != 0) {
-            o.ipow(F, S.f1, Xn, xn, Xd, xd);
-            sarg = fmaf((float)S.f1, arg32(F, true), sarg);
-        }
-        const dc X = xd ? (xn ? o.mul(Xn, conj_(Xd)) : conj_(Xd)) : Xn;   // |Xd|^2 Xn / Xd
-        const double phi = fd_atan2(X.im, X.re);
-        const float kf = rintf((sarg - __double2float_rn(phi)) * 0.15915494f);
-        const double nn = xn ? fma(Xn.re, Xn.re, o.mul(Xn.im, Xn.im)) : 1.0;
-        const double nd = xd ? fma(Xd.re, Xd.re, o.mul(Xd.im, Xd.im)) : 1.0;
-        out.L = dc{fd_half_log_ratio(nn, nd), kf == 0.0f ? phi : fma((double)kf, 2.0 * CUDART_PI, phi)};
-    }
+    if (needU) factor(U, fd_of(fma(U.re, U.re, o.mul(U.im, U.im))), S.u0, S.u1, false);
+    factor(F, fd_of(fma(F.re, F.re, o.mul(F.im, F.im))), S.f0, S.f1, true);
+    out.B = B;
+    out.q = fd_rcp(den);
+    out.L = dc{0.0, 0.0};
+    if constexpr (lam) out.L = dc{fd_half_log(fx_norm(fx_mul(np, fd_rcp(nn)))), fd_from57(arg)};
     return out;
 }
 
@@ -445,14 +487,21 @@ template <int D, int BLOCK, int NS, int HI, bool MIXED> struct FdFold {
     const double (&h)[SlotArr<NS>::N][NS + HI + 1];
     int prow;
     int &signfail;
+    FxM &q0;                          // NS = 0: the corner's real factor, left to the weight
 
     template <int Q, int V>
     __device__ __forceinline__ void run(dc (&out)[Q + __builtin_popcount(V) + HI + 1]) const {
         constexpr int pv = __builtin_popcount(V);
         if constexpr (Q == 0) {
             const FdCorner c = fd_corner<D, BLOCK, NS, HI, V, MIXED>(P, o, prow, signfail);
-            out[0] = c.B;
-            if constexpr (pv + HI >= 1) out[1] = o.mul(c.B, c.L);
+            if constexpr (NS == 0) {
+                q0 = c.q;
+                out[0] = c.B;
+            } else {
+                const double q = qmc_xf_to_double(qmc_xf{c.q.m, c.q.e, 0});
+                out[0] = dc{o.mul(c.B.re, q), o.mul(c.B.im, q)};
+            }
+            if constexpr (pv + HI >= 1) out[1] = o.mul(out[0], c.L);
             if constexpr (pv + HI >= 2) out[2] = o.mul(out[1], dc{fx_half(c.L.re), fx_half(c.L.im)});
             if constexpr (pv + HI >= 3) out[3] = o.mul(out[2], dc{c.L.re * (1.0 / 3), c.L.im * (1.0 / 3)});
         } else {
@@ -494,7 +543,7 @@ __device__ __forceinline__ void fd_points(const QmcLaunch &Lc, uint64_t k0, uint
             walk[i * BLOCK] = make_uint4((uint32_t)Q, (uint32_t)(Q >> 32), (uint32_t)r0, (uint32_t)R);
         }
     }
-    const FdOps o{S.mone, S.nzero};
+    const FdOps o{S.mone, S.nzero, fd_signed(S.mone, true)};
     constexpr int NO = NS + HI + 1;
     dc accN[NO];
 #pragma unroll
@@ -511,30 +560,46 @@ __device__ __forceinline__ void fd_points(const QmcLaunch &Lc, uint64_t k0, uint
             const FxCoord u = fx_next(walk[i * BLOCK], S.zmod[i], S.qz[i], S.rz[i], n32, S.job.inv_n, S.delta[i],
                                       S.dfix[i], walk + i * BLOCK);
             zero |= u.y.m == 0;
-            // t and 1 - t
-            FxM t, v;
+            // t, 1 - t and 1 - 2t (c, negative for t > 1/2)
+            FxM t, v, c;
+            bool cneg;
             if (Lc.transform == 0) {
                 const FxM s = fx_korobov(u);
                 const FxM b = fx_one_minus(s);
                 t = u.lower ? s : b;
                 v = u.lower ? b : s;
+                const uint64_t S2 = s.e >= -64 ? (s.m >> (-1 - s.e)) << 1 : 0;   // 2s (0 for s = 1/2)
+                c = (S2 != 0 || s.e == -1) ? FxM{0 - S2, -1} : FxM{1ULL << 63, 0};
+                cneg = !u.lower;
                 w = fx_norm(fx_mul(w, FxM{__umul64hi(u.y.m, u.big), u.y.e}));
-            } else if (Lc.transform == 1) {             // baker
-                t = FxM{u.y.m, u.y.e + 1};
-                const uint64_t c = 0 - 2 * u.Y;         // 1 - 2y; 0 (u = 1/2): exactly zero
-                v = fx_norm(FxM{c, -1});
-                if (u.Y == 0) v = FxM{1ULL << 63, 0};
-                if (u.Y == 1ULL << 63) v.m = 0;
             } else {
-                t = u.lower ? u.y : FxM{u.big, -1};
-                v = u.lower ? FxM{u.big, -1} : u.y;
+                if (Lc.transform == 1) {                // baker: t = 2y
+                    t = FxM{u.y.m, u.y.e + 1};
+                    v = fx_norm(FxM{0 - 2 * u.Y, -1});  // 1 - 2y
+                    if (u.Y == 0) v = FxM{1ULL << 63, 0};
+                    if (u.Y == 1ULL << 63) v = FxM{1ULL << 63, -61};   // t = 1: p -> 0 with p k = -lambda
+                } else {
+                    t = u.lower ? u.y : FxM{u.big, -1};
+                    v = u.lower ? FxM{u.big, -1} : u.y;
+                }
+                const double x = fx_pack(v) - fx_pack(t);
+                cneg = x < 0.0;
+                const qmc_xf xc = qmc_xf_of(fabs(x));
+                c = FxM{xc.m, xc.m ? xc.e : 0};
             }
-            const double td = fx_pack(t), vd = v.m ? fx_pack(v) : 0.0;
+            const double td = fx_pack(t);
             P.t[i] = td;
-            const double lm = S.lam[i];
-            P.s[i] = o.mul(lm, vd);
-            P.p[i] = o.mul(td, P.s[i]);
-            P.r[i] = fma(-lm, td, P.s[i]);
+            // the real factors of the deformation, by mantissas
+            const FxM lm{S.lamm[i], S.lame[i]};
+            const FxM tv = fx_norm(fx_mul(t, v));
+            c = fx_norm(c);
+            if (c.m == 0 || c.e < -64) c.m = 0;
+            P.p[i] = P.k[i] = P.s[i] = 0.0;
+            if (lm.m) {
+                P.p[i] = fd_signed(fx_pack(fx_norm(fx_mul(lm, tv))), S.lamneg[i] != 0);
+                if (i < NS) P.s[i] = fd_signed(fx_pack(fx_norm(fx_mul(lm, v))), S.lamneg[i] != 0);
+            }
+            if (c.m) P.k[i] = fd_signed(fx_pack(fx_norm(fx_mul(c, fd_rcp(tv)))), cneg);
             if constexpr (MIXED) {
                 const float f = fd_to_float(td);
                 const int pj = S.perm[i];
@@ -549,8 +614,6 @@ __device__ __forceinline__ void fd_points(const QmcLaunch &Lc, uint64_t k0, uint
             }
         }
         if (zero) continue;
-        double W = 1.0;
-        if (Lc.transform == 0) W = fx_pack(fx_norm(fx_mul(fx_mul(w, w), w)));
         double h[NSA][NO];
 #pragma unroll
         for (int q = 0; q < NS; ++q) {
@@ -559,7 +622,13 @@ __device__ __forceinline__ void fd_points(const QmcLaunch &Lc, uint64_t k0, uint
             if constexpr (NS + HI > 2) h[q][2] = o.mul(h[q][1], fx_half(bl[q]));
         }
         dc res[NO];
-        FdFold<D, BLOCK, NS, HI, MIXED>{P, o, h, Lc.prow, signfail}.template run<NS, 0>(res);
+        FxM q0{1ULL << 63, 0};
+        FdFold<D, BLOCK, NS, HI, MIXED>{P, o, h, Lc.prow, signfail, q0}.template run<NS, 0>(res);
+        // the weight (1 without korobov3) and, for NS = 0, the corner's factor
+        FxM wt{1ULL << 63, 0};
+        if (Lc.transform == 0) wt = fx_norm(fx_mul(fx_mul(w, w), w));
+        if constexpr (NS == 0) wt = fx_norm(fx_mul(wt, q0));
+        const double W = qmc_xf_to_double(qmc_xf{wt.m, wt.e, 0});
 #pragma unroll
         for (int i = 0; i < NO; ++i) {
             accN[i].re = fma(res[i].re, W, accN[i].re);
@@ -586,7 +655,8 @@ __device__ __forceinline__ void fd_stage(FdShared &S, const QmcLaunch &Lc) {
     // FP64: only U and F are read; mixed precision also the derivatives of F
     const int nm = MIXED ? src->nmono : nU + nF;
     if (threadIdx.x < 10) S.qc[threadIdx.x] = 0.0;
-    if (threadIdx.x == 10) S.qmask = 0;
+    if (threadIdx.x >= 10 && threadIdx.x < 13) S.qa[threadIdx.x - 10] = 0.0;
+    if (threadIdx.x == 13) S.qmask = 0;
     int slot[3], next = ns;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -637,7 +707,8 @@ __device__ __forceinline__ void fd_stage(FdShared &S, const QmcLaunch &Lc) {
                 int idx = 0;
                 if (first >= 0) idx = second < 0 ? 1 + first : (first == second ? 4 + first : 6 + first + second);
                 atomicAdd(&S.qc[idx], v);
-                if (idx >= 7 && v != 0.0) atomicOr(&S.qmask, 1 << (idx - 7));
+                if (idx >= 4 && idx < 7) atomicAdd(&S.qa[idx - 4], v + v);
+                if (idx >= 4 && v != 0.0) atomicOr(&S.qmask, idx >= 7 ? 1 << (idx - 7) : 8 << (idx - 4));
             }
         }
     }
@@ -682,10 +753,13 @@ __device__ __forceinline__ void fd_stage(FdShared &S, const QmcLaunch &Lc) {
 }
 
 #ifndef QMC_FD_MINB
-#define QMC_FD_MINB 4
+#define QMC_FD_MINB 6
+#endif
+#ifndef QMC_FDM_MINB
+#define QMC_FDM_MINB 6
 #endif
 template <bool MIXED, int BLOCK, int HI>
-__global__ void __launch_bounds__(BLOCK, QMC_FD_MINB * 128 / BLOCK) qmc_deformed_kernel(QmcLaunch Lc, int ppt) {
+__global__ void __launch_bounds__(BLOCK, (MIXED ? QMC_FDM_MINB : QMC_FD_MINB) * 128 / BLOCK) qmc_deformed_kernel(QmcLaunch Lc, int ppt) {
     constexpr int LMAX = 4;
     FdShared &S = fd_shared();
     const int lo = Lc.lo, nord = Lc.norders;
@@ -696,7 +770,8 @@ __global__ void __launch_bounds__(BLOCK, QMC_FD_MINB * 128 / BLOCK) qmc_deformed
         S.nzero = Lc.nzero;
     }
     for (int i = threadIdx.x; i < 3 * QMC_LOG_TABLE_ROWS; i += BLOCK) S.logtab[i] = kLogTable[i];
-    for (int i = threadIdx.x; i < 2 * QMC_ATAN_TABLE_ROWS; i += BLOCK) S.atantab[i] = kAtanTable[i];
+    for (int i = threadIdx.x; i < QMC_ATAN_TABLE_ROWS; i += BLOCK)
+        S.atan60[i] = __double2ll_rn(kAtanTable[2 * i] * 0x1p60) + __double2ll_rn(kAtanTable[2 * i + 1] * 0x1p60);
     for (;;) {
         __syncthreads();  // previous tile fully consumed
         if (threadIdx.x == 0) {
@@ -739,6 +814,10 @@ __global__ void __launch_bounds__(BLOCK, QMC_FD_MINB * 128 / BLOCK) qmc_deformed
             S.rz[i] = (uint32_t)rz;
             S.zmod[i] = (uint32_t)zm;
             S.lam[i] = S.job.lambda[j];
+            const qmc_xf lx = qmc_xf_of(S.job.lambda[j]);
+            S.lamm[i] = lx.m;
+            S.lame[i] = lx.m ? lx.e : 0;
+            S.lamneg[i] = lx.neg;
             if (i == 0) S.minv = minv;
         }
         __syncthreads();
