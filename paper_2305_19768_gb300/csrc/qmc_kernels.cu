@@ -2396,9 +2396,18 @@ __device__ void stage_tile(TileSmem<LMAX> &S, const QmcLaunch &Lc, int jidx) {
 #define QMC_MINB_WIDE_MIXED 4
 #endif
 
+// The Taylor-subtraction classes: their loops wait on local memory and on
+// dependent FP64 operations, and resident warps hide more of that than the
+// registers save. One-loop box in D = 2 - 2 eps, n = 10007, 32 shifts: 9.28 ms
+// at 2 blocks (186 registers), 7.41 at 3, 6.48 at 4 (128), 6.57 at 5; its
+// deformed form at 16 points 111.6, 90.8, 81.9, 79.8.
+#ifndef QMC_MINB_H
+#define QMC_MINB_H 4
+#endif
+
 template <int BLOCK, bool WIDE, bool CPLX_MIXED, bool HS>
 constexpr int qmc_min_blocks() {
-    return HS ? 1
+    return HS ? QMC_MINB_H * 128 / BLOCK
               : WIDE ? ((CPLX_MIXED ? QMC_MINB_WIDE_MIXED : QMC_MINB_WIDE) * 128 + BLOCK - 1) / BLOCK
                      : QMC_MINB * 128 / BLOCK;
 }

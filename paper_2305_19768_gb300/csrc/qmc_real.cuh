@@ -42,9 +42,10 @@
 // the rest and the code stays small. 384-thread blocks for d <= 6 because a
 // block carries the 24.6 KB logarithm table: two of them fit, six of 128 do
 // not. Measured on the double box (n = 10007, evaluations/s): the general
-// kernel 9.7e8; this one 1.89e9 with 16 warps and corners inlined in the fold,
-// 1.91e9 with the rolled corner loop, 2.07e9 at 20 warps, 2.11e9 at 24; the
-// box (n = 100003) 4.2e9 -> 7.4e9 at 16 warps, 8.3e9 at 32.
+// kernel 9.7e8; this one with fixed-point corners for every sector 1.91e9 at 16
+// warps, 2.07e9 at 20, 2.14e9 at 24, and with the general kernel's roundings in
+// the EX sectors 1.66e9 at 24, 1.62e9 at 20 and 1.53e9 at 16. The box
+// (n = 100003) 4.2e9 -> 7.4e9 at 16 warps, 8.3e9 at 32.
 
 // 64-bit mantissa and exponent: value m 2^(e - 63), m not necessarily normalised
 struct FxM {
