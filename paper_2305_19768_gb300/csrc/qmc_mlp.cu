@@ -46,6 +46,7 @@ constexpr int kAStageBytes = kTileM * kBK * 2;           // 16 KB
 constexpr int kBStageBytes = kMaxN * kBK * 2;            // 32 KB
 constexpr int kStageBytes = kAStageBytes + kBStageBytes;
 constexpr int kGemmSmem = kStages * kStageBytes + 1024;  // + slack to align the ring to 1024 B
+static_assert(4 * 32 * (kMaxN + 4) * 4 <= kStages * kStageBytes, "the epilogue's blocks fit the ring");
 // Polls of one mbarrier wait before it gives up (with 64 ns sleeps: a few
 // seconds). The pipeline's waits take their limit from the launch (this value
 // unless a caller asks for fewer); the clean-up after a timeout always waits
@@ -191,8 +192,14 @@ qmc_gemm_bf16_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     ok = __syncthreads_and(ok);
     asm volatile("tcgen05.fence::after_thread_sync;" ::);
     if (ok) {
-        // warp w owns TMEM lanes 32w..32w+31 = rows m0 + 32w + lane
-        const int row = m0 + warp * 32 + lane;
+        // warp w owns TMEM lanes 32w..32w+31 = rows m0 + 32w + lane. A lane holds
+        // a row's columns, so stores straight from it would touch 32 rows at a
+        // time (2048 x 256 x 256: they took most of the kernel's 22 us); the
+        // warp turns its 32 x N block through the ring, which every MMA has
+        // finished reading, and writes whole rows (10 us). Row stride N + 4
+        // floats: 16-byte stores of eight lanes cover all banks.
+        const int ldw = N + 4;
+        float *blk = reinterpret_cast<float *>(ring) + (size_t)warp * 32 * ldw;
         for (int c = 0; c < N; c += 16) {
             uint32_t r[16];
             const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c;
@@ -204,9 +211,21 @@ qmc_gemm_bf16_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant
                   "=r"(r[15])
                 : "r"(taddr));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            float *dst = Cs + (size_t)row * N + c;
 #pragma unroll
-            for (int q = 0; q < 16; ++q) dst[q] = __uint_as_float(r[q]);
+            for (int q = 0; q < 16; q += 4)
+                *reinterpret_cast<uint4 *>(blk + lane * ldw + c + q) = make_uint4(r[q], r[q + 1], r[q + 2], r[q + 3]);
+        }
+        __syncwarp();
+        float *dst = Cs + (size_t)(m0 + warp * 32) * N;
+        const bool vec = (reinterpret_cast<uintptr_t>(Cs) & 15) == 0;
+        for (int row = 0; row < 32; ++row) {
+            const float *src = blk + row * ldw;
+            if (vec) {
+                for (int c = 4 * lane; c < N; c += 128)
+                    *reinterpret_cast<float4 *>(dst + (size_t)row * N + c) = *reinterpret_cast<const float4 *>(src + c);
+            } else {
+                for (int c = lane; c < N; c += 32) dst[(size_t)row * N + c] = src[c];
+            }
         }
     } else {
         if (tid == 0) {
@@ -224,13 +243,25 @@ qmc_gemm_bf16_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kMaxN));
 }
 
+// sum over splits of W[s][i], in split order (the loads eight at a time)
+__device__ __forceinline__ float split_sum(const float *W, int splits, size_t stride, size_t i) {
+    float acc = W[i];
+    int s = 1;
+    for (; s + 8 <= splits; s += 8) {
+        float v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = W[(size_t)(s + q) * stride + i];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc += v[q];
+    }
+    for (; s < splits; ++s) acc += W[(size_t)s * stride + i];
+    return acc;
+}
+
 // C = sum over splits of W[s] (in split order)
 __global__ void qmc_gemm_splitk_sum(const float *W, int splits, size_t stride, float *C, size_t n) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        float acc = W[i];
-        for (int s = 1; s < splits; ++s) acc += W[(size_t)s * stride + i];
-        C[i] = acc;
-    }
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        C[i] = split_sum(W, splits, stride, i);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -278,29 +309,49 @@ SplitWorkspace &workspace() {
 
 }  // namespace
 
+namespace {
+// Splits of K when the M tiles leave most SMs idle: at most
+// gemm_splits_most (grows with K), each of `per` chunks, at least one
+int gemm_splits_most(int M, int K, int sms) {
+    return std::max(1, std::min((K + kBK - 1) / kBK, sms / (M / kTileM)));
+}
+int gemm_splits(int M, int K, int sms, int &per) {
+    const int nchunks = (K + kBK - 1) / kBK, splits = gemm_splits_most(M, K, sms);
+    per = (nchunks + splits - 1) / splits;
+    return (nchunks + per - 1) / per;
+}
+int gemm_sms() {
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+bool gemm_shape_ok(const void *A, const void *B, int M, int N, int K) {
+    if (M <= 0 || M % 128 || K <= 0 || K % 16 || N < 16 || N > 256 || N % 16) return false;
+    return ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0;
+}
+// The product's splits, split s at out + s M N
+int gemm_launch(const void *A, const void *B, float *out, int M, int N, int K, int splits, int per, unsigned *err_dev,
+                cudaStream_t stream, unsigned wait_limit) {
+    static const bool attr_set = cudaFuncSetAttribute(qmc_gemm_bf16_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      kGemmSmem) == cudaSuccess;
+    if (!attr_set) return -1;
+    CUtensorMap mapA, mapB;
+    if (!make_map(&mapA, A, M, K, kTileM) || !make_map(&mapB, B, N, K, N)) return -1;
+    qmc_gemm_bf16_tc<<<dim3(M / kTileM, splits), kGemmThreads, kGemmSmem, stream>>>(
+        mapA, mapB, out, N, K, per, (size_t)M * N, err_dev, wait_limit);
+    return 0;
+}
+}  // namespace
+
 // C[M][N] = A[M][K] B[N][K]^T, device pointers; M % 128 == 0, K % 16 == 0,
 // N % 16 == 0 and 16 <= N <= 256; A, B 16-byte aligned; C rows contiguous
 // (ldc = N). Split-K when the M tiles leave most SMs idle.
 extern "C" int qmc_k_gemm_bf16_limit(const void *A, const void *B, float *C, int M, int N, int K, unsigned *err_dev,
                                      void *stream, unsigned wait_limit) {
-    if (M <= 0 || M % 128 || K <= 0 || K % 16 || N < 16 || N > 256 || N % 16) return -2;
-    if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) return -2;
-    static bool attr_set = false;
-    if (!attr_set) {
-        if (cudaFuncSetAttribute(qmc_gemm_bf16_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem) !=
-            cudaSuccess)
-            return -1;
-        attr_set = true;
-    }
-    CUtensorMap mapA, mapB;
-    if (!make_map(&mapA, A, M, K, kTileM) || !make_map(&mapB, B, N, K, N)) return -1;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int mt = M / kTileM, nchunks = (K + kBK - 1) / kBK;
-    int splits = std::max(1, std::min(nchunks, sms / mt));
-    const int per = (nchunks + splits - 1) / splits;
-    splits = (nchunks + per - 1) / per;   // every split has at least one chunk
+    if (!gemm_shape_ok(A, B, M, N, K)) return -2;
+    int per = 1;
+    const int splits = gemm_splits(M, K, gemm_sms(), per);
     const size_t mn = (size_t)M * N;
     float *out = C;
     std::unique_lock<std::mutex> lock(workspace().mu, std::defer_lock);
@@ -317,9 +368,7 @@ extern "C" int qmc_k_gemm_bf16_limit(const void *A, const void *B, float *C, int
         }
         out = w.ptr;
     }
-    qmc_gemm_bf16_tc<<<dim3(mt, splits), kGemmThreads, kGemmSmem, (cudaStream_t)stream>>>(mapA, mapB, out, N, K,
-                                                                                           per, mn, err_dev,
-                                                                                           wait_limit);
+    if (gemm_launch(A, B, out, M, N, K, splits, per, err_dev, (cudaStream_t)stream, wait_limit)) return -1;
     if (splits > 1) {
         const unsigned blocks = (unsigned)std::min<size_t>((mn + 255) / 256, 4096);
         qmc_gemm_splitk_sum<<<blocks, 256, 0, (cudaStream_t)stream>>>(out, splits, mn, C, mn);
@@ -384,100 +433,162 @@ namespace {
 
 __device__ __forceinline__ __nv_bfloat16 bf(float x) { return __float2bfloat16_rn(x); }
 
+// The elementwise kernels below work on 32 x 32 tiles (blocks of 32 x 8
+// threads): the bf16 operands are wanted in both orders, and the transposed one
+// goes through shared memory so that both are written in whole segments (2-byte
+// stores one row apart filled a sixteenth of each sector). They read the GEMM's splits themselves, in split order, instead of a pass
+// that sums them first.
+struct Splits {
+    const float *W;
+    int n;
+    size_t stride;
+    __device__ __forceinline__ float at(size_t i) const { return split_sum(W, n, stride, i); }
+};
+constexpr int kTile = 32, kTileRows = 8;
+// f(b, o) -> value, stored bf16 as hb [Bp][N] and, through the tile, hbT [N][Bp]
+template <class F>
+__device__ __forceinline__ void tile_both(int Bp, int N, __nv_bfloat16 *hb, __nv_bfloat16 *hbT, F f) {
+    __shared__ __nv_bfloat16 tile[kTile][kTile + 2];
+    const int o = blockIdx.x * kTile + threadIdx.x, b0 = blockIdx.y * kTile;
+#pragma unroll
+    for (int r = 0; r < kTile; r += kTileRows) {
+        const int b = b0 + threadIdx.y + r;
+        if (b < Bp && o < N) {
+            const __nv_bfloat16 v = bf(f(b, o));
+            hb[(size_t)b * N + o] = v;
+            tile[threadIdx.y + r][threadIdx.x] = v;
+        }
+    }
+    __syncthreads();
+    const int bt = b0 + threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < kTile; r += kTileRows) {
+        const int ot = blockIdx.x * kTile + threadIdx.y + r;
+        if (bt < Bp && ot < N) hbT[(size_t)ot * Bp + bt] = tile[threadIdx.x][threadIdx.y + r];
+    }
+}
+
 // h0 = tanh(x W0^T + b0): f32 [Bp][H], bf16 [Bp][H] and [H][Bp]
 __global__ void mlp_layer0_fwd(const float *x, const float *W0, const float *b0, int nin, int H, int Bp,
                                float *h, __nv_bfloat16 *hb, __nv_bfloat16 *hbT) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Bp * H) return;
-    const int b = i / H, o = i % H;
-    float z = b0[o];
-    for (int k = 0; k < nin; ++k) z = fmaf(W0[o * nin + k], x[b * nin + k], z);
-    const float a = tanhf(z);
-    h[i] = a;
-    hb[i] = bf(a);
-    hbT[(size_t)o * Bp + b] = bf(a);
+    tile_both(Bp, H, hb, hbT, [=](int b, int o) {
+        float z = b0[o];
+        for (int k = 0; k < nin; ++k) z = fmaf(W0[o * nin + k], x[b * nin + k], z);
+        const float a = tanhf(z);
+        h[(size_t)b * H + o] = a;
+        return a;
+    });
 }
 
-// a = act(C + bias) for a GEMM output C [Bp][ldc] (columns < N used)
-__global__ void mlp_bias_act(const float *C, const float *bias, int N, int ldc, int Bp, int act, float *h,
-                             __nv_bfloat16 *hb, __nv_bfloat16 *hbT) {
+// h = tanh(C + bias) for a GEMM output C [Bp][N]
+__global__ void mlp_bias_tanh(Splits C, const float *bias, int N, int Bp, float *h, __nv_bfloat16 *hb,
+                              __nv_bfloat16 *hbT) {
+    tile_both(Bp, N, hb, hbT, [=](int b, int o) {
+        const size_t i = (size_t)b * N + o;
+        const float z = tanhf(C.at(i) + bias[o]);
+        h[i] = z;
+        return z;
+    });
+}
+
+// out = C + bias for a GEMM output C [Bp][ldc] (columns < N used)
+__global__ void mlp_bias_out(Splits C, const float *bias, int N, int ldc, int Bp, float *h) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= Bp * N) return;
     const int b = i / N, o = i % N;
-    float z = C[(size_t)b * ldc + o] + bias[o];
-    if (act) z = tanhf(z);
-    h[i] = z;
-    if (hb) hb[i] = bf(z);
-    if (hbT) hbT[(size_t)o * Bp + b] = bf(z);
+    h[i] = C.at((size_t)b * ldc + o) + bias[o];
 }
 
-// weighted squared error: loss += wt_o mask_b (out - y)^2 / B; dout = 2 wt_o mask_b (out - y) / B
+// weighted squared error: loss += wt_o mask_b (out - y)^2 / B; dout = 2 wt_o
+// mask_b (out - y) / B. One atomic per block (one per element, all on one
+// address, took 400 us for 2048 x 144).
 __global__ void mlp_loss(const float *out, const float *y, const float *wt, const float *mask, int No, int Nop,
                          int Bp, float invB, __nv_bfloat16 *dob, __nv_bfloat16 *dobT, float *dof, double *loss) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Bp * Nop) return;
-    const int b = i / Nop, o = i % Nop;
-    float g = 0.f;
-    if (o < No) {
-        const float r = out[(size_t)b * No + o] - y[(size_t)b * No + o];
-        const float w = wt[o] * mask[b];
-        g = 2.f * w * r * invB;
-        if (w != 0.f) atomicAdd(loss, (double)(w * r * r * invB));
+    __shared__ double part[kTileRows];
+    double mine = 0.0;
+    tile_both(Bp, Nop, dob, dobT, [=, &mine](int b, int o) {
+        float g = 0.f;
+        if (o < No) {
+            const float r = out[(size_t)b * No + o] - y[(size_t)b * No + o];
+            const float w = wt[o] * mask[b];
+            g = 2.f * w * r * invB;
+            if (w != 0.f) mine += (double)(w * r * r * invB);
+        }
+        dof[(size_t)b * Nop + o] = g;
+        return g;
+    });
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, off);
+    if (threadIdx.x == 0) part[threadIdx.y] = mine;
+    __syncthreads();
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        double v = 0.0;
+        for (int w = 0; w < kTileRows; ++w) v += part[w];
+        atomicAdd(loss, v);
     }
-    dob[i] = bf(g);
-    dobT[(size_t)o * Bp + b] = bf(g);
-    dof[i] = g;
 }
 
 // dz = dh (1 - h^2) for tanh layers: bf16 [Bp][H], bf16 [H][Bp], f32 [Bp][H]
-__global__ void mlp_tanh_bwd(const float *dh, const float *h, int H, int Bp, __nv_bfloat16 *dzb,
+__global__ void mlp_tanh_bwd(Splits dh, const float *h, int H, int Bp, __nv_bfloat16 *dzb,
                              __nv_bfloat16 *dzbT, float *dzf) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Bp * H) return;
-    const int b = i / H, o = i % H;
-    const float a = h[i];
-    const float g = dh[i] * (1.f - a * a);
-    dzb[i] = bf(g);
-    dzbT[(size_t)o * Bp + b] = bf(g);
-    dzf[i] = g;
+    tile_both(Bp, H, dzb, dzbT, [=](int b, int o) {
+        const size_t i = (size_t)b * H + o;
+        const float a = h[i];
+        const float g = dh.at(i) * (1.f - a * a);
+        dzf[i] = g;
+        return g;
+    });
 }
 
-// column sums: db[o] = sum_b dz[b][o]  (one block per column, fixed order)
-__global__ void mlp_colsum(const float *dz, int N, int ld, int Bp, float *db) {
-    const int o = blockIdx.x;
-    __shared__ float red[256];
-    float s = 0.f;
-    for (int b = threadIdx.x; b < Bp; b += blockDim.x) s += dz[(size_t)b * ld + o];
-    red[threadIdx.x] = s;
+// Column sums over the batch in a fixed order: column o's terms f(b, o) go to
+// 256 partial sums by b mod 256, added in b order, then pairwise by halves.
+// A block takes kCols neighbouring columns, so that a row's segment is read
+// whole, and 1024 threads, each with eight rows' loads in flight.
+constexpr int kCols = 8, kColThreads = 1024;
+// add(s, v, b) folds the loaded v of row b into s
+template <class A>
+__device__ __forceinline__ void column_sums(const float *dz, int N, int ld, int Bp, A add, float *out, int stride) {
+    __shared__ float red[256][kCols];
+    const int c = threadIdx.x % kCols, o = blockIdx.x * kCols + c;
+    for (int t = threadIdx.x / kCols; t < 256; t += kColThreads / kCols) {
+        float s = 0.f;
+        if (o < N)
+            for (int b = t; b < Bp; b += 8 * 256) {
+                float v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) v[q] = b + 256 * q < Bp ? dz[(size_t)(b + 256 * q) * ld + o] : 0.f;
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (b + 256 * q < Bp) s = add(s, v[q], b + 256 * q);
+            }
+        red[t][c] = s;
+    }
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+    for (int w = 128; w > 0; w >>= 1) {
+        for (int i = threadIdx.x; i < w * kCols; i += kColThreads)
+            red[i / kCols][i % kCols] += red[i / kCols + w][i % kCols];
         __syncthreads();
     }
-    if (threadIdx.x == 0) db[o] = red[0];
+    if (threadIdx.x < kCols && o < N) out[(size_t)o * stride] = red[0][c];
+}
+
+// db[o] = sum_b dz[b][o]
+__global__ void mlp_colsum(const float *dz, int N, int ld, int Bp, float *db) {
+    column_sums(dz, N, ld, Bp, [](float s, float v, int) { return s + v; }, db, 1);
 }
 
 // dW0[o][k] = sum_b dz0[b][o] x[b][k]
 __global__ void mlp_layer0_bwd(const float *dz, const float *x, int nin, int H, int Bp, float *dW0) {
-    const int o = blockIdx.x, k = blockIdx.y;
-    __shared__ float red[256];
-    float s = 0.f;
-    for (int b = threadIdx.x; b < Bp; b += blockDim.x) s = fmaf(dz[(size_t)b * H + o], x[b * nin + k], s);
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) dW0[o * nin + k] = red[0];
+    const int k = blockIdx.y;
+    column_sums(dz, H, H, Bp, [=](float s, float v, int b) { return fmaf(v, x[b * nin + k], s); }, dW0 + k, nin);
 }
 
 // copy a [H][Nop] GEMM result (dWout^T) into dWout [No][H]
-__global__ void mlp_untranspose(const float *src, int H, int Nop, int No, float *dst) {
+__global__ void mlp_untranspose(Splits src, int H, int Nop, int No, float *dst) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= No * H) return;
     const int o = i / H, k = i % H;
-    dst[i] = src[(size_t)k * Nop + o];
+    dst[i] = src.at((size_t)k * Nop + o);
 }
 
 // bf16 copies of a weight matrix W [R][C] (rows >= R of the padded copy are 0)
@@ -490,8 +601,17 @@ __global__ void mlp_weights_bf16(const float *W, int R, int Rp, int C, __nv_bflo
     WbT[(size_t)c * Rp + r] = bf(v);
 }
 
+// Where each layer's weight matrix [R][C] lies in the parameters and its bf16
+// copies (row count Rp of the padded ones); layer 0 has none
+struct BfCopies {
+    size_t off[17], end[17];
+    int C[17], Rp[17];
+    __nv_bfloat16 *Wb[17], *WbT[17];
+    int layers;
+};
+// Adam, and the updated weights' bf16 copies (one launch instead of one per layer)
 __global__ void mlp_adam(float *p, const float *g, float *m, float *v, size_t n, float lr, float b1, float b2,
-                         float eps, float c1, float c2) {
+                         float eps, float c1, float c2, const BfCopies L) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float gi = g[i];
@@ -499,7 +619,14 @@ __global__ void mlp_adam(float *p, const float *g, float *m, float *v, size_t n,
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float w = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    p[i] = w;
+    for (int l = 0; l < L.layers; ++l)
+        if (i >= L.off[l] && i < L.end[l]) {
+            const int k = (int)(i - L.off[l]), r = k / L.C[l], c = k - r * L.C[l];
+            L.Wb[l][k] = bf(w);
+            L.WbT[l][(size_t)c * L.Rp[l] + r] = bf(w);
+        }
 }
 
 inline unsigned nblk(size_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
@@ -521,7 +648,7 @@ struct qmc_mlp {
     float *params = nullptr, *grads = nullptr, *am = nullptr, *av = nullptr;
     std::vector<__nv_bfloat16 *> Wb, WbT;   // layers 1..D (index by layer)
     int Bcap = 0;
-    float *x = nullptr, *y = nullptr, *mask = nullptr, *C = nullptr, *tmp = nullptr;
+    float *x = nullptr, *y = nullptr, *mask = nullptr;
     std::vector<float *> hf;                 // [D] f32 activations
     std::vector<__nv_bfloat16 *> hb, hbT;    // [D]
     float *out = nullptr, *dof = nullptr, *dz = nullptr;
@@ -530,6 +657,9 @@ struct qmc_mlp {
     double *loss = nullptr;
     unsigned *err = nullptr;
     int t = 0;
+    float *ws = nullptr;                     // GEMM splits (this network's own; stream ordered)
+    size_t ws_cap = 0;
+    int sms = 0;
 };
 
 namespace {
@@ -538,8 +668,7 @@ int mlp_free_batch(qmc_mlp *m) {
     cudaFree(m->x);
     cudaFree(m->y);
     cudaFree(m->mask);
-    cudaFree(m->C);
-    cudaFree(m->tmp);
+    cudaFree(m->ws);
     cudaFree(m->out);
     cudaFree(m->dof);
     cudaFree(m->dz);
@@ -553,7 +682,8 @@ int mlp_free_batch(qmc_mlp *m) {
     m->hf.assign(m->D, nullptr);
     m->hb.assign(m->D, nullptr);
     m->hbT.assign(m->D, nullptr);
-    m->x = m->y = m->mask = m->C = m->tmp = m->out = m->dof = m->dz = nullptr;
+    m->x = m->y = m->mask = m->ws = m->out = m->dof = m->dz = nullptr;
+    m->ws_cap = 0;
     m->dob = m->dobT = m->dzb = m->dzbT = nullptr;
     m->Bcap = 0;
     return 0;
@@ -568,8 +698,15 @@ int mlp_ensure_batch(qmc_mlp *m, int Bp) {
     A((void **)&m->x, (size_t)Bp * m->nin * 4);
     A((void **)&m->y, (size_t)Bp * No * 4);
     A((void **)&m->mask, (size_t)Bp * 4);
-    A((void **)&m->C, (size_t)Bp * std::max(H, Nop) * 4);
-    A((void **)&m->tmp, (size_t)std::max(H * Nop, (size_t)Bp * H) * 4);
+    // the largest product's splits over the batch sizes up to Bp (splits fall
+    // as the rows grow: bounded by all SMs' tiles, or one split of Bp rows)
+    const size_t N = std::max(H, Nop);
+    size_t cap = 0;
+    for (int rows = kTileM; rows <= Bp; rows += kTileM)
+        cap = std::max(cap, (size_t)gemm_splits_most(rows, (int)N, m->sms) * rows * N);
+    cap = std::max(cap, (size_t)gemm_splits_most(m->H, Bp, m->sms) * H * N);
+    A((void **)&m->ws, cap * 4);
+    m->ws_cap = cap;
     A((void **)&m->out, (size_t)Bp * No * 4);
     A((void **)&m->dof, (size_t)Bp * Nop * 4);
     A((void **)&m->dz, (size_t)Bp * H * 4);
@@ -600,43 +737,60 @@ int mlp_sync_weights(qmc_mlp *m) {
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+// A [M][K] B [N][K]^T into the network's workspace, as splits
+int mlp_gemm(qmc_mlp *m, const void *A, const void *B, int M, int N, int K, Splits &out) {
+    if (!gemm_shape_ok(A, B, M, N, K)) return -1;
+    int per = 1;
+    const int splits = gemm_splits(M, K, m->sms, per);
+    if ((size_t)splits * M * N > m->ws_cap) return -1;
+    out = Splits{m->ws, splits, (size_t)M * N};
+    return gemm_launch(A, B, m->ws, M, N, K, splits, per, m->err, m->stream, kWaitLimit);
+}
+inline dim3 tiles(int N, int Bp) { return dim3((N + kTile - 1) / kTile, (Bp + kTile - 1) / kTile); }
+
 // forward for Bp rows already in m->x; output in m->out [Bp][No]
 int mlp_forward_dev(qmc_mlp *m, int Bp) {
     const int H = m->H;
-    mlp_layer0_fwd<<<nblk((size_t)Bp * H), 256, 0, m->stream>>>(m->x, m->params + m->offW[0], m->params + m->offb[0],
-                                                               m->nin, H, Bp, m->hf[0], m->hb[0], m->hbT[0]);
+    const dim3 tb(kTile, kTileRows);
+    Splits C;
+    mlp_layer0_fwd<<<tiles(H, Bp), tb, 0, m->stream>>>(m->x, m->params + m->offW[0], m->params + m->offb[0], m->nin, H,
+                                                       Bp, m->hf[0], m->hb[0], m->hbT[0]);
     for (int l = 1; l < m->D; ++l) {
-        if (qmc_k_gemm_bf16(m->hb[l - 1], m->Wb[l], m->C, Bp, H, H, m->err, m->stream)) return -1;
-        mlp_bias_act<<<nblk((size_t)Bp * H), 256, 0, m->stream>>>(m->C, m->params + m->offb[l], H, H, Bp, 1,
-                                                                 m->hf[l], m->hb[l], m->hbT[l]);
+        if (mlp_gemm(m, m->hb[l - 1], m->Wb[l], Bp, H, H, C)) return -1;
+        mlp_bias_tanh<<<tiles(H, Bp), tb, 0, m->stream>>>(C, m->params + m->offb[l], H, Bp, m->hf[l], m->hb[l],
+                                                          m->hbT[l]);
     }
-    if (qmc_k_gemm_bf16(m->hb[m->D - 1], m->Wb[m->D], m->C, Bp, m->Nop, H, m->err, m->stream)) return -1;
-    mlp_bias_act<<<nblk((size_t)Bp * m->No), 256, 0, m->stream>>>(m->C, m->params + m->offb[m->D], m->No, m->Nop,
-                                                                 Bp, 0, m->out, nullptr, nullptr);
+    if (mlp_gemm(m, m->hb[m->D - 1], m->Wb[m->D], Bp, m->Nop, H, C)) return -1;
+    mlp_bias_out<<<nblk((size_t)Bp * m->No), 256, 0, m->stream>>>(C, m->params + m->offb[m->D], m->No, m->Nop, Bp,
+                                                                 m->out);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 // loss (into *loss_dst) and gradients (into m->grads) for Bp rows with x, y, mask, wt in place
 int mlp_backward_dev(qmc_mlp *m, int Bp, int B, double *loss_dst) {
     const int H = m->H, D = m->D, Nop = m->Nop, No = m->No;
+    const dim3 tb(kTile, kTileRows);
+    Splits C;
     cudaMemsetAsync(loss_dst, 0, sizeof(double), m->stream);
-    mlp_loss<<<nblk((size_t)Bp * Nop), 256, 0, m->stream>>>(m->out, m->y, m->wt, m->mask, No, Nop, Bp, 1.f / B,
-                                                            m->dob, m->dobT, m->dof, loss_dst);
+    mlp_loss<<<tiles(Nop, Bp), tb, 0, m->stream>>>(m->out, m->y, m->wt, m->mask, No, Nop, Bp, 1.f / B, m->dob, m->dobT,
+                                                   m->dof, loss_dst);
     // output layer: dWout^T = h_{D-1}^T dout  ([H][Nop]), dbout, dh = dout Wout
-    if (qmc_k_gemm_bf16(m->hbT[D - 1], m->dobT, m->tmp, H, Nop, Bp, m->err, m->stream)) return -1;
-    mlp_untranspose<<<nblk((size_t)No * H), 256, 0, m->stream>>>(m->tmp, H, Nop, No, m->grads + m->offW[D]);
-    mlp_colsum<<<No, 256, 0, m->stream>>>(m->dof, No, Nop, Bp, m->grads + m->offb[D]);
-    if (qmc_k_gemm_bf16(m->dob, m->WbT[D], m->C, Bp, H, Nop, m->err, m->stream)) return -1;
+    if (mlp_gemm(m, m->hbT[D - 1], m->dobT, H, Nop, Bp, C)) return -1;
+    mlp_untranspose<<<nblk((size_t)No * H), 256, 0, m->stream>>>(C, H, Nop, No, m->grads + m->offW[D]);
+    mlp_colsum<<<(No + kCols - 1) / kCols, kColThreads, 0, m->stream>>>(m->dof, No, Nop, Bp, m->grads + m->offb[D]);
+    if (mlp_gemm(m, m->dob, m->WbT[D], Bp, H, Nop, C)) return -1;
     for (int l = D - 1; l >= 0; --l) {
-        mlp_tanh_bwd<<<nblk((size_t)Bp * H), 256, 0, m->stream>>>(m->C, m->hf[l], H, Bp, m->dzb, m->dzbT, m->dz);
-        mlp_colsum<<<H, 256, 0, m->stream>>>(m->dz, H, H, Bp, m->grads + m->offb[l]);
+        mlp_tanh_bwd<<<tiles(H, Bp), tb, 0, m->stream>>>(C, m->hf[l], H, Bp, m->dzb, m->dzbT, m->dz);
+        mlp_colsum<<<H / kCols, kColThreads, 0, m->stream>>>(m->dz, H, H, Bp, m->grads + m->offb[l]);
         if (l == 0) {
-            mlp_layer0_bwd<<<dim3(H, m->nin), 256, 0, m->stream>>>(m->dz, m->x, m->nin, H, Bp, m->grads + m->offW[0]);
+            mlp_layer0_bwd<<<dim3(H / kCols, m->nin), kColThreads, 0, m->stream>>>(m->dz, m->x, m->nin, H, Bp,
+                                                                           m->grads + m->offW[0]);
         } else {
             // dW_l = dz^T h_{l-1}  ([H][H]); dh_{l-1} = dz W_l
-            if (qmc_k_gemm_bf16(m->dzbT, m->hbT[l - 1], m->grads + m->offW[l], H, H, Bp, m->err, m->stream))
-                return -1;
-            if (qmc_k_gemm_bf16(m->dzb, m->WbT[l], m->C, Bp, H, H, m->err, m->stream)) return -1;
+            if (mlp_gemm(m, m->dzbT, m->hbT[l - 1], H, H, Bp, C)) return -1;
+            qmc_gemm_splitk_sum<<<nblk((size_t)H * H), 256, 0, m->stream>>>(C.W, C.n, C.stride, m->grads + m->offW[l],
+                                                                           C.stride);
+            if (mlp_gemm(m, m->dzb, m->WbT[l], Bp, H, H, C)) return -1;
         }
     }
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
@@ -680,6 +834,7 @@ int qmc_mlp_create(qmc_mlp **out, int device, int nin, int width, int depth, int
     if (cudaSetDevice(device) != cudaSuccess) return QMC_E_CUDA_LOCAL;
     qmc_mlp *m = new qmc_mlp();
     m->device = device;
+    cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, device);
     m->nin = nin;
     m->H = width;
     m->D = depth;
@@ -818,6 +973,17 @@ int qmc_mlp_train(qmc_mlp *m, const float *x, const float *y, const float *wt, i
     double *hist = nullptr;
     if (cudaMalloc(&hist, (size_t)std::max(steps, 1) * sizeof(double)) != cudaSuccess) return QMC_E_CUDA_LOCAL;
     int rc = 0;
+    BfCopies copies{};
+    copies.layers = m->D;
+    for (int l = 1; l <= m->D; ++l) {
+        const int R = l == m->D ? m->No : m->H;
+        copies.off[l - 1] = m->offW[l];
+        copies.end[l - 1] = m->offW[l] + (size_t)R * m->H;
+        copies.C[l - 1] = m->H;
+        copies.Rp[l - 1] = l == m->D ? m->Nop : m->H;
+        copies.Wb[l - 1] = m->Wb[l];
+        copies.WbT[l - 1] = m->WbT[l];
+    }
     for (int s = 0; s < steps && !rc; ++s) {
         if (mlp_forward_dev(m, Bp) || mlp_backward_dev(m, Bp, B, hist + s)) {
             rc = QMC_E_CUDA_LOCAL;
@@ -826,8 +992,8 @@ int qmc_mlp_train(qmc_mlp *m, const float *x, const float *y, const float *wt, i
         ++m->t;
         const float c1 = 1.f - std::pow(b1, (float)m->t), c2 = 1.f - std::pow(b2, (float)m->t);
         mlp_adam<<<nblk(m->nparams), 256, 0, m->stream>>>(m->params, m->grads, m->am, m->av, m->nparams, lr, b1,
-                                                           b2, eps, c1, c2);
-        if (mlp_sync_weights(m)) rc = QMC_E_CUDA_LOCAL;
+                                                           b2, eps, c1, c2, copies);
+        if (cudaGetLastError() != cudaSuccess) rc = QMC_E_CUDA_LOCAL;
     }
     if (!rc && losses && steps > 0) {
         std::vector<double> h(steps);
