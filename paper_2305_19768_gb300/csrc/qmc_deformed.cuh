@@ -35,8 +35,7 @@
 // pipe 87 % busy); massless box, 16 physical points at n = 4001, 5.9e8 (555)
 // -> 1.06e9 (453) with complex logarithms of the factors' product -> 1.86e9
 // (204, 78 %); the massive box in mixed precision, 256 points at n = 1009,
-// 2.85e9 -> 6.1e9. 24 warps per SM (85 registers) are as good as 16 for the
-// massless box and better for the others (6.7e9 -> 7.4e9; 5.4e9 -> 6.1e9).
+// 2.85e9 -> 6.6e9.
 // MIXED: derivatives of F and U(z), F(z) from FP32 monomial products in the
 // order of the general mixed kernel, everything after them in FP64.
 
@@ -53,6 +52,11 @@ struct alignas(16) FdShared {
     int32_t qmask;                   // bits 0..2: qc[7..9] present; 3..5: qc[4..6]
     int32_t d, ns, nU, nF, dbase, prow;
     int32_t dFoff[3], dFn[3], Hoff[QMC_NHESS], Hn[QMC_NHESS];
+    // MIXED: derivatives of F that are constants (F of degree <= 2 has only such
+    // second ones): dF by variable, d2F by slot pair (diagonal, then 01, 02, 12)
+    float gconst[3];
+    double hconst[6];
+    int32_t gvar, hvar;              // bits: those that are not
     int32_t perm[QMC_DMAX], slotof[QMC_DMAX], avar[QMC_DMAX], bvar[QMC_DMAX];
     double bd[QMC_DMAX], lam[QMC_DMAX];
     uint64_t lamm[QMC_DMAX];         // lambda as mantissa, exponent and sign
@@ -66,7 +70,7 @@ struct alignas(16) FdShared {
     QmcJobDev job;
     unsigned long long tile;
     int cached_sector, cached_point, job_index;
-    double red[8][8];
+    double red[16][8];
 };
 __device__ __forceinline__ FdShared &fd_shared() { return *reinterpret_cast<FdShared *>(qmc_fx_raw); }
 
@@ -176,6 +180,22 @@ struct FdOps {
     }
 };
 
+// The factors of a corner, out of line: inlined, their copies in every corner
+// of every path overflowed the instruction cache when sectors of several shapes
+// run side by side (the amplitude: 5 of 14 stall cycles per instruction).
+// B x^e or, for e < 0, B conj(x)^-e
+__device__ __noinline__ dc fd_mulpow(dc B, dc x, int e) {
+    const FdShared &S = fd_shared();
+    const FdOps o{S.mone, S.nzero, fd_signed(S.mone, true)};
+    return o.mul(B, o.pow(e < 0 ? conj_(x) : x, e < 0 ? -e : e));
+}
+// a n^e, 1 <= e <= 4
+__device__ __noinline__ FxM fd_mulnorm(FxM a, FxM n, int e) { return fx_norm(fx_mul(a, fx_pow(n, n, e))); }
+// re^2 + im^2
+__device__ __noinline__ FxM fd_norm2(double re, double im) {
+    return fd_of(fma(re, re, fma(im, im, fd_shared().nzero)));
+}
+
 // MIXED: the thread's FP32 power tables (real rows, then complex rows, prow
 // per variable) and the sums over them, products and sums in the order of the
 // general mixed kernel; out of line, one copy for every polynomial and corner
@@ -252,7 +272,7 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
     double Ad[D], Ao[3];                                // d2F: diagonal (MIXED), off-diagonal (01, 02, 12)
     dc F, U{1.0, 0.0};
     const bool needU = S.u0 != 0 || (lam && S.u1 != 0);
-    const int qm = MIXED ? 63 : S.qmask;
+    const int qm = S.qmask;
     if constexpr (!MIXED) {
 #pragma unroll
         for (int j = 0; j < D; ++j) {
@@ -274,23 +294,12 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
         // FP32 derivatives, original variable order
 #pragma unroll
         for (int j = 0; j < D; ++j) fd_put<BLOCK>(j, prow, (V >> S.slotof[j] & 1) ? 0.0f : P.tf[j]);
-        float gf[3], Hf[3][3];
+        float gf[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            gf[j] = 0.0f;
-            if (j < D) gf[j] = fd_poly<BLOCK>(S.dbase + S.dFoff[j], S.dFn[j]);
+        for (int j = 0; j < D; ++j) {
+            gf[j] = S.gconst[j];
+            if (S.gvar >> j & 1) gf[j] = fd_poly<BLOCK>(S.dbase + S.dFoff[j], S.dFn[j]);
         }
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-#pragma unroll
-            for (int k = j; k < 3; ++k) {
-                Hf[j][k] = 0.0f;
-                if (k < D) {
-                    const int h = j * QMC_DMAX - j * (j - 1) / 2 + (k - j);
-                    Hf[j][k] = fd_poly<BLOCK>(S.dbase + S.Hoff[h], S.Hn[h]);
-                }
-                Hf[k][j] = Hf[j][k];
-            }
         // to slot order
 #pragma unroll
         for (int i = 0; i < D; ++i) {
@@ -299,15 +308,15 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
 #pragma unroll
             for (int k = i; k < D; ++k) {
                 if ((V >> i & 1) || (V >> k & 1)) continue;
-                const int pk = S.perm[k];
-                float h = 0.0f;
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-#pragma unroll
-                    for (int b = 0; b < 3; ++b)
-                        if (pi == a && pk == b) h = Hf[a][b];
-                if (i == k) Ad[i] = fd_to_double(h);
-                else Ao[i + k - 1] = fd_to_double(h);
+                const int at = i == k ? i : 2 + i + k;
+                double h = S.hconst[at];
+                if (S.hvar >> at & 1) {
+                    const int a = min(pi, S.perm[k]), b = max(pi, S.perm[k]);
+                    const int q = a * QMC_DMAX - a * (a - 1) / 2 + (b - a);
+                    h = fd_to_double(fd_poly<BLOCK>(S.dbase + S.Hoff[q], S.Hn[q]));
+                }
+                if (i == k) Ad[i] = h;
+                else Ao[i + k - 1] = h;
             }
         }
     }
@@ -443,14 +452,12 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
     int64_t arg = 0;
     auto factor = [&](dc x, FxM n, int e0, int e1, bool m0) {
         if (e0) {
-            const int a = e0 < 0 ? -e0 : e0;
-            B = o.mul(B, o.pow(e0 < 0 ? conj_(x) : x, a));
-            if (e0 < 0) den = fx_norm(fx_mul(den, fx_pow(n, n, a)));
+            B = fd_mulpow(B, x, e0);
+            if (e0 < 0) den = fd_mulnorm(den, n, -e0);
         }
         if (lam && e1) {
-            const int a = e1 < 0 ? -e1 : e1;
-            if (e1 > 0) np = fx_norm(fx_mul(np, fx_pow(n, n, a)));
-            else nn = fx_norm(fx_mul(nn, fx_pow(n, n, a)));
+            if (e1 > 0) np = fd_mulnorm(np, n, e1);
+            else nn = fd_mulnorm(nn, n, -e1);
             arg += (int64_t)e1 * (fd_arg(x.im, x.re, m0) >> 3);
         }
     };
@@ -463,16 +470,16 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
             const FxM n = fd_of(fma(gl, gl, o.one));
             if (!(V >> j & 1)) {
                 B = dc{fma(-gl, B.im, B.re), fma(gl, B.re, B.im)};
-                den = fx_norm(fx_mul(den, n));
+                den = fd_mulnorm(den, n, 1);
             }
             factor(dc{1.0, -gl}, n, 0, S.bvar[j], false);
         } else if (S.regular >> j & 1) {
             const dc z{P.t[j], -y[j]};
-            factor(z, fd_of(fma(z.re, z.re, o.mul(z.im, z.im))), S.avar[j], S.bvar[j], false);
+            factor(z, fd_norm2(z.re, z.im), S.avar[j], S.bvar[j], false);
         }
     }
-    if (needU) factor(U, fd_of(fma(U.re, U.re, o.mul(U.im, U.im))), S.u0, S.u1, false);
-    factor(F, fd_of(fma(F.re, F.re, o.mul(F.im, F.im))), S.f0, S.f1, true);
+    if (needU) factor(U, fd_norm2(U.re, U.im), S.u0, S.u1, false);
+    factor(F, fd_norm2(F.re, F.im), S.f0, S.f1, true);
     out.B = B;
     out.q = fd_rcp(den);
     out.L = dc{0.0, 0.0};
@@ -555,7 +562,7 @@ __device__ __forceinline__ void fd_points(const QmcLaunch &Lc, uint64_t k0, uint
         double hb[NSA], bl[NSA];
         bool zero = false;
         P.tf[0] = P.tf[1] = P.tf[2] = 1.0f;
-#pragma unroll
+#pragma unroll 1
         for (int i = 0; i < D; ++i) {
             const FxCoord u = fx_next(walk[i * BLOCK], S.zmod[i], S.qz[i], S.rz[i], n32, S.job.inv_n, S.delta[i],
                                       S.dfix[i], walk + i * BLOCK);
@@ -602,10 +609,7 @@ __device__ __forceinline__ void fd_points(const QmcLaunch &Lc, uint64_t k0, uint
             if (c.m) P.k[i] = fd_signed(fx_pack(fx_norm(fx_mul(c, fd_rcp(tv)))), cneg);
             if constexpr (MIXED) {
                 const float f = fd_to_float(td);
-                const int pj = S.perm[i];
-                if (pj == 0) P.tf[0] = f;
-                else if (pj == 1) P.tf[1] = f;
-                else P.tf[2] = f;
+                P.tf[S.perm[i]] = f;
             }
             if (i < NS && u.y.m) {
                 const qmc_xf r = qmc_xf_rcp3(qmc_xf{t.m, t.e, 0});
@@ -656,7 +660,7 @@ __device__ __forceinline__ void fd_stage(FdShared &S, const QmcLaunch &Lc) {
     const int nm = MIXED ? src->nmono : nU + nF;
     if (threadIdx.x < 10) S.qc[threadIdx.x] = 0.0;
     if (threadIdx.x >= 10 && threadIdx.x < 13) S.qa[threadIdx.x - 10] = 0.0;
-    if (threadIdx.x == 13) S.qmask = 0;
+    if (threadIdx.x == 13) S.qmask = S.gvar = S.hvar = 0;
     int slot[3], next = ns;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -750,16 +754,47 @@ __device__ __forceinline__ void fd_stage(FdShared &S, const QmcLaunch &Lc) {
         S.cached_point = pidx;
     }
     __syncthreads();
+    if constexpr (MIXED) {
+        // the constant derivatives (no monomial, or the constant one alone)
+        if (threadIdx.x < 9) {
+            const int i = threadIdx.x;
+            int m0 = 0, n = 0;
+            if (i < 3) {
+                if (i < d) {
+                    m0 = S.dFoff[i];
+                    n = S.dFn[i];
+                }
+            } else {
+                const int x = i < 6 ? i - 3 : (i == 8 ? 1 : 0), z = i < 6 ? x : (i == 6 ? 1 : 2);   // slots
+                if (z < d) {
+                    const int a = min(S.perm[x], S.perm[z]), b = max(S.perm[x], S.perm[z]);
+                    const int q = a * QMC_DMAX - a * (a - 1) / 2 + (b - a);
+                    m0 = S.Hoff[q];
+                    n = S.Hn[q];
+                }
+            }
+            const bool constant = n == 0 || (n == 1 && S.mdesc[S.dbase + m0].w == 0);
+            const float v = n == 0 || !constant ? 0.0f : S.cvalf[S.dbase + m0];
+            if (i < 3) {
+                S.gconst[i] = v;
+                if (!constant) atomicOr(&S.gvar, 1 << i);
+            } else {
+                S.hconst[i - 3] = (double)v;
+                if (!constant) atomicOr(&S.hvar, 1 << (i - 3));
+                // the coupling (slots 01, 02, 12) enters the minors
+                if (i >= 6 && !(constant && v == 0.0f)) atomicOr(&S.qmask, 1 << (i - 6));
+            }
+        }
+    }
 }
 
-#ifndef QMC_FD_MINB
-#define QMC_FD_MINB 6
-#endif
-#ifndef QMC_FDM_MINB
-#define QMC_FDM_MINB 6
-#endif
+// Resident 128-thread units the registers must allow. Measured at 4 and 6: FP64
+// massive box 7.3e9 and 7.7e9 evaluations/s, massless box 1.86e9 and 1.72e9;
+// mixed massive box 5.9e9 and 6.6e9; the mixed amplitude (sums to eps^1)
+// 36.6 and 38.9 ms.
+template <bool MIXED, int HI> constexpr int fd_min_units() { return MIXED && HI == 0 ? 6 : 4; }
 template <bool MIXED, int BLOCK, int HI>
-__global__ void __launch_bounds__(BLOCK, (MIXED ? QMC_FDM_MINB : QMC_FD_MINB) * 128 / BLOCK) qmc_deformed_kernel(QmcLaunch Lc, int ppt) {
+__global__ void __launch_bounds__(BLOCK, fd_min_units<MIXED, HI>() * 128 / BLOCK) qmc_deformed_kernel(QmcLaunch Lc, int ppt) {
     constexpr int LMAX = 4;
     FdShared &S = fd_shared();
     const int lo = Lc.lo, nord = Lc.norders;
@@ -853,22 +888,14 @@ __global__ void __launch_bounds__(BLOCK, (MIXED ? QMC_FDM_MINB : QMC_FD_MINB) * 
                 if (Lc.job_fail) atomicAdd(Lc.job_fail + S.job_index, v);
             }
         }
-        // block reduction: warp shuffles, then warps in index order
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        // block reduction: warp sums, then warps in index order
+        double flat[2 * LMAX];
 #pragma unroll
         for (int q = 0; q < LMAX; ++q) {
-            if (q >= nord) continue;
-            double vr = acc[q].re, vi = acc[q].im;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                vr += __shfl_down_sync(0xffffffffu, vr, off);
-                vi += __shfl_down_sync(0xffffffffu, vi, off);
-            }
-            if (lane == 0) {
-                S.red[warp][2 * q] = vr;
-                S.red[warp][2 * q + 1] = vi;
-            }
+            flat[2 * q] = acc[q].re;
+            flat[2 * q + 1] = acc[q].im;
         }
+        fx_block_sums(flat, 2 * nord, S.red);
         __syncthreads();
         if (threadIdx.x < 2 * nord) {
             double sum = 0.0;

@@ -14,6 +14,7 @@
 #include <memory>
 #include <sstream>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "qmc_ctx.h"
@@ -739,14 +740,16 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         if (v.empty()) continue;
         // the tile queue hands out tiles in job order: costly jobs first (more
         // singular variables, larger lattices) shortens the tail of the launch,
-        // and jobs of one sector shape run side by side on the SMs
+        // and jobs of one sector shape, then of one sector, run side by side on
+        // the SMs (point by point instead, an amplitude's shapes alternate and
+        // overflow the instruction cache)
         {
             std::vector<int> ord(v.size());
             for (size_t u = 0; u < ord.size(); ++u) ord[u] = (int)u;
             auto key = [&](int u) {
                 const qmc_job &J = jobs[per_orig[slot][u]];
-                const int ns = ctx->integrals[J.integral_id].sectors[J.sector].ns;
-                return std::make_pair(ns, (double)v[u].n * v[u].shifts);
+                const HostSector &S = ctx->integrals[J.integral_id].sectors[J.sector];
+                return std::make_tuple(S.ns, (double)v[u].n * v[u].shifts, S.d, S.global_index);
             };
             std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return key(a) > key(b); });
             std::vector<QmcJobDev> v2;

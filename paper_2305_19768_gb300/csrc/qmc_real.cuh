@@ -97,6 +97,47 @@ template <int DMAX, int BLOCK> __device__ __forceinline__ unsigned char *fx_pt(i
     return qmc_fx_raw + sizeof(FxShared) + 16 * DMAX * BLOCK + esize * threadIdx.x;
 }
 
+// Warp sums of N values per lane (N a power of two, <= 8): while more than one
+// is left, the lanes of each pair keep half of them and hand over the others,
+// so that eight values take 9 additions instead of 40 (an FP64 addition holds
+// its pipe for 76 cycles; at four points a thread the 40 were a twelfth of the
+// deformed kernel's FP64 work). The same pairs as a shuffle-down tree per
+// value, so the same bits. Lane l returns the sum of value l / (32 / N).
+template <int N> __device__ __forceinline__ double fx_warp_sum(double (&v)[N]) {
+    const int lane = threadIdx.x & 31;
+    int off = 16;
+#pragma unroll
+    for (int h = N / 2; h >= 1; h /= 2, off /= 2) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const double give = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+        }
+    }
+#pragma unroll
+    for (int o = 16 / N; o >= 1; o /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
+}
+// The block's warps write the sums of values [0, count) to red[warp][]
+template <int LMAX, int W>
+__device__ __forceinline__ void fx_block_sums(const double (&acc)[LMAX], int count, double (&red)[16][W]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto sum = [&](auto tag) {
+        constexpr int N = decltype(tag)::value;
+        double v[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = i < LMAX ? acc[i < LMAX ? i : 0] : 0.0;
+        const double s = fx_warp_sum<N>(v);
+        const int q = lane / (32 / N);
+        if (lane % (32 / N) == 0 && q < count) red[warp][q] = s;
+    };
+    if (count <= 1) sum(std::integral_constant<int, 1>{});
+    else if (count <= 2) sum(std::integral_constant<int, 2>{});
+    else if (count <= 4) sum(std::integral_constant<int, 4>{});
+    else sum(std::integral_constant<int, 8>{});
+}
+
 // x / n and x mod n for n < 2^32 with minv = floor((2^64 - 1) / n): the
 // quotient estimate is at most 2 short
 __device__ __forceinline__ uint64_t fx_divmod(uint64_t x, uint64_t n, uint64_t minv, uint64_t &r) {
@@ -917,16 +958,8 @@ __global__ void __launch_bounds__(BLOCK, (DMAX > 3 ? QMC_FX6_MINB : QMC_FX_MINB)
                 else fx_points<DMAX, BLOCK, 4, HI, MIXED, LMAX>(Lc, k0, kend, lo, nord, acc);
             }
         }
-        // block reduction: warp shuffles, then warps in index order
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-        for (int o = 0; o < LMAX; ++o) {
-            if (o >= nord) continue;
-            double v = acc[o];
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-            if (lane == 0) S.red[warp][o] = v;
-        }
+        // block reduction: warp sums, then warps in index order
+        fx_block_sums(acc, nord, S.red);
         __syncthreads();
         if (threadIdx.x < 2 * nord) {
             double sum = 0.0;
