@@ -90,9 +90,6 @@ struct qmc_ctx {
 struct ClassLaunch {
     int cls = 0;
     QmcLaunch L{};
-    QmcJobDev *d_jobs = nullptr;
-    double *d_partials = nullptr;
-    unsigned long long *d_queue = nullptr;
     unsigned int *d_jobfail = nullptr;   // per-job sign-check failures
     std::vector<int> orig;               // caller's index of each class-local job
     int block = 128, ppt = 16, grid = 0;
@@ -112,6 +109,9 @@ struct qmc_plan {
     double evals = 0.0;                  // lattice points x shifts of one run
     size_t out_size = 0;
     double *d_out = nullptr;
+    unsigned char *d_arena = nullptr;   // the plan's one device allocation; the pointers below and in the launches lie in it
+    unsigned char *d_zero = nullptr;
+    size_t zero_bytes = 0;              // from d_zero, cleared before each run: tile queues, failure counts, status
     unsigned long long *d_status = nullptr;
     std::vector<ClassLaunch> launches;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;

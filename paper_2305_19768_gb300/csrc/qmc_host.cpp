@@ -456,18 +456,14 @@ bool fd_job_ok(const HostSector &S, int cls) {
     return true;
 }
 
+constexpr size_t kStatusBytes = 2 * sizeof(unsigned long long);   // sign failures, non-finite tiles
+constexpr size_t kOneCopy = 4096;   // results up to this many numbers come back with the status (32 KB on the stack)
+
 void free_plan_buffers(qmc_plan *p) {
-    for (ClassLaunch &c : p->launches) {
-        cudaFree(c.d_jobs);
-        cudaFree(c.d_partials);
-        cudaFree(c.d_queue);
-        cudaFree(c.d_jobfail);
-    }
     if (p->gexec) cudaGraphExecDestroy(p->gexec);
     p->gexec = nullptr;
     p->launches.clear();
-    cudaFree(p->d_out);
-    cudaFree(p->d_status);
+    cudaFree(p->d_arena);
     if (p->ev0) cudaEventDestroy(p->ev0);
     if (p->ev1) cudaEventDestroy(p->ev1);
     for (cudaEvent_t e : p->kev) cudaEventDestroy(e);
@@ -478,6 +474,7 @@ void free_plan_buffers(qmc_plan *p) {
     p->join.clear();
     if (p->fork) cudaEventDestroy(p->fork);
     p->fork = nullptr;
+    p->d_arena = nullptr;
     p->d_out = nullptr;
     p->d_status = nullptr;
 }
@@ -729,9 +726,6 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         if (e_ != cudaSuccess)                                                                  \
             return bail(fail(ctx, QMC_E_CUDA, "%s: %s", #call, cudaGetErrorString(e_)));        \
     } while (0)
-    PLAN_TRY(cudaMalloc(&p->d_out, std::max<size_t>(1, p->out_size) * sizeof(double)));
-    PLAN_TRY(cudaMalloc(&p->d_status, 2 * sizeof(unsigned long long)));
-    PLAN_TRY(cudaMemset(p->d_status, 0, 2 * sizeof(unsigned long long)));
     PLAN_TRY(cudaEventCreate(&p->ev0));
     PLAN_TRY(cudaEventCreate(&p->ev1));
     for (int slot = 0; slot < 2 * QMC_NCLASS; ++slot) {
@@ -799,19 +793,11 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
             D.tile_begin = tiles;
             tiles += (uint64_t)D.tiles_per_shift * D.shifts;
         }
-        PLAN_TRY(cudaMalloc(&c.d_jobs, v.size() * sizeof(QmcJobDev)));
-        PLAN_TRY(cudaMemcpy(c.d_jobs, v.data(), v.size() * sizeof(QmcJobDev), cudaMemcpyHostToDevice));
-        PLAN_TRY(cudaMalloc(&c.d_partials, std::max<uint64_t>(1, tiles) * 2 * norders * sizeof(double)));
-        PLAN_TRY(cudaMalloc(&c.d_queue, sizeof(unsigned long long)));
-        PLAN_TRY(cudaMemset(c.d_queue, 0, sizeof(unsigned long long)));
-        PLAN_TRY(cudaMalloc(&c.d_jobfail, v.size() * sizeof(unsigned int)));
-        PLAN_TRY(cudaMemset(c.d_jobfail, 0, v.size() * sizeof(unsigned int)));
         c.grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(tiles, (uint64_t)ctx->sm_count * occ));
         QmcLaunch &L = c.L;
         L.sectors = ctx->d_sectors;
         L.monos = ctx->d_monos;
         L.kin = ctx->d_kin;
-        L.jobs = c.d_jobs;
         L.njobs = (int)v.size();
         L.ninv = ctx->ninv;
         L.lo = lo;
@@ -822,12 +808,52 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         L.prow = prow;
         L.mone = -1.0;
         L.nzero = -0.0;
-        L.partials = c.d_partials;
-        L.queue = c.d_queue;
-        L.status = p->d_status;
-        L.out = p->d_out;
-        L.job_fail = c.d_jobfail;
         p->launches.push_back(c);
+    }
+    // One allocation and one copy for everything a plan holds on the device
+    // (six, and a copy or a fill each, took 32 us of a one-shot call's 90 for a
+    // plan's set-up and release; with this the call takes 70). In order:
+    //   [jobs]  [queues, failure counts, status | results]  [partial sums]
+    // so that one fill clears what a run must find at zero and a small plan's
+    // status and results come back in one copy.
+    {
+        auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+        size_t zero = 0, njob_bytes = 0, part = 0;
+        std::vector<size_t> at_queue, at_jobs, at_part;
+        for (const ClassLaunch &c : p->launches) {
+            at_queue.push_back(zero);
+            zero += 16 + (c.orig.size() * sizeof(unsigned int) + 15) / 16 * 16;
+            at_jobs.push_back(njob_bytes);
+            njob_bytes += up(c.orig.size() * sizeof(QmcJobDev));
+            at_part.push_back(part);
+            part += up(std::max<uint64_t>(1, c.L.ntiles) * 2 * norders * sizeof(double));
+        }
+        zero = up(zero + kStatusBytes);   // the status ends the cleared part
+        const size_t part_at = up(njob_bytes + zero + std::max<size_t>(1, p->out_size) * sizeof(double));
+        PLAN_TRY(cudaMalloc(&p->d_arena, part_at + part));
+        p->d_zero = p->d_arena + njob_bytes;
+        p->zero_bytes = zero;
+        p->d_status = (unsigned long long *)(p->d_zero + zero - kStatusBytes);
+        p->d_out = (double *)(p->d_zero + zero);
+        std::vector<unsigned char> head(njob_bytes + zero, 0);
+        size_t k = 0;
+        for (int slot = 0; slot < 2 * QMC_NCLASS; ++slot) {
+            if (per[slot].empty()) continue;
+            ClassLaunch &c = p->launches[k];
+            memcpy(head.data() + at_jobs[k], per[slot].data(), per[slot].size() * sizeof(QmcJobDev));
+            c.d_jobfail = (unsigned int *)(p->d_zero + at_queue[k] + 16);
+            c.L.queue = (unsigned long long *)(p->d_zero + at_queue[k]);
+            c.L.jobs = (const QmcJobDev *)(p->d_arena + at_jobs[k]);
+            c.L.partials = (double *)(p->d_arena + part_at + at_part[k]);
+            c.L.status = p->d_status;
+            c.L.out = p->d_out;
+            c.L.job_fail = c.d_jobfail;
+            ++k;
+        }
+        PLAN_TRY(cudaMemcpy(p->d_arena, head.data(), head.size(), cudaMemcpyHostToDevice));
+        // a copy from pageable memory may return before its last transfer is
+        // done, and a run may be on any stream
+        PLAN_TRY(cudaStreamSynchronize(cudaStreamLegacy));
     }
     // the largest class first: it sets the length of the run, the others fill its tail
     std::stable_sort(p->launches.begin(), p->launches.end(), [](const ClassLaunch &a, const ClassLaunch &b) {
@@ -867,7 +893,7 @@ namespace {
 int plan_enqueue(qmc_plan *plan, double *out, cudaStream_t st, bool capturing) {
     qmc_ctx *ctx = plan->ctx;
     const unsigned evflags = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
-    CUDA_TRY(ctx, cudaMemsetAsync(plan->d_status, 0, 2 * sizeof(unsigned long long), st));
+    CUDA_TRY(ctx, cudaMemsetAsync(plan->d_zero, 0, plan->zero_bytes, st));   // queues, failure counts, status
     CUDA_TRY(ctx, cudaEventRecordWithFlags(plan->ev0, st, evflags));
     if (plan->fork) CUDA_TRY(ctx, cudaEventRecord(plan->fork, st));
     int launches = 0;
@@ -877,7 +903,6 @@ int plan_enqueue(qmc_plan *plan, double *out, cudaStream_t st, bool capturing) {
         if (i > 0) CUDA_TRY(ctx, cudaStreamWaitEvent(cs, plan->fork, 0));
         c.L.out = out;
         c.L.kin = ctx->d_kin;
-        CUDA_TRY(ctx, cudaMemsetAsync(c.d_jobfail, 0, c.orig.size() * sizeof(unsigned int), cs));
         CUDA_TRY(ctx, cudaEventRecordWithFlags(plan->kev[2 * i], cs, evflags));
         if (c.L.ntiles > 0) {
             const bool fx = c.fx && !c.general;
@@ -984,11 +1009,24 @@ int qmc_plan_results(qmc_plan *plan, double *out, uint64_t *sign_failures) {
     cudaSetDevice(ctx->device);
     cudaStream_t st = plan->last_stream ? plan->last_stream : ctx->stream;
     unsigned long long status[2] = {0, 0};
-    if (out && plan->out_size)
-        CUDA_TRY(ctx, cudaMemcpyAsync(out, plan->last_out ? plan->last_out : plan->d_out,
-                                      plan->out_size * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(ctx, cudaMemcpyAsync(status, plan->d_status, sizeof status, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(ctx, cudaStreamSynchronize(st));
+    const double *src = plan->last_out ? plan->last_out : plan->d_out;
+    if (out && plan->out_size && src == plan->d_out && plan->out_size <= kOneCopy) {
+        // the status lies directly before the results: one copy of both. Larger
+        // results go straight to the caller's memory: the second pass over
+        // them would cost more than a copy's few microseconds.
+        static_assert(sizeof status == kStatusBytes, "status words and results are copied together");
+        double both[2 + kOneCopy];
+        CUDA_TRY(ctx, cudaMemcpyAsync(both, plan->d_status, (2 + plan->out_size) * sizeof(double),
+                                      cudaMemcpyDeviceToHost, st));
+        CUDA_TRY(ctx, cudaStreamSynchronize(st));
+        memcpy(status, both, sizeof status);
+        memcpy(out, both + 2, plan->out_size * sizeof(double));
+    } else {
+        if (out && plan->out_size)
+            CUDA_TRY(ctx, cudaMemcpyAsync(out, src, plan->out_size * sizeof(double), cudaMemcpyDeviceToHost, st));
+        CUDA_TRY(ctx, cudaMemcpyAsync(status, plan->d_status, sizeof status, cudaMemcpyDeviceToHost, st));
+        CUDA_TRY(ctx, cudaStreamSynchronize(st));
+    }
     if (sign_failures) *sign_failures = status[0];
     if (status[1]) return fail(ctx, QMC_E_NONFINITE, "%llu tile partial sums were not finite", status[1]);
     if (status[0]) return fail(ctx, QMC_E_SIGN_CHECK, "%llu deformed points had Im F > 0", status[0]);
