@@ -114,12 +114,27 @@ QMC_HD qmc_xf qmc_xf_rcp(qmc_xf a) {
     // y0 in (1, 2]: Q62 from its bits (2.0 clamps just below 2^63)
     int64_t Y = ((yb >> 23) & 0xFF) >= 128 ? (int64_t)0x7FFFFFFFFFFFFFFFLL
                                            : (int64_t)((1ULL << 62) | ((uint64_t)(yb & 0x7FFFFFu) << 39));
-    for (int it = 0; it < 2; ++it) {
-        const int64_t P = (int64_t)qmc_umulhi64(a.m, (uint64_t)Y);    // m y 2^62
-        const int64_t E = (int64_t)(1ULL << 62) - P;                 // (1 - m y) 2^62
-        Y += qmc_smulhi(Y, E) << 2;
-        if (Y < 0) Y = 0x7FFFFFFFFFFFFFFFLL;            // (never: y < 2)
+    // y <- y + y e, e = 1 - m y, twice. The first y has 24 bits and the second
+    // e (of Q62) 32, so of the four 64 x 64 products only one is left whole; the
+    // others are the same numbers from 32 x 32 ones.
+    int64_t P, E;
+    if (yb < 0x40000000u) {
+        const uint32_t Y0 = (yb & 0x7FFFFFu) | (1u << 23);                        // y in Q23
+        const uint64_t p0 = (uint64_t)(uint32_t)a.m * Y0;
+        P = (int64_t)(((uint64_t)(uint32_t)(a.m >> 32) * Y0 + (p0 >> 32)) << 7 | ((uint32_t)p0 >> 25));   // m y 2^62
+        E = (int64_t)(1ULL << 62) - P;                                            // e 2^62, |e| < 2^-20
+        Y += (((int64_t)((uint64_t)((int64_t)(int32_t)(E >> 32) * (int64_t)Y0) << 7)) +
+              (int64_t)(((uint64_t)(uint32_t)E * Y0) >> 25)) * 4;
+    } else {
+        P = (int64_t)qmc_umulhi64(a.m, (uint64_t)Y);
+        E = (int64_t)(1ULL << 62) - P;
+        Y += qmc_smulhi(Y, E) * 4;
     }
+    P = (int64_t)qmc_umulhi64(a.m, (uint64_t)Y);
+    const int32_t e2 = (int32_t)((int64_t)(1ULL << 62) - P);                       // |e| < 2^-40
+    const uint32_t yl = (uint32_t)Y;
+    const int64_t lo = (int64_t)(((uint64_t)yl * (uint32_t)e2) >> 32) - (e2 < 0 ? (int64_t)yl : 0);
+    Y += (((int64_t)(int32_t)(Y >> 32) * e2 + lo) >> 32) * 4;
     // 1/|a| = y 2^(-a.e - 1) with y = Y 2^-62 in (1, 2)
     r.m = (uint64_t)Y << 1;
     r.e = -a.e - 1;
