@@ -1635,6 +1635,263 @@ __device__ __noinline__ void eval_real_taylor(const TileSmem<LMAX> &S, const dou
     }
 }
 
+// The same for the common case: sums up to eps^0, one or two singular
+// variables, every p_q 1 or 2 (R: the slots with p_q = 2). Everything has a
+// compile-time extent, so series, jets and the Taylor coefficients stay in
+// registers, and no term is formed that cannot reach eps^0 or is zero by
+// structure: base(V) has the orders 0..|V|, the sums over kappa -|V|..0, the
+// jets 1, 2 or 4 coefficients whose logarithm and exponential are written
+// out. What is left is rounded as above, step by step (products that the loops
+// store are not contracted into the sums that follow), so the results are the
+// same bits. FP64-bound; the loops carry full series at run-time extents in
+// local memory. The one-loop box in D = 2 - 2 eps, 12 sectors x 32
+// shifts x 10007 points, takes 1.92 ms against 6.33 ms with the loops.
+namespace taylor {
+// out = a b for the orders LO .. LO + NO - 1, a from order LA, b from order LB;
+// per order in ascending order of a's term
+template <int LA, int NA, int LB, int NB, int LO, int NO>
+__device__ __forceinline__ void ser(const double (&a)[NA], const double (&b)[NB], double (&out)[NO]) {
+#pragma unroll
+    for (int o = 0; o < NO; ++o) {
+        double v = 0.0;
+        bool first = true;
+#pragma unroll
+        for (int k = 0; k < NA; ++k) {
+            const int j = LO + o - (LA + k) - LB;
+            if (j >= 0 && j < NB) {
+                v = first ? __dmul_rn(a[k], b[j]) : fma(a[k], b[j], v);
+                first = false;
+            }
+        }
+        out[o] = v;
+    }
+}
+
+// One V: acc (orders -NS .. 0) += base psi T. ju, jf: U and F over the box at
+// t_V = 0; phi[q][k]: orders -1 .. NS - 1; psi[q]: orders 0 .. NS - 1.
+template <int NS, int R, int V, int LMAX>
+__device__ __forceinline__ void corner1(const TileSmem<LMAX> &S, const double (&ju)[4], const double (&jf)[4],
+                                        double Cc, double Lc, const double (&phi)[NS][2][NS + 1],
+                                        const double (&psi)[NS][NS], double (&acc)[NS + 1]) {
+    constexpr int N = (V & 1) + (V >> 1);          // |V|
+    constexpr int D = V & R;
+    constexpr int K = (D & 1) + (D >> 1), J = 1 << K;
+    const QmcSectorDev &sec = S.sec;
+    const uint64_t *tab = S.logtab;
+    const double U0 = ju[0], F0 = jf[0];
+    const double rU = qrcp(U0), rF = qrcp(F0);
+    // g_i[kappa] = [exp(A) B^i / i!]_kappa
+    double g0[J], g1[J], g2 = 0.0;
+    g0[0] = 1.0;
+    g1[0] = 0.0;
+    if constexpr (K >= 1) {
+        double xu[J], xf[J], A[J], B[J];
+#pragma unroll
+        for (int i = 1; i < J; ++i) {
+            xu[i] = __dmul_rn(ju[i], rU);
+            xf[i] = __dmul_rn(jf[i], rF);
+        }
+        if constexpr (K == 2) {                    // ln(1 + x) = x (1 - x / 2)
+            xu[3] = __dadd_rn(xu[3], fma(xu[2], -0.5 * xu[1], __dmul_rn(xu[1], -0.5 * xu[2])));
+            xf[3] = __dadd_rn(xf[3], fma(xf[2], -0.5 * xf[1], __dmul_rn(xf[1], -0.5 * xf[2])));
+        }
+#pragma unroll
+        for (int i = 1; i < J; ++i) {
+            A[i] = fma(sec.u0, xu[i], __dmul_rn(sec.f0, xf[i]));
+            B[i] = fma(sec.u1, xu[i], __dmul_rn(sec.f1, xf[i]));
+            g0[i] = A[i];
+            g1[i] = B[i];
+        }
+        if constexpr (K == 2) {
+            g0[3] = __dadd_rn(A[3], fma(A[2], 0.5 * A[1], __dmul_rn(A[1], 0.5 * A[2])));
+            g1[3] = fma(A[2], B[1], fma(A[1], B[2], B[3]));
+            g2 = 0.5 * fma(B[2], B[1], __dmul_rn(B[1], B[2]));
+        }
+    }
+    double Bv = Cc;
+    Bv *= sec.u0_int ? ipow_signed<double>(U0, rU, (int)sec.u0) : exp(sec.u0 * qlog_call(U0, tab));
+    Bv *= sec.f0_int ? ipow_signed<double>(F0, rF, (int)sec.f0) : exp(sec.f0 * qlog_call(F0, tab));
+    // base: orders 0 .. N
+    double base[N + 1];
+    base[0] = Bv;
+    if constexpr (N >= 1) {
+        const double Lam = fma(sec.f1, qlog_call(F0, tab), fma(sec.u1, qlog_call(U0, tab), Lc));
+        base[1] = __dmul_rn(Bv, Lam);
+        if constexpr (N >= 2) base[2] = 0.5 * __dmul_rn(base[1], Lam);
+    }
+#pragma unroll
+    for (int q = 0; q < NS; ++q)
+        if (!((V >> q) & 1)) {
+            double w[N + 1];
+            ser<0, N + 1, 0, NS, 0, N + 1>(base, psi[q], w);
+#pragma unroll
+            for (int i = 0; i <= N; ++i) base[i] = w[i];
+        }
+    if constexpr (V == 0) {
+        acc[NS] = __dadd_rn(acc[NS], base[0]);
+    } else {
+        double T[N + 1];                           // orders -N .. 0
+#pragma unroll
+        for (int kap = 0; kap < J; ++kap) {
+            double P[N + 1], Q[N + 1];
+            if constexpr (N == 1) {
+                constexpr int q = V - 1;
+                P[0] = phi[q][kap][0];
+                P[1] = phi[q][kap][1];
+            } else {
+                const int k0 = (D & 1) ? kap & 1 : 0, k1 = (D & 2) ? kap >> (D & 1) : 0;
+                ser<-1, NS + 1, -1, NS + 1, -2, 3>(phi[0][k0], phi[1][k1], P);
+            }
+            double g[N + 1];
+            g[0] = g0[kap];
+            g[1] = g1[kap];
+            if constexpr (N >= 2) g[2] = kap == 3 ? g2 : 0.0;
+            if (kap == 0) {
+#pragma unroll
+                for (int i = 0; i <= N; ++i) T[i] = P[i];
+            } else {
+                ser<0, N + 1, -N, N + 1, -N, N + 1>(g, P, Q);
+#pragma unroll
+                for (int i = 0; i <= N; ++i) T[i] = __dadd_rn(T[i], Q[i]);
+            }
+        }
+        double Q[N + 1];
+        ser<0, N + 1, -N, N + 1, -N, N + 1>(base, T, Q);
+#pragma unroll
+        for (int i = 0; i <= N; ++i) acc[NS - N + i] = __dadd_rn(acc[NS - N + i], Q[i]);
+    }
+}
+}  // namespace taylor
+
+template <int DMAX, int NS, int R, int LMAX>
+__device__ __forceinline__ void eval_real_taylor1(const TileSmem<LMAX> &S, const double (&t)[DMAX], int lo, int nord,
+                                                  double (&res)[LMAX]) {
+    const QmcSectorDev &sec = S.sec;
+    const int d = sec.d;
+    const uint64_t *tab = S.logtab;
+    double Cc = 1.0, Lc = 0.0;
+#pragma unroll
+    for (int j = 0; j < DMAX; ++j)
+        if (j < d && ((sec.regular_mask >> j) & 1)) {
+            if (sec.a[j] > 0) Cc *= ipow_signed<double>(t[j], 1.0, sec.a[j]);
+            if (sec.b[j] != 0.0) Lc = fma(sec.b[j], qlog_call(t[j], tab), Lc);
+        }
+    double psi[NS][NS], phi[NS][2][NS + 1];
+    uint32_t bit[NS];
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+        const bool two = (R >> q) & 1;             // p_q = 2
+        const int sq = sec.sing[q];
+        bit[q] = 1u << sq;
+        double tq = t[0];
+#pragma unroll
+        for (int j = 1; j < DMAX; ++j)
+            if (j == sq) tq = t[j];
+        const double tinv = qrcp(tq), bq = sec.b[sq];
+        const double bl = NS > 1 ? bq * qlog_call(tq, tab) : 0.0;
+        const double tp = two ? __dmul_rn(tinv, tinv) : tinv;
+        // phi(p - 1) = 1/(b eps) - t^{-1 + b eps}, phi(p - 2) = 1/(-1 + b eps) - t^{-2 + b eps}
+        const int top = two ? 1 : 0;
+        psi[q][0] = tp;
+        phi[q][top][0] = qrcp(bq);
+        phi[q][top][1] = -tinv;
+        if (two) {
+            phi[q][0][0] = 0.0;
+            phi[q][0][1] = __dadd_rn(-tp, -1.0);
+        }
+        if constexpr (NS > 1) {
+            psi[q][1] = __dmul_rn(tp, bl);
+            phi[q][top][2] = __dmul_rn(-tinv, bl);
+            if (two) phi[q][0][2] = __dadd_rn(__dmul_rn(-tp, bl), -bq);
+        }
+    }
+    // U and F over the box of each V, per V in the monomials' order
+    constexpr int NV = 1 << NS;
+    double jw[2][NV][4];
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+#pragma unroll
+        for (int V = 0; V < NV; ++V)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) jw[w][V][i] = 0.0;
+        const int m1 = w == 0 ? sec.nU : sec.nU + sec.nF;
+#pragma unroll 1
+        for (int m = w == 0 ? 0 : sec.nU; m < m1; ++m) {
+            const uint32_t ex = S.exps[m];
+            const double c = S.cval[m];
+            uint32_t has = 0;                      // variables with an exponent
+#pragma unroll
+            for (int j = 0; j < DMAX; ++j)
+                if (j < d && ((ex >> (4 * j)) & 15u)) has |= 1u << j;
+            int eq[NS];
+#pragma unroll
+            for (int q = 0; q < NS; ++q) eq[q] = (int)((ex >> (4 * sec.sing[q])) & 15u);
+#pragma unroll
+            for (int V = 0; V < NV; ++V) {
+                constexpr int DR = R;
+                int idx = 0, sh = 0;
+                bool keep = true;
+                uint32_t rest = has;
+#pragma unroll
+                for (int q = 0; q < NS; ++q)
+                    if ((V >> q) & 1) {
+                        rest &= ~bit[q];
+                        if ((DR >> q) & 1) {
+                            keep = keep && eq[q] < 2;
+                            idx |= eq[q] << sh;
+                            ++sh;
+                        } else {
+                            keep = keep && eq[q] == 0;
+                        }
+                    }
+                if (!keep) continue;               // the same for the whole tile
+                double v = c;
+#pragma unroll 1
+                for (; rest; rest &= rest - 1) {
+                    const int j = __ffs((int)rest) - 1;
+                    const uint32_t e = (ex >> (4 * j)) & 15u;
+                    double x = t[0];
+#pragma unroll
+                    for (int k = 1; k < DMAX; ++k)
+                        if (j == k) x = t[k];
+                    double p = x;
+                    if (e > 1) {
+                        p = __dmul_rn(x, x);
+                        if (e == 3) p = __dmul_rn(p, x);
+                        if (e == 4) p = __dmul_rn(p, p);
+                    }
+                    v = __dmul_rn(v, p);
+                }
+                const int nj = 1 << sh;
+                double a = jw[w][V][0];
+#pragma unroll
+                for (int i = 1; i < 4; ++i)
+                    if (i < nj && idx == i) a = jw[w][V][i];
+                a = __dadd_rn(a, v);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (i < nj && idx == i) jw[w][V][i] = a;
+            }
+        }
+    }
+    double acc[NS + 1];
+#pragma unroll
+    for (int i = 0; i <= NS; ++i) acc[i] = 0.0;
+    taylor::corner1<NS, R, 0, LMAX>(S, jw[0][0], jw[1][0], Cc, Lc, phi, psi, acc);
+    taylor::corner1<NS, R, 1, LMAX>(S, jw[0][1], jw[1][1], Cc, Lc, phi, psi, acc);
+    if constexpr (NS > 1) {
+        taylor::corner1<NS, R, 2, LMAX>(S, jw[0][2], jw[1][2], Cc, Lc, phi, psi, acc);
+        taylor::corner1<NS, R, 3, LMAX>(S, jw[0][3], jw[1][3], Cc, Lc, phi, psi, acc);
+    }
+#pragma unroll
+    for (int o = 0; o < LMAX; ++o) {
+        res[o] = 0.0;
+#pragma unroll
+        for (int i = 0; i <= NS; ++i)
+            if (o < nord && i == lo + o + NS) res[o] = acc[i];
+    }
+}
+
 // ---------------------------------------------------------------- deformed integrand
 // z_j = t_j - i lambda_j t_j (1 - t_j) dF/dt_j at the (corner) point, with
 // rho_j = z_j / t_j for singular variables and J = dz/dt; every quantity of
@@ -2437,6 +2694,17 @@ __device__ __forceinline__ void thread_points(const TileSmem<LMAX> &S, const Qmc
 #pragma unroll
     for (int j = 0; j < DMAX; ++j) walk_init(wk[j], (j < d) ? (k0 * (uint64_t)S.zmod[j]) % n : 0, n);
 #pragma unroll 1
+    // Taylor subtraction: the instantiation of eval_real_taylor1 that serves
+    // the tile's sector (4: one variable, p = 2; 1 .. 3: two, the bits of those
+    // with p = 2), 0 for the loops, which take any p, order and number of
+    // variables
+    int kind = 0;
+    if constexpr (HS && !CPLX && DMAX <= 3) {
+        const QmcSectorDev &sec = S.sec;
+        const int p0 = sec.ns >= 1 ? -sec.a[sec.sing[0]] : 0, p1 = sec.ns >= 2 ? -sec.a[sec.sing[1]] : 0;
+        if (hi == 0 && sec.ns == 1 && p0 == 2) kind = 4;
+        if (hi == 0 && sec.ns == 2 && p0 <= 2 && p1 <= 2) kind = (p0 == 2 ? 1 : 0) | (p1 == 2 ? 2 : 0);
+    }
     for (uint64_t k = k0; k < kend; ++k) {
         double t[DMAX], omt[DMAX];
         double Ws = 1.0;  // prod u(1-u); the korobov3 weight is 140^d Ws^3
@@ -2499,8 +2767,15 @@ __device__ __forceinline__ void thread_points(const TileSmem<LMAX> &S, const Qmc
             } else if constexpr (CPLX) {
                 eval_deformed<DMAX, SMAX, LMAX, MIXED>(S, t, omt, lo, hi, nord, res, signfail_tile);
             } else {
-                if constexpr (HS) {
-                    eval_real_taylor<DMAX, SMAX, LMAX, (DMAX <= 3 ? QMC_JMAX3 : QMC_JMAX6)>(S, t, lo, hi, nord, res);
+                if constexpr (HS && DMAX <= 3) {
+                    // uniform per tile
+                    if (kind == 4) eval_real_taylor1<DMAX, 1, 1, LMAX>(S, t, lo, nord, res);
+                    else if (kind == 1) eval_real_taylor1<DMAX, 2, 1, LMAX>(S, t, lo, nord, res);
+                    else if (kind == 2) eval_real_taylor1<DMAX, 2, 2, LMAX>(S, t, lo, nord, res);
+                    else if (kind == 3) eval_real_taylor1<DMAX, 2, 3, LMAX>(S, t, lo, nord, res);
+                    else eval_real_taylor<DMAX, SMAX, LMAX, QMC_JMAX3>(S, t, lo, hi, nord, res);
+                } else if constexpr (HS) {
+                    eval_real_taylor<DMAX, SMAX, LMAX, QMC_JMAX6>(S, t, lo, hi, nord, res);
                 } else if constexpr (DMAX <= 3) {
                     // one instantiation per number of singular variables (uniform per tile)
                     if (S.sec.ns == 2) eval_real<DMAX, SMAX, LMAX, MIXED, 2>(S, t, lo, hi, nord, res);
