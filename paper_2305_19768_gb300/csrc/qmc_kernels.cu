@@ -1645,7 +1645,7 @@ __device__ __noinline__ void eval_real_taylor(const TileSmem<LMAX> &S, const dou
 // store are not contracted into the sums that follow), so the results are the
 // same bits. FP64-bound; the loops carry full series at run-time extents in
 // local memory. The one-loop box in D = 2 - 2 eps, 12 sectors x 32
-// shifts x 10007 points, takes 1.92 ms against 6.33 ms with the loops.
+// shifts x 10007 points, takes 1.87 ms against 6.33 ms with the loops.
 namespace taylor {
 // out = a b for the orders LO .. LO + NO - 1, a from order LA, b from order LB;
 // per order in ascending order of a's term
@@ -1667,6 +1667,15 @@ __device__ __forceinline__ void ser(const double (&a)[NA], const double (&b)[NB]
     }
 }
 
+// x^e, 2 <= e <= 4, as powers() forms it; out of line, since an FP64
+// instruction switched off by a predicate holds the pipe all the same
+__device__ __noinline__ double power_call(double x, uint32_t e) {
+    double p = __dmul_rn(x, x);
+    if (e == 3) p = __dmul_rn(p, x);
+    if (e == 4) p = __dmul_rn(p, p);
+    return p;
+}
+
 // One V: acc (orders -NS .. 0) += base psi T. ju, jf: U and F over the box at
 // t_V = 0; phi[q][k]: orders -1 .. NS - 1; psi[q]: orders 0 .. NS - 1.
 template <int NS, int R, int V, int LMAX>
@@ -1679,7 +1688,9 @@ __device__ __forceinline__ void corner1(const TileSmem<LMAX> &S, const double (&
     const QmcSectorDev &sec = S.sec;
     const uint64_t *tab = S.logtab;
     const double U0 = ju[0], F0 = jf[0];
-    const double rU = qrcp(U0), rF = qrcp(F0);
+    const double rF = qrcp(F0);
+    double rU = 1.0;                               // without jets only for a negative or fractional power
+    if (K > 0 || !sec.u0_int || sec.u0 < 0.0) rU = qrcp(U0);
     // g_i[kappa] = [exp(A) B^i / i!]_kappa
     double g0[J], g1[J], g2 = 0.0;
     g0[0] = 1.0;
@@ -1764,8 +1775,8 @@ __device__ __forceinline__ void corner1(const TileSmem<LMAX> &S, const double (&
 }  // namespace taylor
 
 template <int DMAX, int NS, int R, int LMAX>
-__device__ __forceinline__ void eval_real_taylor1(const TileSmem<LMAX> &S, const double (&t)[DMAX], int lo, int nord,
-                                                  double (&res)[LMAX]) {
+__device__ __forceinline__ void eval_real_taylor1(const TileSmem<LMAX> &S, const double (&t)[DMAX],
+                                                  const double (&rb)[2], int lo, int nord, double (&res)[LMAX]) {
     const QmcSectorDev &sec = S.sec;
     const int d = sec.d;
     const uint64_t *tab = S.logtab;
@@ -1793,7 +1804,7 @@ __device__ __forceinline__ void eval_real_taylor1(const TileSmem<LMAX> &S, const
         // phi(p - 1) = 1/(b eps) - t^{-1 + b eps}, phi(p - 2) = 1/(-1 + b eps) - t^{-2 + b eps}
         const int top = two ? 1 : 0;
         psi[q][0] = tp;
-        phi[q][top][0] = qrcp(bq);
+        phi[q][top][0] = rb[q];                    // 1/b_q
         phi[q][top][1] = -tinv;
         if (two) {
             phi[q][0][0] = 0.0;
@@ -1819,6 +1830,7 @@ __device__ __forceinline__ void eval_real_taylor1(const TileSmem<LMAX> &S, const
         for (int m = w == 0 ? 0 : sec.nU; m < m1; ++m) {
             const uint32_t ex = S.exps[m];
             const double c = S.cval[m];
+            const bool unit = __double_as_longlong(c) == 0x3FF0000000000000LL;
             uint32_t has = 0;                      // variables with an exponent
 #pragma unroll
             for (int j = 0; j < DMAX; ++j)
@@ -1845,23 +1857,20 @@ __device__ __forceinline__ void eval_real_taylor1(const TileSmem<LMAX> &S, const
                         }
                     }
                 if (!keep) continue;               // the same for the whole tile
-                double v = c;
-#pragma unroll 1
-                for (; rest; rest &= rest - 1) {
+                auto factor = [&]() {              // the next variable's power
                     const int j = __ffs((int)rest) - 1;
                     const uint32_t e = (ex >> (4 * j)) & 15u;
+                    rest &= rest - 1;
                     double x = t[0];
 #pragma unroll
                     for (int k = 1; k < DMAX; ++k)
                         if (j == k) x = t[k];
-                    double p = x;
-                    if (e > 1) {
-                        p = __dmul_rn(x, x);
-                        if (e == 3) p = __dmul_rn(p, x);
-                        if (e == 4) p = __dmul_rn(p, p);
-                    }
-                    v = __dmul_rn(v, p);
-                }
+                    return e > 1 ? taylor::power_call(x, e) : x;
+                };
+                double v = c;
+                if (unit && rest) v = factor();    // 1 x = x
+#pragma unroll 1
+                while (rest) v = __dmul_rn(v, factor());
                 const int nj = 1 << sh;
                 double a = jw[w][V][0];
 #pragma unroll
@@ -2657,7 +2666,9 @@ __device__ void stage_tile(TileSmem<LMAX> &S, const QmcLaunch &Lc, int jidx) {
 // dependent FP64 operations, and resident warps hide more of that than the
 // registers save. One-loop box in D = 2 - 2 eps, n = 10007, 32 shifts: 9.28 ms
 // at 2 blocks (186 registers), 7.41 at 3, 6.48 at 4 (128), 6.57 at 5; its
-// deformed form at 16 points 111.6, 90.8, 81.9, 79.8.
+// deformed form at 16 points 111.6, 90.8, 81.9, 79.8. (These are the loops; the
+// written-out first-degree form is bound by the FP64 pipe and takes 1.9 ms there
+// at 3, 4 and 5 blocks alike.)
 #ifndef QMC_MINB_H
 #define QMC_MINB_H 4
 #endif
@@ -2699,11 +2710,14 @@ __device__ __forceinline__ void thread_points(const TileSmem<LMAX> &S, const Qmc
     // with p = 2), 0 for the loops, which take any p, order and number of
     // variables
     int kind = 0;
+    double rb[2] = {0.0, 0.0};   // 1/b of the singular variables
     if constexpr (HS && !CPLX && DMAX <= 3) {
         const QmcSectorDev &sec = S.sec;
         const int p0 = sec.ns >= 1 ? -sec.a[sec.sing[0]] : 0, p1 = sec.ns >= 2 ? -sec.a[sec.sing[1]] : 0;
         if (hi == 0 && sec.ns == 1 && p0 == 2) kind = 4;
         if (hi == 0 && sec.ns == 2 && p0 <= 2 && p1 <= 2) kind = (p0 == 2 ? 1 : 0) | (p1 == 2 ? 2 : 0);
+        if (kind) rb[0] = qrcp(sec.b[sec.sing[0]]);
+        if (kind && kind < 4) rb[1] = qrcp(sec.b[sec.sing[1]]);
     }
     for (uint64_t k = k0; k < kend; ++k) {
         double t[DMAX], omt[DMAX];
@@ -2769,10 +2783,10 @@ __device__ __forceinline__ void thread_points(const TileSmem<LMAX> &S, const Qmc
             } else {
                 if constexpr (HS && DMAX <= 3) {
                     // uniform per tile
-                    if (kind == 4) eval_real_taylor1<DMAX, 1, 1, LMAX>(S, t, lo, nord, res);
-                    else if (kind == 1) eval_real_taylor1<DMAX, 2, 1, LMAX>(S, t, lo, nord, res);
-                    else if (kind == 2) eval_real_taylor1<DMAX, 2, 2, LMAX>(S, t, lo, nord, res);
-                    else if (kind == 3) eval_real_taylor1<DMAX, 2, 3, LMAX>(S, t, lo, nord, res);
+                    if (kind == 4) eval_real_taylor1<DMAX, 1, 1, LMAX>(S, t, rb, lo, nord, res);
+                    else if (kind == 1) eval_real_taylor1<DMAX, 2, 1, LMAX>(S, t, rb, lo, nord, res);
+                    else if (kind == 2) eval_real_taylor1<DMAX, 2, 2, LMAX>(S, t, rb, lo, nord, res);
+                    else if (kind == 3) eval_real_taylor1<DMAX, 2, 3, LMAX>(S, t, rb, lo, nord, res);
                     else eval_real_taylor<DMAX, SMAX, LMAX, QMC_JMAX3>(S, t, lo, hi, nord, res);
                 } else if constexpr (HS) {
                     eval_real_taylor<DMAX, SMAX, LMAX, QMC_JMAX6>(S, t, lo, hi, nord, res);
@@ -2804,8 +2818,7 @@ __device__ __forceinline__ void thread_points(const TileSmem<LMAX> &S, const Qmc
     }
 }
 
-// FIX: the real classes' kernel for sums up to eps^0 (highest order 0, every
-// sum the integrator forms), with only the compile-time paths; the general
+// FIX: the real classes' kernel for sums up to eps^0 (highest order 0), with only the compile-time paths; the general
 // kernel (FIX = false) serves every other order window. Two instantiations
 // keep each kernel's code, and its instruction-cache footprint, small.
 template <int DMAX, int SMAX, int LMAX, bool CPLX, bool MIXED, int BLOCK, bool HS = false, bool FIX = false>
