@@ -115,12 +115,21 @@ PROFILED = {
         "warp_inst_per_eval": 445.4, "issue_busy": 0.364},
 }
 
+# What the roofline counts (flops.py): the specialised evaluators run part of
+# it on the integer pipe, so a fraction of the DFMA peak built on it is
+# FP64-equivalent work and may pass 1
+FLOPS_OF = ("the general evaluator's formulation; qmc_real_kernel and qmc_deformed_kernel run part of it on the "
+            "integer pipe (FP64-equivalent, not a share of the FP64 pipe)")
+
+
 def kernel_sha1():
     import hashlib
 
-    path = os.path.join(ROOT, "paper_2305_19768_gb300", "csrc", "qmc_kernels.cu")
-    with open(path, "rb") as fh:
-        return hashlib.sha1(fh.read()).hexdigest()
+    h = hashlib.sha1()
+    for name in ("qmc_kernels.cu", "qmc_real.cuh", "qmc_deformed.cuh"):
+        with open(os.path.join(ROOT, "paper_2305_19768_gb300", "csrc", name), "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()
 
 
 def _env_int(name, default):
@@ -275,7 +284,7 @@ def box_extra(device, opts, sptr, flush, peak_gflops, seed):
         out["box1L_massless"] = {
             "workload": W["desc"].format(n=W["n"], m=W["m"]), "evals_per_s": rate, "eval_ms": float(np.mean(ms)),
             "roofline": {"achieved": fl * rate / 1e9, "peak": peak_gflops, "frac": fl * rate / 1e9 / peak_gflops,
-                         "flops_per_eval": fl, "unit": "GFLOP/s (fp64)"}}
+                         "flops_per_eval": fl, "flops_of": FLOPS_OF, "unit": "GFLOP/s (fp64)"}}
         for prec, key in ((qmc.QMC_PRECISION_FP64, "fp64"), (qmc.QMC_PRECISION_MIXED, "mixed")):
             c2 = qmc.qmc_create(device, precision=prec, **opts)
             try:
@@ -330,7 +339,7 @@ def batch_extra(device, opts, sptr, flush, peak_gflops, seed, n=100003, m=32):
     return {"box1L_massive_batch": {
         "workload": W["desc"].format(n=n, m=m), "evals_per_s": rate, "eval_ms": float(np.mean(ms)),
         "roofline": {"achieved": fl * rate / 1e9, "peak": peak_gflops, "frac": fl * rate / 1e9 / peak_gflops,
-                     "flops_per_eval": fl, "unit": "GFLOP/s (fp64)"}}}
+                     "flops_per_eval": fl, "flops_of": FLOPS_OF, "unit": "GFLOP/s (fp64)"}}}
 
 
 def mixed_extra(device, opts, I, W, kin, jobs, nj, evals_per_step, out_dev, sptr, seed, skip_oracle):
@@ -558,9 +567,8 @@ def main():
         t_e2e += time.perf_counter() - t0
     e2e_val = evals_per_step * n_e2e * world / t_e2e
 
-    # roofline of the evaluator kernels: FP64 flops of the formulation (no
-    # credit for the steps on the integer pipe) / their event time, against
-    # the DFMA peak measured in this run; FP32 work of the mixed classes
+    # roofline of the evaluator kernels: FP64 flops of the general evaluator's
+    # formulation / their event time, against the DFMA peak measured in this run; FP32 work of the mixed classes
     # against the FFMA peak; transcendentals per evaluation beside them
     work = flopmod.workload_work(I, LO, NORD, mixed=args.precision == "mixed")
     avg_eval_ms = float(np.mean(eval_ms))
@@ -570,15 +578,14 @@ def main():
     prof = PROFILED.get((sha, args.workload, args.precision, args.decomposition, args.n), {})
     roof = {"bound": "alu", "achieved": achieved, "peak": peak_gflops, "unit": "GFLOP/s (fp64)",
             "frac": achieved / peak_gflops, "traffic": prof.get("traffic"),
-            "flops_per_eval": work.fp64, "peak_source": "DFMA probe in this run (of measured)",
+            "flops_per_eval": work.fp64, "flops_of": FLOPS_OF, "peak_source": "DFMA probe in this run (of measured)",
             "transcendentals_per_eval": {k: getattr(work, k) for k in ("log", "atan2", "rcp", "exp", "rcp_int")},
             "fp64_executed_flops_per_eval": prof.get("fp64_executed_flops_per_eval"),
             "fp64_pipe_busy": prof.get("fp64_pipe_busy"),
             "evals_per_launch": evals_per_step, "eval_ms_per_step": avg_eval_ms,
             "kernel_sha1": sha}
-    # the same formulation counted as if all of it ran in FP64 (the corner stage
-    # that the d <= 6 kernel runs on the integer pipe included): algorithmic,
-    # not FP64-pipe work
+    # the same formulation counted as if all of it ran in FP64, the d <= 6 corner
+    # stage included: algorithmic, not FP64-pipe work
     eq = flopmod.workload_work(I, LO, NORD, mixed=args.precision == "mixed", fp64_corners=True).fp64
     if eq != work.fp64:
         roof["algorithmic_fp64_equivalent"] = {"flops_per_eval": eq, "achieved": eq * rate / 1e9,

@@ -1,8 +1,11 @@
 """FP64 and FP32 work per integrand evaluation (the roofline numerator).
 
 One evaluation = one lattice point of one sector for one shift, all eps
-orders, all subtraction corners. The count follows the evaluator's own
-formulation of the method, operation by operation:
+orders, all subtraction corners. The count follows the general evaluator's
+formulation of the method (qmc_eval_kernel), operation by operation. The
+specialised evaluators (qmc_real_kernel, qmc_deformed_kernel) need fewer FP64
+operations for the same sums and run more on the integer pipe; at their rates
+this count is FP64-equivalent work, not a share of the FP64 pipe.
 
 * FP64 flops: add, subtract and multiply count 1, a fused multiply-add 2.
   Steps that the evaluator computes on the integer pipe count 0 FP64 flops:
