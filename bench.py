@@ -110,9 +110,9 @@ PROFILED = {
     # double box, n = 1000003, m = 32 (the default line): traffic from a 1-pass
     # capture of one full launch; instruction counts and pipe activity from the
     # full capture of the same kernel at n = 20011 (per evaluation, the same code)
-    ("76aa350fe61515433bc16a2675f5d037ffad47af", "box2L_planar_massless", "fp64", "iterative", 1000003): {
-        "traffic": 1628160 + 3601233152, "fp64_executed_flops_per_eval": 290.7, "fp64_pipe_busy": 0.419,
-        "warp_inst_per_eval": 445.4, "issue_busy": 0.364},
+    ("d3f921baac652e14754100c686ca113859c905de", "box2L_planar_massless", "fp64", "iterative", 1000003): {
+        "traffic": 111145199104 + 2148485046272, "fp64_executed_flops_per_eval": 269.4, "fp64_pipe_busy": 0.477,
+        "warp_inst_per_eval": 386.3, "issue_busy": 0.529},
 }
 
 # What the roofline counts (flops.py): the specialised evaluators run part of
