@@ -787,8 +787,10 @@ __device__ __forceinline__ void fx_stage(FxShared &S, const QmcLaunch &Lc) {
         const QmcMono &Mo = Lc.monos[src->monoU + m];
         double v = Mo.coef[0];
         for (int i = 0; i < Lc.ninv && i + 1 < QMC_NCOEF; ++i) v = fma(Mo.coef[i + 1], kin[i], v);
-        S.cfix[m] = (uint64_t)__double_as_longlong(v);
-        atomicMax(&S.emax[m < nU ? 0 : 1], (int)((uint64_t)__double_as_longlong(v) >> 52) - 1023);
+        // v >= 0 here, but -0.0 too: without its sign, which would read as an exponent bit
+        const uint64_t vb = (uint64_t)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFULL;
+        S.cfix[m] = vb;
+        atomicMax(&S.emax[m < nU ? 0 : 1], (int)(vb >> 52) - 1023);
         uint32_t off[6] = {0, 0, 0, 0, 0, 0};
         uint32_t k = 0;
 #pragma unroll
