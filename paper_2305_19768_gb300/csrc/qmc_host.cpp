@@ -391,6 +391,11 @@ bool fx_job_ok(const qmc_ctx *ctx, const HostSector &S, int cls, int point) {
     const size_t ninv = (size_t)ctx->ninv;
     if ((size_t)point * ninv + ninv > ctx->h_kin.size() && ninv > 0) return false;
     const double *kin = ctx->h_kin.data() + (size_t)point * ninv;
+    // mixed precision holds the coefficients and their products in FP32: inside
+    // this range none overflows, and what FP32's subnormals lose is below 2^-59
+    // of c0; beyond it the general kernel's infinities and NaN must show
+    const bool fp32 = cls == QMC_CLASS_REAL3M || cls == QMC_CLASS_REAL6M;
+    const double least = fp32 ? 1e-20 : 1e-100;
     for (const std::vector<Term> *P : {&S.U, &S.F}) {
         double sum = 0.0, c0 = 0.0;
         for (const Term &T : *P) {
@@ -402,7 +407,7 @@ bool fx_job_ok(const qmc_ctx *ctx, const HostSector &S, int cls, int point) {
             for (int j = 0; j < S.d; ++j) constant = constant && T.e[j] == 0;
             if (constant) c0 += v;
         }
-        if (!(c0 > 1e-100) || !(sum < 1e100) || !(sum <= 128.0 * c0)) return false;
+        if (!(c0 > least) || !(sum < 1.0 / least) || !(sum <= 128.0 * c0)) return false;
     }
     return true;
 }

@@ -1,5 +1,7 @@
 """Coefficients, kinematics and sectors at the edges of what the evaluators of
 csrc/qmc_real.cuh and csrc/qmc_deformed.cuh take (GPU)."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -7,9 +9,11 @@ from paper_2305_19768_gb300 import qmc
 from paper_2305_19768_gb300.inputs import workloads as w
 
 from parity import Gpu
-from test_gpu_real_integer import _compare, _specs
+from test_gpu_real_integer import _compare, _specs, general
 
 pytestmark = pytest.mark.gpu
+
+NONFINITE = -7
 
 
 class _Text:
@@ -57,5 +61,29 @@ def test_signed_zero_coefficients(name, mixed):
         a, _, ra = g.eval(zid, [dict(sp, integral_id=zid) for sp in specs], lo, nord)
         assert ra == 0 and rb == 0
         _compare(I, specs, a, b, kin, 2, lo, nord, 0)
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("scale", [1e40, 1e22, 1e-22, 1e-42])
+@pytest.mark.parametrize("name", ["box", "double_box"])
+def test_mixed_coefficients_near_and_beyond_the_fp32_range(name, scale):
+    """Where FP32 coefficients overflow or lose bits, mixed jobs give what the
+    general kernel gives: its sums, or its status for sums that are not finite."""
+    build, lo = (w.box_massless, -2) if name == "box" else (w.double_box_massless, -4)
+    I = build()
+    g = Gpu(precision=qmc.QMC_PRECISION_MIXED)
+    try:
+        iid, gid = g.load(I), g.load(general(I, Fraction(-1, 10 ** 250)))
+        qmc.qmc_set_kinematics(g.ctx, np.array([[-3.0 * scale, -2.0 * scale]]))
+        specs = _specs(iid, I, name, 1, 1009, 2)
+        nord = 1 - lo
+        a, _, ra = g.eval(iid, specs, lo, nord)
+        b, _, rb = g.eval(gid, [dict(sp, integral_id=gid) for sp in specs], lo, nord)
+        assert ra == rb
+        if scale == 1e40 and name == "box":
+            assert rb == NONFINITE
+        if rb == 0:
+            assert np.all(np.abs(a - b) <= 1e-9 * np.abs(b).max())
     finally:
         g.close()
