@@ -74,11 +74,16 @@ struct alignas(16) FdShared {
 };
 __device__ __forceinline__ FdShared &fd_shared() { return *reinterpret_cast<FdShared *>(qmc_fx_raw); }
 
-// Positive FP64 values as mantissa and exponent; zero (or worse) gives a tiny
-// one: the integrand is singular there and the sum not finite
+// A squared norm as mantissa and exponent. Zero, subnormal, infinite and NaN
+// ones get the exponent kFdBad, beyond anything that products of the others
+// reach (|e| < 2^15), so that one look at a product's exponent finds them: a
+// negative power or a logarithm of such a factor has no value, and the corner is
+// NaN (mantissas alone would give a finite number, since conj(0) / 2^-1022 = 0).
+constexpr int kFdBad = 1 << 20;
 __device__ __forceinline__ FxM fd_of(double x) {
-    const qmc_xf a = qmc_xf_of(x);
-    return a.m ? FxM{a.m, a.e} : FxM{1ULL << 63, -1022};
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    const uint32_t ex = (uint32_t)(b >> 52) & 0x7FFu;
+    return FxM{(b << 11) | (1ULL << 63), ex - 1u < 0x7FEu ? (int)ex - 1023 : kFdBad};
 }
 __device__ __forceinline__ FxM fd_rcp(FxM a) {
     const qmc_xf r = qmc_xf_rcp3(qmc_xf{a.m, a.e, 0});
@@ -480,6 +485,7 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
     }
     if (needU) factor(U, fd_norm2(U.re, U.im), S.u0, S.u1, false);
     factor(F, fd_norm2(F.re, F.im), S.f0, S.f1, true);
+    if (max(den.e, max(np.e, nn.e)) > kFdBad / 2) B.re = B.im = __longlong_as_double(0x7FF8000000000000LL);
     out.B = B;
     out.q = fd_rcp(den);
     out.L = dc{0.0, 0.0};

@@ -7,6 +7,7 @@ import pytest
 
 from paper_2305_19768_gb300 import qmc
 from paper_2305_19768_gb300.inputs import workloads as w
+from paper_2305_19768_gb300.inputs.integral import Integral
 
 from parity import Gpu
 from test_gpu_real_integer import _compare, _specs, general
@@ -87,3 +88,61 @@ def test_mixed_coefficients_near_and_beyond_the_fp32_range(name, scale):
             assert np.all(np.abs(a - b) <= 1e-9 * np.abs(b).max())
     finally:
         g.close()
+
+TOY = """qmc-sectors 1
+name toy
+loops 1 propagators 3 dim 4
+invariants 1 s
+prefactor 0 1 1.0 0.0
+nsectors 1
+sector 0 d 1 deform 1
+a 0
+b 0.0
+U 0.0 0.0 1
+0 1.0 0.0
+F {f0} {f1} 2
+0 0.0 1.0
+1 0.0 -2.0
+end
+"""
+
+
+def _status(I, lo, nord, kin, lam, mixed=False, n=1009, z=None, transform=0, flags=0):
+    """(general kernel's status, the job's own)"""
+    g = Gpu(transform=transform, precision=qmc.QMC_PRECISION_MIXED if mixed else qmc.QMC_PRECISION_FP64)
+    try:
+        iid = g.load(I)
+        qmc.qmc_set_kinematics(g.ctx, np.array([kin]))
+        J = Integral.from_text(I.to_text())
+        specs = [dict(integral_id=iid, sector=s, point=0, shifts=1 if flags else 2, n=n, seed=3, stream=s, flags=flags,
+                      **{"lambda": lam}, **({} if z is None else {"z": z})) for s in range(len(J.sectors))]
+        got = g.eval(iid, specs, lo, nord)[2]
+        gid = g.load(general(J, Fraction(1, 10 ** 250)))
+        return g.eval(gid, [dict(sp, integral_id=gid) for sp in specs], lo, nord)[2], got
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("s", [0.0, 1e160, 1e-170])
+@pytest.mark.parametrize("name,lo,nord", [("triangle", -2, 3), ("bubble", -1, 3)])
+def test_zero_and_unrepresentable_F_are_reported(name, lo, nord, s, mixed):
+    """F = 0 everywhere (s = 0), also where only its logarithm enters (the bubble
+    to eps^1), and |F|^2 outside FP64's normal range: the sums are not finite,
+    and the status says so, as with the general kernel."""
+    I = w.triangle_one_offshell(0, "s") if name == "triangle" else w.bubble(0, "s")
+    ref, got = _status(I, lo, nord, [s], 0.5, mixed)
+    assert got == NONFINITE
+    if not mixed:
+        assert ref == NONFINITE
+
+
+@pytest.mark.parametrize("f0,f1,nord,status", [(-1.0, 0.0, 1, NONFINITE), (-2.0, -1.0, 1, NONFINITE),
+                                               (0.0, -1.0, 2, NONFINITE), (1.0, 0.0, 1, 0), (1.0, 0.0, 2, 0)])
+def test_one_point_with_F_zero(f0, f1, nord, status):
+    """F = s (1 - 2 t), undeformed (lambda = 0), unshifted lattice of 1024 points
+    without a transform: F = 0 at t = 1/2, an error for a negative power or a
+    logarithm and a plain zero for a positive power."""
+    ref, got = _status(_Text(TOY.format(f0=f0, f1=f1)), 0, nord, [3.0], 0.0, n=1024, z=[1, 1, 1, 1, 1, 1],
+                       transform=2, flags=qmc.QMC_JOB_UNSHIFTED)
+    assert got == status and ref == status
