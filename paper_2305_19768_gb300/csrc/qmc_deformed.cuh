@@ -140,24 +140,41 @@ __device__ __forceinline__ double fd_from57(int64_t a) {
     return fd_signed(fx_pack(fx_norm(FxM{u, 6})), a < 0);
 }
 
-// FP32 <-> FP64 conversions on the integer pipe (normal range; below it 0)
+// FP32 <-> FP64 conversions on the integer pipe (RN; subnormals, infinities and
+// NaN too, behind one test)
 __device__ __forceinline__ float fd_to_float(double x) {
-    const uint64_t b = (uint64_t)__double_as_longlong(x);
-    const uint32_t hi = (uint32_t)(b >> 32);
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
     const int e = (int)((hi >> 20) & 0x7FFu) - 896;                    // FP32's biased exponent
-    uint32_t m = (uint32_t)(b >> 29) & 0x7FFFFFu;
-    const uint32_t rest = (uint32_t)b & 0x1FFFFFFFu;
-    const uint32_t up = (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u))) ? 1u : 0u;
-    const uint32_t v = ((uint32_t)e << 23) + m + up;
-    return e >= 255 ? __double2float_rn(x) : (e > 0 ? __uint_as_float((hi & 0x80000000u) | v) : 0.0f);
+    uint32_t m = (hi << 3 | lo >> 29) & 0x7FFFFFu, rest = lo << 3, out = (uint32_t)e << 23;
+    if (__builtin_expect((uint32_t)e - 1u >= 254u, 0)) {
+        out = 0;
+        if (e >= 255) {                                                // infinite, too large, NaN
+            m = 0x7F800000u | (e == 1151 && (m | rest) ? 0x400000u : 0u);
+            rest = 0;
+        } else if (e >= -24) {                                         // below FP32's normal range
+            const uint64_t f = ((uint64_t)(m | 0x800000u) << 32 | rest) >> (1 - e);
+            rest = (uint32_t)f | (rest ? 1u : 0u);
+            m = (uint32_t)(f >> 32);
+        } else {                                                       // below half the smallest
+            m = rest = 0;
+        }
+    }
+    out += m + ((rest > 0x80000000u || (rest == 0x80000000u && (m & 1u))) ? 1u : 0u);
+    return __uint_as_float((hi & 0x80000000u) | out);
 }
 __device__ __forceinline__ double fd_to_double(float x) {
     const uint32_t b = __float_as_uint(x);
-    const uint32_t e = (b >> 23) & 255u;
-    if (e == 0) return 0.0;
-    if (e == 255) return (double)x;
-    const uint32_t hi = (b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7FFFFFu) >> 3);
-    return __hiloint2double((int)hi, (int)(b << 29));
+    uint32_t e = ((b >> 23) & 255u) + 896u, m = b & 0x7FFFFFu;
+    if (__builtin_expect(e - 897u >= 254u, 0)) {
+        if (e != 896u) {
+            e = 2047u;                                                 // infinite, NaN
+        } else {
+            const int p = __clz((int)m) - 8;                           // 0 or subnormal
+            e = m ? 897u - (uint32_t)p : 0u;
+            m = (m << p) & 0x7FFFFFu;
+        }
+    }
+    return __hiloint2double((int)((b & 0x80000000u) | (e << 20) | (m >> 3)), (int)(m << 29));
 }
 
 // complex arithmetic in FMAs (an FP64 multiply holds the pipe longer than an FMA)
@@ -165,10 +182,16 @@ struct FdOps {
     double mone, nzero, one;
     __device__ __forceinline__ double mul(double a, double b) const { return fma(a, b, nzero); }
     __device__ __forceinline__ double add(double a, double b) const { return fma(b, one, a); }
-    // 2 a on the exponent (a normal, or 0 for anything below)
+    // 2 a on the exponent; behind one test, zero and subnormals on the mantissa,
+    // and infinities and NaN stay
     __device__ __forceinline__ double dbl(double a) const {
-        const int h = __double2hiint(a);
-        return (h & 0x7FF00000) ? __hiloint2double(h + 0x00100000, __double2loint(a)) : 0.0;
+        const uint64_t b = (uint64_t)__double_as_longlong(a), sign = b & 0x8000000000000000ULL;
+        const uint32_t e = (uint32_t)(b >> 52) & 0x7FFu;
+        if (__builtin_expect(e - 1u >= 0x7FDu, 0)) {
+            const uint64_t v = e == 0 ? sign | (b << 1) : (e == 0x7FEu ? sign | 0x7FF0000000000000ULL : b);
+            return __longlong_as_double((long long)v);
+        }
+        return __longlong_as_double((long long)(b + (1ULL << 52)));
     }
     __device__ __forceinline__ double sub(double a, double b) const { return fma(b, mone, a); }
     __device__ __forceinline__ dc mul(dc a, dc b) const {

@@ -146,3 +146,23 @@ def test_one_point_with_F_zero(f0, f1, nord, status):
     ref, got = _status(_Text(TOY.format(f0=f0, f1=f1)), 0, nord, [3.0], 0.0, n=1024, z=[1, 1, 1, 1, 1, 1],
                        transform=2, flags=qmc.QMC_JOB_UNSHIFTED)
     assert got == status and ref == status
+
+
+@pytest.mark.parametrize("s", [9e-39, 9e-40, 9e-42, 9.0])
+def test_mixed_deformed_keeps_fp32_subnormals(s):
+    """F, its derivatives and the contour in FP32's subnormal range: the same
+    FP32 values as in the general kernel, which serves a window up to eps^2."""
+    I = w.bubble(0, "s")
+    g = Gpu(precision=qmc.QMC_PRECISION_MIXED)
+    try:
+        iid = g.load(I)
+        qmc.qmc_set_kinematics(g.ctx, np.array([[s]]))
+        specs = [dict(integral_id=iid, sector=i, point=0, shifts=2, n=1009, seed=3, stream=i, **{"lambda": 0.5 / s})
+                 for i in range(len(I.sectors))]
+        a, fa, ra = g.eval(iid, specs, -1, 3)
+        b, fb, rb = g.eval(iid, specs, -1, 4)
+        assert ra == rb == 0 and fa == fb
+        a, b = a.reshape(-1, 3, 2), b.reshape(-1, 4, 2)[:, :3]
+        assert np.all(np.abs(a - b) <= 1e-11 * np.abs(b).max())
+    finally:
+        g.close()
