@@ -8,7 +8,7 @@
 //   x = 2^e m, m in [1, 2); F = 1 + j/1024 nearest to m (j = 0..1024);
 //   f = (m - F)/F, |f| <= 2^-11, held as f 2^74 in an int64;
 //   log1p(f) = f (1 - f c(f)),  c(f) = 1/2 - f/3 + f^2/4 - f^3/5 + f^4/6
-//     (truncation below 2^-58 relative), c by Horner, each coefficient to
+//     (truncation below 2^-68 relative), c by Horner, each coefficient to
 //     the bits that its weight leaves visible (Q32 inside, Q63 outside);
 //   ln x = e ln2 + ln F + log1p(f), summed in a signed 128-bit Q116 number
 //     (|ln x| < 745 < 2^9.6, and the smallest nonzero result, near x = 1,
@@ -35,8 +35,7 @@
 #define QMC_ILOG_LN2_HI 0xb17217f7d1cf7ULL      //                  high word
 #define QMC_ILOG_C2 0x4000000000000000ULL       // RN(2^63 / k), k = 2, 3
 #define QMC_ILOG_C3 0x2aaaaaaaaaaaaaabULL
-#define QMC_ILOG_C4_32 0x40000000u              // RN(2^32 / k), k = 4, 5, 6
-#define QMC_ILOG_C5_32 0x33333333u
+#define QMC_ILOG_C5_32 0x33333333u              // RN(2^32 / k), k = 5, 6
 #define QMC_ILOG_C6_32 0x2aaaaaabu
 
 typedef unsigned __int128 qmc_u128;
@@ -101,23 +100,24 @@ QMC_HD double qmc_ilog_core(int e, uint64_t frac63, const uint64_t *tab) {
     const uint64_t ra = fneg ? (uint64_t)(-ri) : (uint64_t)ri;
     // |f| 2^74 = |m - F| 2^63 RN(2^63/F) 2^-52 (truncated; exact for F = 1, 2)
     const uint64_t fm = (uint64_t)(((qmc_u128)ra * tab[3 * j]) >> 52);
-    // c(f) by Horner on |f| with the sign of f carried into each sum. c enters
-    // log1p with weight f^2 <= 2^-22 relative, and each inner coefficient with
-    // one more factor 2^-11, so the inner two run in Q32 (c4 within 2^-30),
-    // 1/3 - f c4 in Q63 from a 32 x 32 product (within 2^-42: 2^-64 of
-    // log1p), and only the outer two products take 64 x 64 bits.
+    // c(f) by Horner on |f| with the sign of f carried into each sum (a - b - 1
+    // for a - b: a + ~b). c enters log1p with weight f^2 <= 2^-22 relative, and
+    // each inner coefficient with one more factor 2^-11: f c5 to 2^-42 comes from
+    // a 32 x 32 product of |f| 2^43 and c5 in Q32, f c4 = f/4 - f (f c5) from f's
+    // own bits and another (within 2^-52: 2^-74 of log1p), and only the outer
+    // products take 64 x 64 bits. (With c4 in Q32 log1p kept 2^-64, and some
+    // results in 10^4 lost their rounding.)
+    const uint64_t sm = fneg ? 0ULL : ~0ULL;
     const uint32_t f32 = (uint32_t)(fm >> 31);                    // |f| 2^43
-    const uint32_t t6 = qmc_umulhi32(f32, QMC_ILOG_C6_32) >> 11;
-    const uint32_t c5 = fneg ? QMC_ILOG_C5_32 + t6 : QMC_ILOG_C5_32 - t6;
-    const uint32_t t5 = qmc_umulhi32(f32, c5) >> 11;
-    const uint32_t c4 = fneg ? QMC_ILOG_C4_32 + t5 : QMC_ILOG_C4_32 - t5;
-    const uint64_t t4 = ((uint64_t)f32 * c4) >> 12;
-    const uint64_t c3 = fneg ? QMC_ILOG_C3 + t4 : QMC_ILOG_C3 - t4;
-    const uint64_t t3 = qmc_umulhi64(fm, c3) >> 10;
-    const uint64_t c = fneg ? QMC_ILOG_C2 + t3 : QMC_ILOG_C2 - t3;
-    const uint64_t t2 = qmc_umulhi64(fm, c) >> 10;
-    const uint64_t h = fneg ? (1ULL << 63) + t2 : (1ULL << 63) - t2;   // (1 - f c) 2^63
-    const qmc_u128 lp = ((qmc_u128)fm * h) >> 21;     // |log1p f| 2^116
+    const uint32_t c5 = QMC_ILOG_C5_32 + ((qmc_umulhi32(f32, QMC_ILOG_C6_32) >> 11) ^ (uint32_t)sm);
+    const uint64_t t4 = (fm >> 13) + ((((uint64_t)f32 * qmc_umulhi32(f32, c5)) >> 23) ^ sm);
+    const uint64_t c3 = QMC_ILOG_C3 + (t4 ^ sm);
+    const uint64_t c = QMC_ILOG_C2 + ((qmc_umulhi64(fm, c3) >> 10) ^ sm);
+    // log1p f = f - f^2 c in Q116, |f| c with all the bits of its product (Q73);
+    // for f < 0 the truncated f^2 c is rounded up, so that next to 1, where
+    // f - f^2/2 can be a rounding tie, the terms beyond Q116 still decide it
+    const qmc_u128 f2 = (((qmc_u128)fm * qmc_umulhi64(fm, c)) >> 31) + (fneg ? 1 : 0);
+    const qmc_u128 f1 = (qmc_u128)(__int128)(fneg ? -(int64_t)fm : (int64_t)fm) << 42;
     // |e| RN(2^116 ln 2): |e| < 2^11, four 32-bit words
     const uint32_t ea = (uint32_t)(e < 0 ? -e : e);
     const uint64_t p0 = (uint64_t)ea * (uint32_t)QMC_ILOG_LN2_LO;
@@ -126,7 +126,7 @@ QMC_HD double qmc_ilog_core(int e, uint64_t frac63, const uint64_t *tab) {
     const uint64_t elh = (((uint64_t)ea * (uint32_t)(QMC_ILOG_LN2_HI >> 32)) << 32) + p2;
     const qmc_u128 el = ((qmc_u128)elh << 64) | ((p1 << 32) | (uint32_t)p0);
     const qmc_u128 lf = ((qmc_u128)tab[3 * j + 2] << 64) | tab[3 * j + 1];
-    qmc_u128 S = lf + (fneg ? (qmc_u128)0 - lp : lp) + (e < 0 ? (qmc_u128)0 - el : el);   // mod 2^128
+    qmc_u128 S = lf + f1 - f2 + (e < 0 ? (qmc_u128)0 - el : el);   // mod 2^128
     const bool neg = (uint64_t)(S >> 127) != 0;
     if (neg) S = (qmc_u128)0 - S;
     const uint64_t hi = (uint64_t)(S >> 64), lo = (uint64_t)S;
