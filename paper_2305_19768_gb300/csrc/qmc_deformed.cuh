@@ -22,8 +22,8 @@
 //    M_jj = A_jj + (1 - 2t) / (t (1 - t)) g_j: its minors take one FMA each;
 //  * x^-e enters as conj(x)^e / |x|^2e: the complex products collect in FP64,
 //    the norms as mantissas, whose logarithm is also the corner's Re L; its
-//    Im L is the sum of the factors' principal arguments in fixed point (an
-//    integer arctangent), so that no branch has to be restored;
+//    Im L is the sum of the factors' principal arguments, in 128-bit fixed point
+//    (an integer arctangent), so that no branch has to be restored;
 //  * transform, weight, the real factors of the deformation, 1/t, ln t,
 //    reciprocals, logarithms and arguments run on the integer pipe (an FP64
 //    negation or doubling by itself takes the FP64 pipe too: both go through
@@ -41,7 +41,7 @@
 
 struct alignas(16) FdShared {
     uint64_t logtab[3 * QMC_LOG_TABLE_ROWS + 1];
-    int64_t atan60[QMC_ATAN_TABLE_ROWS];   // atan(j / 64) 2^60
+    int64_t atan63[QMC_ATAN_TABLE_ROWS];   // atan(j / 64) 2^63
     uint32_t exps[QMC_MAXMONO];      // FP64: variables in slot order (singular first)
     uint4 mdesc[QMC_MAXMONO];        // MIXED: factors as in FxShared, original variable order
     double cval[QMC_MAXMONO];
@@ -93,51 +93,15 @@ __device__ __noinline__ double fd_half_log(FxM x) {
     return fx_half(qmc_ilog_xf(qmc_xf{x.m, x.e, 0}, fd_shared().logtab));
 }
 
-// Argument of x + i y times 2^60 in fixed point, in (-pi, pi]; with m0 a zero
-// y counts as -0 (the prescription F - i0). The reduction of qatan2: with
-// mn <= mx the smaller and larger of |x|, |y| and c = j/64 nearest mn/mx,
-// atan(mn/mx) = atan(c) + atan(d), d = (mn - c mx) / (mx + c mn), |d| <= 2^-7,
-// and atan(d) = d - d^3 (1/3 - d^2 (1/5 - d^2 / 7)) (truncation below 2^-66);
-// the inner coefficients in 32 bits. Absolute error a few 2^-60. Out of line.
-__device__ __noinline__ int64_t fd_arg(double y, double x, bool m0) {
-    const qmc_xf ax = qmc_xf_of(x), ay = qmc_xf_of(y);
-    const bool sw = ay.e > ax.e || (ay.e == ax.e && ay.m > ax.m);
-    const uint64_t mx = sw ? ay.m : ax.m, ms = sw ? ax.m : ay.m;
-    const int dd = sw ? ay.e - ax.e : ax.e - ay.e;
-    int64_t r = 0;
-    if (mx != 0 && ms != 0 && dd < 64) {
-        const uint64_t mn = ms >> dd;                  // both in units of mx's last place
-        int j = 0;
-        if (dd <= 7) {
-            const float fs = __int_as_float(0x3F800000 | (int)((ms >> 40) & 0x7FFFFFu));
-            const float fx = __int_as_float(0x3F800000 | (int)((mx >> 40) & 0x7FFFFFu));
-            j = min(__float2int_rn(__fdividef(fs, fx) * __int_as_float((133 - dd) << 23)), 64);
-        }
-        const int64_t num = (int64_t)((mn << 6) - (uint64_t)j * mx);      // 64 (mn - c mx)
-        const uint64_t an = (uint64_t)(num < 0 ? -num : num);
-        const FxM den = fx_norm(FxM{(mx >> 1) + __umul64hi(mn, (uint64_t)j << 57), 0});   // (mx + c mn) / 2
-        const FxM q = fd_rcp(FxM{den.m, 0});           // 2^63 / den.m
-        const uint64_t d = __umul64hi(an, q.m) << (q.e + 1 - den.e);      // |d| 2^70
-        const uint64_t z = __umul64hi(d, d);           // d^2 2^76
-        const uint32_t z45 = (uint32_t)(z >> 31);
-        const uint32_t c5 = 0x33333333u - (__umulhi(z45, 0x24924925u) >> 13);
-        const uint64_t c3 = 0x2AAAAAAAAAAAAAABULL - (((uint64_t)z45 * c5) >> 14);
-        const uint64_t at = (d >> 10) - (__umul64hi(__umul64hi(d, z), c3) >> 21);
-        r = fd_shared().atan60[j] + (num < 0 ? -(int64_t)at : (int64_t)at);
-    }
-    if (sw) r = 0x1921FB54442D1847LL - r;
-    if (ax.neg) r = 0x3243F6A8885A308DLL - r;
-    return (ay.neg || (m0 && ay.m == 0)) ? -r : r;
+// sum + k arg(x + i y), |k| <= 4 (qmc_iarg.h). Out of line. In 64-bit fixed point
+// (2^-57) a nearly real integrand's imaginary part, a sum of small arguments, had
+// fewer bits than FP64 has.
+__device__ __noinline__ qmc_u128 fd_addarg(qmc_u128 sum, double y, double x, int k, bool m0) {
+    return qmc_iarg_add(sum, qmc_iarg(y, x, m0, fd_shared().atan63), k);
 }
 // -x or x on the sign bit (a negation by itself takes the FP64 pipe)
 __device__ __forceinline__ double fd_signed(double x, bool neg) {
     return __hiloint2double(__double2hiint(x) ^ (neg ? (int)0x80000000 : 0), __double2loint(x));
-}
-// a 2^-57 as FP64
-__device__ __forceinline__ double fd_from57(int64_t a) {
-    const uint64_t u = (uint64_t)(a < 0 ? -a : a);
-    if (u == 0) return 0.0;
-    return fd_signed(fx_pack(fx_norm(FxM{u, 6})), a < 0);
 }
 
 // FP32 <-> FP64 conversions on the integer pipe (RN; subnormals, infinities and
@@ -473,11 +437,11 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
     // F^f0, a factor x^-e as conj(x)^e / |x|^2e: B collects the complex
     // products and q the real ones, in mantissas. Its exponent
     // L = sum of e ln x over rho^b, z^b, U^u1, F^f1: ln |x|^2 of the product
-    // of norms in mantissas, and the principal arguments in fixed point.
+    // of norms in mantissas, and the sum of the principal arguments.
     FdCorner out;
     dc B = J;
     FxM den{1ULL << 63, 0}, np{1ULL << 63, 0}, nn{1ULL << 63, 0};
-    int64_t arg = 0;
+    qmc_u128 arg = 0;
     auto factor = [&](dc x, FxM n, int e0, int e1, bool m0) {
         if (e0) {
             B = fd_mulpow(B, x, e0);
@@ -486,7 +450,7 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
         if (lam && e1) {
             if (e1 > 0) np = fd_mulnorm(np, n, e1);
             else nn = fd_mulnorm(nn, n, -e1);
-            arg += (int64_t)e1 * (fd_arg(x.im, x.re, m0) >> 3);
+            arg = fd_addarg(arg, x.im, x.re, e1, m0);
         }
     };
 #pragma unroll
@@ -512,7 +476,7 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
     out.B = B;
     out.q = fd_rcp(den);
     out.L = dc{0.0, 0.0};
-    if constexpr (lam) out.L = dc{fd_half_log(fx_norm(fx_mul(np, fd_rcp(nn)))), fd_from57(arg)};
+    if constexpr (lam) out.L = dc{fd_half_log(fx_norm(fx_mul(np, fd_rcp(nn)))), qmc_iarg_sum(arg)};
     return out;
 }
 
@@ -835,7 +799,7 @@ __global__ void __launch_bounds__(BLOCK, fd_min_units<MIXED, HI>() * 128 / BLOCK
     }
     for (int i = threadIdx.x; i < 3 * QMC_LOG_TABLE_ROWS; i += BLOCK) S.logtab[i] = kLogTable[i];
     for (int i = threadIdx.x; i < QMC_ATAN_TABLE_ROWS; i += BLOCK)
-        S.atan60[i] = __double2ll_rn(kAtanTable[2 * i] * 0x1p60) + __double2ll_rn(kAtanTable[2 * i + 1] * 0x1p60);
+        S.atan63[i] = __double2ll_rn(kAtanTable[2 * i] * 0x1p63) + __double2ll_rn(kAtanTable[2 * i + 1] * 0x1p63);
     for (;;) {
         __syncthreads();  // previous tile fully consumed
         if (threadIdx.x == 0) {

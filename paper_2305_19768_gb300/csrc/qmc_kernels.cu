@@ -27,6 +27,7 @@
 #include "qmc_ilog.h"
 #include "qmc_internal.h"
 #include "qmc_log_table.h"
+#include "qmc_iarg.h"
 #include "qmc_xf.h"
 
 #ifndef QMC_PART

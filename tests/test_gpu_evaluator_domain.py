@@ -166,3 +166,28 @@ def test_mixed_deformed_keeps_fp32_subnormals(s):
         assert np.all(np.abs(a - b) <= 1e-11 * np.abs(b).max())
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("lam", [1e-3, 1e-6, 1e-9])
+def test_imaginary_parts_of_nearly_real_sums(lam):
+    """With a small lambda at Euclidean kinematics every argument is small and
+    the sums' imaginary parts are proportional to it: the same relative accuracy
+    as the general kernel's. Six points a sum, so that neither the corners nor the
+    points cancel by more than 10^3: some 10^3 2^-53 each side, bar 1e-11."""
+    I, lo, kin = w.box_massless(deform=True), -2, [-3.0, -2.0]
+    g = Gpu()
+    try:
+        iid, gid = g.load(I), g.load(general(I, Fraction(1, 10 ** 250)))
+        qmc.qmc_set_kinematics(g.ctx, np.array([kin]))
+        specs = [dict(integral_id=iid, sector=s, point=0, shifts=1, n=7, z=[1, 2, 3, 1, 1, 1], seed=3, stream=s,
+                      flags=qmc.QMC_JOB_UNSHIFTED, **{"lambda": lam}) for s in range(len(I.sectors))]
+        for hi in (0, 1):
+            nord = hi - lo + 1
+            a, _, ra = g.eval(iid, specs, lo, nord)
+            b, _, rb = g.eval(gid, [dict(sp, integral_id=gid) for sp in specs], lo, nord)
+            assert ra == rb == 0
+            a, b = a.reshape(-1, nord, 2)[..., 1], b.reshape(-1, nord, 2)[..., 1]
+            top = np.abs(b).max(axis=0)
+            assert top[-1] > 0 and np.all(np.abs(a - b) <= 1e-11 * top), np.abs(a - b).max(axis=0) / top
+    finally:
+        g.close()
