@@ -905,10 +905,8 @@ template <bool MIXED, int BLOCK> constexpr int fd_dyn_smem(int prow) {
 }
 
 template <bool MIXED, int BLOCK, int HI> bool fd_allow() {
-    static const bool ok = cudaFuncSetAttribute(qmc_deformed_kernel<MIXED, BLOCK, HI>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                fd_dyn_smem<MIXED, BLOCK>(QMC_EMAX)) == cudaSuccess;
-    return ok;
+    static std::atomic<uint64_t> done{0};
+    return qmc_allow_smem(done, qmc_deformed_kernel<MIXED, BLOCK, HI>, fd_dyn_smem<MIXED, BLOCK>(QMC_EMAX));
 }
 
 template <bool MIXED, int BLOCK, int HI>

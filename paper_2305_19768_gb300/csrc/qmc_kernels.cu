@@ -27,6 +27,7 @@
 #include "qmc_ilog.h"
 #include "qmc_internal.h"
 #include "qmc_log_table.h"
+#include "qmc_device_once.h"
 #include "qmc_iarg.h"
 #include "qmc_xf.h"
 
@@ -3080,10 +3081,8 @@ constexpr int eval_dyn_smem(int block, int prow) {
 template <int DMAX, int SMAX, int LMAX, bool CPLX, bool MIXED, int BLOCK, bool HS, bool FIX>
 bool allow_dyn_smem() {
     constexpr int dmax = eval_dyn_smem<DMAX, CPLX, HS, FIX>(BLOCK, QMC_EMAX);
-    static const bool ok =
-        dmax == 0 || cudaFuncSetAttribute(qmc_eval_kernel<DMAX, SMAX, LMAX, CPLX, MIXED, BLOCK, HS, FIX>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, dmax) == cudaSuccess;
-    return ok;
+    static std::atomic<uint64_t> done{0};
+    return dmax == 0 || qmc_allow_smem(done, qmc_eval_kernel<DMAX, SMAX, LMAX, CPLX, MIXED, BLOCK, HS, FIX>, dmax);
 }
 
 template <int DMAX, int SMAX, int LMAX, bool CPLX, bool MIXED, int BLOCK, bool HS, bool FIX>

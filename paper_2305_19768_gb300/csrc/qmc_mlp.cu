@@ -30,6 +30,7 @@
 
 #include "../../include/qmc.h"
 
+#include "qmc_device_once.h"
 #include "qmc_internal.h"
 
 #define QMC_E_INVAL_LOCAL QMC_E_INVAL
@@ -333,9 +334,8 @@ bool gemm_shape_ok(const void *A, const void *B, int M, int N, int K) {
 // The product's splits, split s at out + s M N
 int gemm_launch(const void *A, const void *B, float *out, int M, int N, int K, int splits, int per, unsigned *err_dev,
                 cudaStream_t stream, unsigned wait_limit) {
-    static const bool attr_set = cudaFuncSetAttribute(qmc_gemm_bf16_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      kGemmSmem) == cudaSuccess;
-    if (!attr_set) return -1;
+    static std::atomic<uint64_t> done{0};
+    if (!qmc_allow_smem(done, qmc_gemm_bf16_tc, kGemmSmem)) return -1;
     CUtensorMap mapA, mapB;
     if (!make_map(&mapA, A, M, K, kTileM) || !make_map(&mapB, B, N, K, N)) return -1;
     qmc_gemm_bf16_tc<<<dim3(M / kTileM, splits), kGemmThreads, kGemmSmem, stream>>>(

@@ -982,10 +982,9 @@ constexpr int fx_dyn_smem(int prow, bool mixed) {
 
 template <int DMAX, int SMAX, int LMAX, bool MIXED, int BLOCK, int HI>
 bool fx_allow() {
-    static const bool ok = cudaFuncSetAttribute(qmc_real_kernel<DMAX, SMAX, LMAX, MIXED, BLOCK, HI>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                fx_dyn_smem<DMAX, BLOCK>(QMC_EMAX, MIXED)) == cudaSuccess;
-    return ok;
+    static std::atomic<uint64_t> done{0};
+    return qmc_allow_smem(done, qmc_real_kernel<DMAX, SMAX, LMAX, MIXED, BLOCK, HI>,
+                          fx_dyn_smem<DMAX, BLOCK>(QMC_EMAX, MIXED));
 }
 
 // One block size per kernel: the tile's points over its threads, whatever
