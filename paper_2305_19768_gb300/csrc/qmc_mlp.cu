@@ -340,7 +340,7 @@ int gemm_launch(const void *A, const void *B, float *out, int M, int N, int K, i
     if (!make_map(&mapA, A, M, K, kTileM) || !make_map(&mapB, B, N, K, N)) return -1;
     qmc_gemm_bf16_tc<<<dim3(M / kTileM, splits), kGemmThreads, kGemmSmem, stream>>>(
         mapA, mapB, out, N, K, per, (size_t)M * N, err_dev, wait_limit);
-    return 0;
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 }  // namespace
 
@@ -445,11 +445,15 @@ struct Splits {
     __device__ __forceinline__ float at(size_t i) const { return split_sum(W, n, stride, i); }
 };
 constexpr int kTile = 32, kTileRows = 8;
-// f(b, o) -> value, stored bf16 as hb [Bp][N] and, through the tile, hbT [N][Bp]
+// f(b, o) -> value, stored bf16 as hb [Bp][N] and, through the tile, hbT [N][Bp];
+// one block per tile, the columns' tiles of 32 rows side by side (a grid's
+// first dimension alone has room for more than two million rows)
 template <class F>
 __device__ __forceinline__ void tile_both(int Bp, int N, __nv_bfloat16 *hb, __nv_bfloat16 *hbT, F f) {
     __shared__ __nv_bfloat16 tile[kTile][kTile + 2];
-    const int o = blockIdx.x * kTile + threadIdx.x, b0 = blockIdx.y * kTile;
+    const int across = (N + kTile - 1) / kTile;
+    const int o0 = blockIdx.x % across * kTile, b0 = blockIdx.x / across * kTile;
+    const int o = o0 + threadIdx.x;
 #pragma unroll
     for (int r = 0; r < kTile; r += kTileRows) {
         const int b = b0 + threadIdx.y + r;
@@ -463,7 +467,7 @@ __device__ __forceinline__ void tile_both(int Bp, int N, __nv_bfloat16 *hb, __nv
     const int bt = b0 + threadIdx.x;
 #pragma unroll
     for (int r = 0; r < kTile; r += kTileRows) {
-        const int ot = blockIdx.x * kTile + threadIdx.y + r;
+        const int ot = o0 + threadIdx.y + r;
         if (bt < Bp && ot < N) hbT[(size_t)ot * Bp + bt] = tile[threadIdx.x][threadIdx.y + r];
     }
 }
@@ -746,7 +750,9 @@ int mlp_gemm(qmc_mlp *m, const void *A, const void *B, int M, int N, int K, Spli
     out = Splits{m->ws, splits, (size_t)M * N};
     return gemm_launch(A, B, m->ws, M, N, K, splits, per, m->err, m->stream, kWaitLimit);
 }
-inline dim3 tiles(int N, int Bp) { return dim3((N + kTile - 1) / kTile, (Bp + kTile - 1) / kTile); }
+inline unsigned tiles(int N, int Bp) { return (unsigned)((N + kTile - 1) / kTile) * (unsigned)((Bp + kTile - 1) / kTile); }
+// whether the launch before was accepted (asked at each: a later call may clear the error)
+inline bool launched() { return cudaGetLastError() == cudaSuccess; }
 
 // forward for Bp rows already in m->x; output in m->out [Bp][No]
 int mlp_forward_dev(qmc_mlp *m, int Bp) {
@@ -756,14 +762,14 @@ int mlp_forward_dev(qmc_mlp *m, int Bp) {
     mlp_layer0_fwd<<<tiles(H, Bp), tb, 0, m->stream>>>(m->x, m->params + m->offW[0], m->params + m->offb[0], m->nin, H,
                                                        Bp, m->hf[0], m->hb[0], m->hbT[0]);
     for (int l = 1; l < m->D; ++l) {
-        if (mlp_gemm(m, m->hb[l - 1], m->Wb[l], Bp, H, H, C)) return -1;
+        if (!launched() || mlp_gemm(m, m->hb[l - 1], m->Wb[l], Bp, H, H, C)) return -1;
         mlp_bias_tanh<<<tiles(H, Bp), tb, 0, m->stream>>>(C, m->params + m->offb[l], H, Bp, m->hf[l], m->hb[l],
                                                           m->hbT[l]);
     }
-    if (mlp_gemm(m, m->hb[m->D - 1], m->Wb[m->D], Bp, m->Nop, H, C)) return -1;
+    if (!launched() || mlp_gemm(m, m->hb[m->D - 1], m->Wb[m->D], Bp, m->Nop, H, C)) return -1;
     mlp_bias_out<<<nblk((size_t)Bp * m->No), 256, 0, m->stream>>>(C, m->params + m->offb[m->D], m->No, m->Nop, Bp,
                                                                  m->out);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return launched() ? 0 : -1;
 }
 
 // loss (into *loss_dst) and gradients (into m->grads) for Bp rows with x, y, mask, wt in place
@@ -775,10 +781,10 @@ int mlp_backward_dev(qmc_mlp *m, int Bp, int B, double *loss_dst) {
     mlp_loss<<<tiles(Nop, Bp), tb, 0, m->stream>>>(m->out, m->y, m->wt, m->mask, No, Nop, Bp, 1.f / B, m->dob, m->dobT,
                                                    m->dof, loss_dst);
     // output layer: dWout^T = h_{D-1}^T dout  ([H][Nop]), dbout, dh = dout Wout
-    if (mlp_gemm(m, m->hbT[D - 1], m->dobT, H, Nop, Bp, C)) return -1;
+    if (!launched() || mlp_gemm(m, m->hbT[D - 1], m->dobT, H, Nop, Bp, C)) return -1;
     mlp_untranspose<<<nblk((size_t)No * H), 256, 0, m->stream>>>(C, H, Nop, No, m->grads + m->offW[D]);
     mlp_colsum<<<(No + kCols - 1) / kCols, kColThreads, 0, m->stream>>>(m->dof, No, Nop, Bp, m->grads + m->offb[D]);
-    if (mlp_gemm(m, m->dob, m->WbT[D], Bp, H, Nop, C)) return -1;
+    if (!launched() || mlp_gemm(m, m->dob, m->WbT[D], Bp, H, Nop, C)) return -1;
     for (int l = D - 1; l >= 0; --l) {
         mlp_tanh_bwd<<<tiles(H, Bp), tb, 0, m->stream>>>(C, m->hf[l], H, Bp, m->dzb, m->dzbT, m->dz);
         mlp_colsum<<<H / kCols, kColThreads, 0, m->stream>>>(m->dz, H, H, Bp, m->grads + m->offb[l]);
@@ -787,13 +793,13 @@ int mlp_backward_dev(qmc_mlp *m, int Bp, int B, double *loss_dst) {
                                                                            m->grads + m->offW[0]);
         } else {
             // dW_l = dz^T h_{l-1}  ([H][H]); dh_{l-1} = dz W_l
-            if (mlp_gemm(m, m->dzbT, m->hbT[l - 1], H, H, Bp, C)) return -1;
+            if (!launched() || mlp_gemm(m, m->dzbT, m->hbT[l - 1], H, H, Bp, C)) return -1;
             qmc_gemm_splitk_sum<<<nblk((size_t)H * H), 256, 0, m->stream>>>(C.W, C.n, C.stride, m->grads + m->offW[l],
                                                                            C.stride);
-            if (mlp_gemm(m, m->dzb, m->WbT[l], Bp, H, H, C)) return -1;
+            if (!launched() || mlp_gemm(m, m->dzb, m->WbT[l], Bp, H, H, C)) return -1;
         }
     }
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return launched() ? 0 : -1;
 }
 
 // stage a host batch (B rows) padded to Bp rows
