@@ -207,8 +207,12 @@ int qmc_set_kinematics(qmc_ctx *ctx, const double *inv, int npoints, int ninv);
  * table, sizes the tile queue and partial-sum scratch, and picks the kernel
  * class of every job. Each job yields per-shift estimates of the eps orders
  * lo .. lo+norders-1 of its sector integral (orders below the sector's
- * leading pole are 0). *out owns its device buffers; destroy with
- * qmc_plan_destroy (or with the context). Errors: QMC_E_INVAL, QMC_E_CUDA. */
+ * leading pole are 0). A lattice is summed in tiles whose size follows from the
+ * lattice sizes and shifts of all jobs of the plan (options.ppt, if not 0, fixes
+ * the points per thread): one job gives the same bits in every run of a
+ * plan, and in two plans sums that agree to rounding. *out owns its device
+ * buffers; destroy with qmc_plan_destroy (or with the context).
+ * Errors: QMC_E_INVAL, QMC_E_CUDA. */
 int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int norders,
                     qmc_plan **out);
 
@@ -466,7 +470,8 @@ int qmc_stats(qmc_ctx *ctx, double *evaluations, double *seconds);
  * buffer of n doubles in place over all ranks (the per-shift sums, sign-check
  * flags and timings of the pass, zeros where another rank evaluated), so that
  * every rank holds the same statistics and takes the same allocation
- * decisions: the results equal a one-rank call bit for bit. The callback
+ * decisions, and each rank's tiles follow from the jobs of the whole pass: the
+ * results equal a one-rank call bit for bit. The callback
  * returns 0 on success; it is called the same number of times on every rank.
  * world = 1 (or allreduce = NULL) restores single-rank integration. */
 typedef int (*qmc_allreduce_fn)(void *user, double *buf, size_t n);

@@ -131,3 +131,10 @@ struct qmc_plan {
 
 // Record `fmt` as the context's last error and return `code`.
 int qmc_fail(qmc_ctx *ctx, int code, const char *fmt, ...);
+
+// qmc_plan_create for a rank's share of a pass: the plan of the jobs with
+// mine[i] != 0 (all of them if mine is null), its outputs in their order, with
+// tiles chosen from all jobs. The order of summation follows from the tiles, so
+// that a job's sums are the same bits whichever rank evaluates it.
+int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsigned char *mine, int lo, int norders,
+                      qmc_plan **out);

@@ -414,13 +414,12 @@ bool fx_job_ok(const qmc_ctx *ctx, const HostSector &S, int cls, int point) {
 
 // Points per thread of a launch by qmc_real.cuh or qmc_deformed.cuh: the
 // estimate (waves of `resident` tiles) x (points + setup), for a tile's
-// staging and lattice set-up, over the tiles that the lattices' sizes give.
+// staging and lattice set-up, over the tiles that the lattices (shifts of each
+// size) give.
 // Few tiles: small ones, so that every SM works (one shift of a pilot lattice
 // would otherwise keep a few blocks busy for 16 points a thread); many: the
 // size that leaves the fewest threads of the last tile of a lattice idle.
-int fx_points_per_thread(const std::vector<QmcJobDev> &jobs, int block, uint64_t resident) {
-    std::map<uint64_t, uint64_t> shifts;             // lattice size -> shifts
-    for (const QmcJobDev &D : jobs) shifts[D.n] += (uint64_t)D.shifts;
+int fx_points_per_thread(const std::map<uint64_t, uint64_t> &shifts, int block, uint64_t resident) {
     int best = 1;
     double best_cost = 0.0;
     // the d <= 6 blocks are large, and warps that finish a tile early wait for
@@ -647,6 +646,13 @@ int qmc_set_kinematics(qmc_ctx *ctx, const double *inv, int npoints, int ninv) {
 }
 
 int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int norders, qmc_plan **out) {
+    return plan_create_share(ctx, jobs, njobs, nullptr, lo, norders, out);
+}
+
+}  // extern "C"
+
+int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsigned char *mine, int lo, int norders,
+                      qmc_plan **out) {
     if (!ctx || !out || (njobs > 0 && !jobs) || njobs < 0 || norders < 1)
         return fail(ctx, QMC_E_INVAL, "qmc_plan_create: bad arguments");
     *out = nullptr;
@@ -657,6 +663,13 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
     // those of the evaluators of qmc_real.cuh and qmc_deformed.cuh
     std::vector<std::vector<QmcJobDev>> per(2 * QMC_NCLASS);
     std::vector<std::vector<int>> per_orig(2 * QMC_NCLASS);
+    // what the tiles are chosen from, over all jobs: the shifts of each lattice
+    // size, and the power-table rows (the largest exponent among the sectors:
+    // fewer rows, less shared memory per block, more resident blocks)
+    std::vector<std::map<uint64_t, uint64_t>> lattices(2 * QMC_NCLASS);
+    std::vector<int> prows(2 * QMC_NCLASS, 1);
+    std::vector<int> own(njobs, -1);   // index among the plan's jobs
+    int nown = 0;
     uint64_t out_off = 0;
     double evals = 0.0;
     for (int i = 0; i < njobs; ++i) {
@@ -694,6 +707,11 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         if (norders > qmc_class_lmax(cls) || hi + S.ns + 1 > qmc_class_lmax(cls))
             return fail(ctx, QMC_E_INVAL, "job %d: orders %d..%d with %d poles exceed the evaluator's series length %d",
                         i, lo, hi, S.ns, qmc_class_lmax(cls));
+        const int slot = 2 * cls + (fx_order_ok(hi, cls) && (fd_job_ok(S, cls) || fx_job_ok(ctx, S, cls, J.point)) ? 1 : 0);
+        lattices[slot][J.n] += (uint64_t)J.shifts;
+        prows[slot] = std::max(prows[slot], S.prow);
+        if (mine && !mine[i]) continue;
+        own[i] = nown++;
         QmcJobDev D{};
         D.sector = S.global_index;
         D.point = I.invariants.empty() ? 0 : J.point;
@@ -709,7 +727,6 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         D.flags = J.flags & QMC_JOB_UNSHIFTED;
         out_off += (uint64_t)J.shifts * norders * 2;
         evals += (double)J.n * J.shifts;
-        const int slot = 2 * cls + (fx_order_ok(hi, cls) && (fd_job_ok(S, cls) || fx_job_ok(ctx, S, cls, J.point)) ? 1 : 0);
         per[slot].push_back(D);
         per_orig[slot].push_back(i);
     }
@@ -717,7 +734,7 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
     p->ctx = ctx;
     p->lo = lo;
     p->norders = norders;
-    p->njobs = njobs;
+    p->njobs = nown;
     p->out_size = (size_t)out_off;
     p->evals = evals;
     auto bail = [&](int rc) {
@@ -762,32 +779,25 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
         }
         ClassLaunch c;
         c.cls = cls;
-        c.orig = per_orig[slot];
+        for (int u : per_orig[slot]) c.orig.push_back(own[u]);
         c.fx = (slot & 1) != 0;
         if (c.fx && cls != QMC_CLASS_CPLX3 && cls != QMC_CLASS_CPLX3M)
-            for (int u : c.orig) c.fx_jobs.push_back({jobs[u].integral_id, jobs[u].sector, jobs[u].point});
+            for (int u : per_orig[slot]) c.fx_jobs.push_back({jobs[u].integral_id, jobs[u].sector, jobs[u].point});
         c.block = ctx->opt.block == 256 ? 256 : (ctx->opt.block == 128 ? 128 : (ctx->tuned_block[cls] ? ctx->tuned_block[cls] : 128));
         if (qmc_class_dmax(cls) > 3) c.block = 128;   // the d <= 6 classes exist with 128-thread blocks only
         c.ppt = ctx->opt.ppt > 0 ? ctx->opt.ppt : (ctx->tuned_ppt[cls] ? ctx->tuned_ppt[cls] : 16);
         if (ctx->opt.ppt <= 0 && !ctx->tuned_ppt[cls]) {
             // small lattices: tiles of 512 points instead of 2048, so that a
             // lattice of a few thousand points does not leave most threads idle
-            uint64_t nmax = 0;
-            for (const QmcJobDev &D : v) nmax = std::max<uint64_t>(nmax, D.n);
-            if (nmax < 16384) c.ppt = 4;
+            if (lattices[slot].rbegin()->first < 16384) c.ppt = 4;
         }
-        // power-table rows: the largest exponent among the launch's sectors
-        // (fewer rows, less shared memory per block, more resident blocks)
-        int prow = 1, occ = 1;
-        for (int u : c.orig) {
-            const qmc_job &J = jobs[u];
-            prow = std::max(prow, ctx->integrals[J.integral_id].sectors[J.sector].prow);
-        }
+        const int prow = prows[slot];
+        int occ = 1;
         if (c.fx) {
             c.block = qmc_class_dmax(cls) > 3 ? QMC_FX6_BLOCK : QMC_FX3_BLOCK;   // their one block size
             occ = std::max(1, qmc_k_occupancy_real(cls, hi, prow));
             if (ctx->opt.ppt <= 0 && !ctx->tuned_ppt[cls])
-                c.ppt = fx_points_per_thread(v, c.block, (uint64_t)ctx->sm_count * occ);
+                c.ppt = fx_points_per_thread(lattices[slot], c.block, (uint64_t)ctx->sm_count * occ);
         } else {
             occ = std::max(1, qmc_k_occupancy(cls, c.block, prow));
         }
@@ -886,6 +896,8 @@ int qmc_plan_create(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int no
     *out = p;
     return QMC_OK;
 }
+
+extern "C" {
 
 size_t qmc_plan_output_size(const qmc_plan *plan) { return plan ? plan->out_size : 0; }
 

@@ -389,11 +389,12 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
     std::vector<double> tau(slots.size(), 1.0);
     std::vector<double> amp_val((size_t)npts * namp * norders * 2), amp_var((size_t)npts * namp * norders);
     std::vector<double> amp_vre((size_t)npts * namp * norders), amp_vim((size_t)npts * namp * norders);
-    // evaluate host jobs (this rank's share): the caller's evaluator or one GPU
-    // plan; per-shift sums, per-job sign-check failures, evaluator seconds per
-    // class (slot QMC_NCLASS: one figure for all classes, from an evaluator
-    // that is not timed per class)
-    auto eval_jobs = [&](const std::vector<qmc_job> &jobs, std::vector<double> &out, std::vector<uint32_t> &fails,
+    // evaluate host jobs (this rank's share of `all`, whose members are marked in
+    // `own`): the caller's evaluator or one GPU plan; per-shift sums, per-job
+    // sign-check failures, evaluator seconds per class (slot QMC_NCLASS: one
+    // figure for all classes, from an evaluator that is not timed per class)
+    auto eval_jobs = [&](const std::vector<qmc_job> &all, const std::vector<unsigned char> &own,
+                         const std::vector<qmc_job> &jobs, std::vector<double> &out, std::vector<uint32_t> &fails,
                          std::vector<double> &cls_s) -> int {
         out.assign(jobs.size() * (size_t)m * sn * 2, 0.0);
         fails.assign(jobs.size(), 0);
@@ -409,7 +410,7 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
             return QMC_OK;
         }
         qmc_plan *plan = nullptr;
-        int rc = qmc_plan_create(ctx, jobs.data(), (int)jobs.size(), slo, sn, &plan);
+        int rc = plan_create_share(ctx, all.data(), (int)all.size(), own.data(), slo, sn, &plan);
         if (rc) return rc;
         rc = qmc_plan_run(plan, nullptr, nullptr);
         uint64_t sf = 0;
@@ -445,11 +446,11 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
         std::vector<double> cost(todo.size());
         for (size_t u = 0; u < todo.size(); ++u) cost[u] = (double)slots[todo[u]].n * slots[todo[u]].cost;
         const std::vector<int> owner = partition(cost);
-        std::vector<qmc_job> jobs;
+        std::vector<qmc_job> all, jobs;
+        std::vector<unsigned char> own;
         std::vector<size_t> mine;
         std::vector<uint32_t> cand;
         for (size_t u = 0; u < todo.size(); ++u) {
-            if (owner[u] != rank) continue;
             const size_t q = todo[u];
             const Slot &sl = slots[q];
             const int d = ctx->integrals[ids[sl.i]].sectors[sl.s].d;
@@ -468,8 +469,11 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
                     J.lambda[j] = sl.lambda;
                     J.z[j] = zc[(size_t)c * 6 + j];
                 }
-                jobs.push_back(J);
+                all.push_back(J);
+                own.push_back(owner[u] == rank);
+                if (owner[u] == rank) jobs.push_back(J);
             }
+            if (owner[u] != rank) continue;
             mine.push_back(u);
             cand.insert(cand.end(), zc.begin(), zc.end());
         }
@@ -485,7 +489,7 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
                 if (rc && rc != QMC_E_SIGN_CHECK) return fail(ctx, rc, "qmc_integrate: the evaluator failed (%d)", rc);
             } else {
                 qmc_plan *plan = nullptr;
-                int rc = qmc_plan_create(ctx, jobs.data(), (int)jobs.size(), slo, sn, &plan);
+                int rc = plan_create_share(ctx, all.data(), (int)all.size(), own.data(), slo, sn, &plan);
                 if (rc) return rc;
                 rc = qmc_plan_run(plan, nullptr, nullptr);
                 if (!rc) rc = qmc_plan_results(plan, est.data(), nullptr);
@@ -539,10 +543,10 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
                 std::vector<double> cost(dirty.size());
                 for (size_t u = 0; u < dirty.size(); ++u) cost[u] = (double)slots[dirty[u]].n * slots[dirty[u]].cost;
                 const std::vector<int> owner = partition(cost);
-                std::vector<qmc_job> jobs;
+                std::vector<qmc_job> all, jobs;
+                std::vector<unsigned char> own;
                 std::vector<size_t> mine;
                 for (size_t u = 0; u < dirty.size(); ++u) {
-                    if (owner[u] != rank) continue;
                     const size_t q = dirty[u];
                     Slot &sl = slots[q];
                     qmc_job J = job_for(q);
@@ -554,12 +558,15 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
                         J.lambda[j] = sl.lambda;
                         J.z[j] = median ? sl.z[j] : 0;
                     }
+                    all.push_back(J);
+                    own.push_back(owner[u] == rank);
+                    if (owner[u] != rank) continue;
                     jobs.push_back(J);
                     mine.push_back(u);
                 }
                 std::vector<double> out, cls_s;
                 std::vector<uint32_t> fails;
-                int rc = eval_jobs(jobs, out, fails, cls_s);
+                int rc = eval_jobs(all, own, jobs, out, fails, cls_s);
                 if (rc) return rc;
                 double own_evals = 0.0;
                 for (const qmc_job &J : jobs) own_evals += (double)J.n * J.shifts;
