@@ -62,7 +62,10 @@ typedef struct {
 typedef struct {
     int shifts;            /* m random shifts per lattice [32] */
     uint64_t seed;         /* seed of the shift streams [1] */
-    int block;             /* threads per block of the evaluator, 128 or 256 [autotuned] */
+    int block;             /* threads per block of the general evaluators, 128 or 256 [autotuned];
+                              128 for d > 3. The evaluators for real sectors with non-negative
+                              coefficients and for deformed sectors (integer exponents, sums up to
+                              eps^0, for d <= 3 eps^1) have one block size: 256, 384 for d > 3 */
     int ppt;               /* lattice points per thread [autotuned] */
     uint64_t min_points;   /* smallest lattice (pilot pass) [10000] */
     uint64_t max_points;   /* largest lattice qmc_integrate may use [largest tabulated] */
@@ -293,11 +296,13 @@ int qmc_presample_lambda(qmc_ctx *ctx, qmc_job *jobs, int njobs, int lo, int nor
  * mixed-precision variant, 11: real d <= 6 with exponents a_j <= -2, 12:
  * deformed d <= 3 with exponents a_j <= -2; class 2 then holds the d <= 6
  * sectors with 4): on up to 32 of the
- * given jobs per class (at most 8 shifts each) every block size in
- * {128, 256} and points per thread in {1, 2, 4, 8, 16, 32} is timed with CUDA
- * events; the fastest is kept in the context and used by later plans whose
- * options leave block/ppt at 0. best_block/best_ppt (may be NULL) receive
- * QMC_NUM_CLASSES entries (0 = class absent). */
+ * given jobs per class (at most 8 shifts each) every block size that their
+ * evaluators have (128 and 256 for the general ones up to d = 3) and points per
+ * thread in {1, 2, 4, 8, 16, 32} is timed with CUDA events; the fastest is
+ * kept in the context and used by later plans whose options leave block/ppt at
+ * 0. best_block/best_ppt (may be NULL) receive QMC_NUM_CLASSES entries (0 =
+ * class absent); best_block is 256 or 384 for a class whose jobs all run an
+ * evaluator with that one block size. */
 #define QMC_NUM_CLASSES 13
 int qmc_autotune(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo, int norders, int *best_block,
                  int *best_ppt);

@@ -1058,13 +1058,14 @@ extern "C" int qmc_autotune(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo
     const int blocks[2] = {128, 256};
     const int ppts[6] = {1, 2, 4, 8, 16, 32};
     const qmc_options saved = ctx->opt;
+    int one_block[QMC_NCLASS] = {};   // the block size of a class whose jobs all run an evaluator that has one
     for (int cls = 0; cls < QMC_NCLASS; ++cls) {
         if (per[cls].empty()) continue;
         double best = INFINITY;
         int bb = 128, bp = 16;
         for (int b : blocks)
             for (int p : ppts) {
-                if (b == 256 && qmc_class_dmax(cls) > 3) continue;   // 128-thread blocks only
+                if (b == 256 && (qmc_class_dmax(cls) > 3 || one_block[cls])) continue;   // one block size
                 ctx->opt.block = b;
                 ctx->opt.ppt = p;
                 qmc_plan *plan = nullptr;
@@ -1072,6 +1073,14 @@ extern "C" int qmc_autotune(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo
                 if (rc) {
                     ctx->opt = saved;
                     return rc;
+                }
+                one_block[cls] = 0;
+                for (const ClassLaunch &c : plan->launches) {
+                    if (!c.fx) {
+                        one_block[cls] = 0;
+                        break;
+                    }
+                    one_block[cls] = c.block;
                 }
                 float ms = 0.f, best_ms = INFINITY;
                 for (int rep = 0; rep < 3 && !rc; ++rep) {
@@ -1095,7 +1104,7 @@ extern "C" int qmc_autotune(qmc_ctx *ctx, const qmc_job *jobs, int njobs, int lo
     }
     ctx->opt = saved;
     for (int cls = 0; cls < QMC_NCLASS; ++cls) {
-        if (best_block) best_block[cls] = ctx->tuned_block[cls];
+        if (best_block) best_block[cls] = one_block[cls] ? one_block[cls] : ctx->tuned_block[cls];
         if (best_ppt) best_ppt[cls] = ctx->tuned_ppt[cls];
     }
     return QMC_OK;
