@@ -2706,7 +2706,6 @@ __device__ __forceinline__ void thread_points(const TileSmem<LMAX> &S, const Qmc
     const uint32_t n32 = (uint32_t)n;
 #pragma unroll
     for (int j = 0; j < DMAX; ++j) walk_init(wk[j], (j < d) ? (k0 * (uint64_t)S.zmod[j]) % n : 0, n);
-#pragma unroll 1
     // Taylor subtraction: the instantiation of eval_real_taylor1 that serves
     // the tile's sector (4: one variable, p = 2; 1 .. 3: two, the bits of those
     // with p = 2), 0 for the loops, which take any p, order and number of
@@ -2721,6 +2720,7 @@ __device__ __forceinline__ void thread_points(const TileSmem<LMAX> &S, const Qmc
         if (kind) rb[0] = qrcp(sec.b[sec.sing[0]]);
         if (kind && kind < 4) rb[1] = qrcp(sec.b[sec.sing[1]]);
     }
+#pragma unroll 1
     for (uint64_t k = k0; k < kend; ++k) {
         double t[DMAX], omt[DMAX];
         double Ws = 1.0;  // prod u(1-u); the korobov3 weight is 140^d Ws^3
