@@ -202,8 +202,8 @@ int qmc_integral_info(qmc_ctx *ctx, int integral_id, int *nsectors, int *max_pol
                       int *prefactor_lo, qmc_c64 *prefactor, int cap, int *prefactor_len);
 
 /* Set the kinematic points: inv is a host array [npoints][ninv] of the
- * invariants in the order of the sector description. Replaces earlier points.
- * Errors: QMC_E_INVAL, QMC_E_CUDA. */
+ * invariants in the order of the sector description. Replaces earlier points;
+ * a plan made before runs on the new ones. Errors: QMC_E_INVAL, QMC_E_CUDA. */
 int qmc_set_kinematics(qmc_ctx *ctx, const double *inv, int npoints, int ninv);
 
 /* Build an evaluation plan for `njobs` jobs (host array): uploads the job
@@ -226,7 +226,8 @@ size_t qmc_plan_output_size(const qmc_plan *plan);
  * the context's stream) writing per-shift sums to `out_dev` (device, layout
  * [job][shift][order][re, im], qmc_plan_output_size doubles; NULL = the
  * plan's own buffer). Asynchronous: returns after the launches are queued.
- * Errors: QMC_E_CUDA. */
+ * Errors: QMC_E_CUDA, QMC_E_INVAL (the kinematics set since the plan was made
+ * lack a point of its jobs or have another number of invariants). */
 int qmc_plan_run(qmc_plan *plan, double *out_dev, void *stream);
 
 /* Wait for the plan's last run, then copy its per-shift sums to the host

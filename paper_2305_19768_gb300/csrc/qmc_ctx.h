@@ -106,6 +106,7 @@ struct qmc_plan {
     qmc_ctx *ctx = nullptr;
     int lo = 0, norders = 0, njobs = 0;
     uint64_t kin_version = 0;            // the kinematics its launches were chosen for
+    int ninv = 0, max_point = -1;        // what its jobs read of the kinematics: invariants a point, the last point
     double evals = 0.0;                  // lattice points x shifts of one run
     size_t out_size = 0;
     double *d_out = nullptr;

@@ -669,7 +669,7 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
     std::vector<std::map<uint64_t, uint64_t>> lattices(2 * QMC_NCLASS);
     std::vector<int> prows(2 * QMC_NCLASS, 1);
     std::vector<int> own(njobs, -1);   // index among the plan's jobs
-    int nown = 0;
+    int nown = 0, max_point = -1;
     uint64_t out_off = 0;
     double evals = 0.0;
     for (int i = 0; i < njobs; ++i) {
@@ -712,6 +712,7 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
         prows[slot] = std::max(prows[slot], S.prow);
         if (mine && !mine[i]) continue;
         own[i] = nown++;
+        if (!I.invariants.empty()) max_point = std::max(max_point, J.point);
         QmcJobDev D{};
         D.sector = S.global_index;
         D.point = I.invariants.empty() ? 0 : J.point;
@@ -735,6 +736,8 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
     p->lo = lo;
     p->norders = norders;
     p->njobs = nown;
+    p->max_point = max_point;
+    p->ninv = max_point < 0 ? 0 : ctx->ninv;
     p->out_size = (size_t)out_off;
     p->evals = evals;
     auto bail = [&](int rc) {
@@ -814,7 +817,7 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
         L.monos = ctx->d_monos;
         L.kin = ctx->d_kin;
         L.njobs = (int)v.size();
-        L.ninv = ctx->ninv;
+        L.ninv = p->ninv;
         L.lo = lo;
         L.norders = norders;
         L.ntiles = tiles;
@@ -958,7 +961,11 @@ int qmc_plan_run(qmc_plan *plan, double *out_dev, void *stream) {
     double *out = out_dev ? out_dev : plan->d_out;
     if (plan->kin_version != ctx->kin_version) {
         // new kinematics: the integer evaluator's jobs must still qualify, and
-        // a captured graph holds the old table's address
+        // a captured graph holds the old table's address. The kernels read the
+        // table by the plan's points and invariants: both must still be there
+        if (plan->max_point >= 0 && (plan->ninv != ctx->ninv || plan->max_point >= ctx->npoints))
+            return fail(ctx, QMC_E_INVAL, "qmc_plan_run: the plan reads point %d of %d invariants, the kinematics set since "
+                        "hold %d points of %d", plan->max_point, plan->ninv, ctx->npoints, ctx->ninv);
         for (ClassLaunch &c : plan->launches) {
             c.general = false;
             for (const ClassLaunch::FxJob &J : c.fx_jobs)
