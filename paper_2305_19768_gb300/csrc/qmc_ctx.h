@@ -73,7 +73,7 @@ struct qmc_ctx {
     int tuned_ppt[QMC_NCLASS] = {};
     double presample_evals = 0.0;       // lattice points x shifts spent in qmc_presample_lambda
     bool host_only = false;             // QMC_DEVICE_NONE: no GPU, caller-supplied evaluator only
-    uint64_t kin_version = 0;           // counts qmc_set_kinematics calls
+    uint64_t kin_version = 0;           // counts the device tables made: kinematics and sectors
     std::vector<double> h_kin;          // host copy of the kinematics [npoints][ninv]
     // coefficients of qmc_set_coefficients: [npoints][namp][nint][ncoef]
     int coef_namp = 0, coef_npoints = 0, coef_nint = 0, coef_lo = 0, coef_n = 0;

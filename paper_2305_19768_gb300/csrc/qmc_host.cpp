@@ -360,16 +360,26 @@ int upload_tables(qmc_ctx *ctx) {
     }
     ctx->nsectors_dev = (int)secs.size();
     if (ctx->host_only) return QMC_OK;   // tables checked and indexed, nothing to upload
+    // new tables beside the old ones, which plans may be reading and which stay if
+    // this fails; plans take the addresses when they run
+    QmcSectorDev *d_sectors = nullptr;
+    QmcMono *d_monos = nullptr;
+    cudaError_t e = cudaMalloc(&d_sectors, std::max<size_t>(1, secs.size()) * sizeof(QmcSectorDev));
+    if (!e) e = cudaMalloc(&d_monos, std::max<size_t>(1, monos.size()) * sizeof(QmcMono));
+    if (!e) e = cudaMemcpy(d_sectors, secs.data(), secs.size() * sizeof(QmcSectorDev), cudaMemcpyHostToDevice);
+    if (!e) e = cudaMemcpy(d_monos, monos.data(), monos.size() * sizeof(QmcMono), cudaMemcpyHostToDevice);
+    // (a copy from pageable memory may return before its last transfer is done)
+    if (!e) e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e) {
+        cudaFree(d_sectors);
+        cudaFree(d_monos);
+        return fail(ctx, QMC_E_CUDA, "sector tables: %s", cudaGetErrorString(e));
+    }
     cudaFree(ctx->d_sectors);
     cudaFree(ctx->d_monos);
-    ctx->d_sectors = nullptr;
-    ctx->d_monos = nullptr;
-    CUDA_TRY(ctx, cudaMalloc(&ctx->d_sectors, std::max<size_t>(1, secs.size()) * sizeof(QmcSectorDev)));
-    CUDA_TRY(ctx, cudaMalloc(&ctx->d_monos, std::max<size_t>(1, monos.size()) * sizeof(QmcMono)));
-    CUDA_TRY(ctx, cudaMemcpy(ctx->d_sectors, secs.data(), secs.size() * sizeof(QmcSectorDev),
-                             cudaMemcpyHostToDevice));
-    CUDA_TRY(ctx, cudaMemcpy(ctx->d_monos, monos.data(), monos.size() * sizeof(QmcMono),
-                             cudaMemcpyHostToDevice));
+    ctx->d_sectors = d_sectors;
+    ctx->d_monos = d_monos;
+    ++ctx->kin_version;
     ctx->nsectors_dev = (int)secs.size();
     return QMC_OK;
 }
@@ -813,9 +823,6 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
         }
         c.grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(tiles, (uint64_t)ctx->sm_count * occ));
         QmcLaunch &L = c.L;
-        L.sectors = ctx->d_sectors;
-        L.monos = ctx->d_monos;
-        L.kin = ctx->d_kin;
         L.njobs = (int)v.size();
         L.ninv = p->ninv;
         L.lo = lo;
@@ -922,6 +929,8 @@ int plan_enqueue(qmc_plan *plan, double *out, cudaStream_t st, bool capturing) {
         cudaStream_t cs = i == 0 ? st : plan->side[i - 1];
         if (i > 0) CUDA_TRY(ctx, cudaStreamWaitEvent(cs, plan->fork, 0));
         c.L.out = out;
+        c.L.sectors = ctx->d_sectors;
+        c.L.monos = ctx->d_monos;
         c.L.kin = ctx->d_kin;
         CUDA_TRY(ctx, cudaEventRecordWithFlags(plan->kev[2 * i], cs, evflags));
         if (c.L.ntiles > 0) {
@@ -961,7 +970,7 @@ int qmc_plan_run(qmc_plan *plan, double *out_dev, void *stream) {
     double *out = out_dev ? out_dev : plan->d_out;
     if (plan->kin_version != ctx->kin_version) {
         // new kinematics: the integer evaluator's jobs must still qualify, and
-        // a captured graph holds the old table's address. The kernels read the
+        // a captured graph holds the old tables' addresses. The kernels read the
         // table by the plan's points and invariants: both must still be there
         if (plan->max_point >= 0 && (plan->ninv != ctx->ninv || plan->max_point >= ctx->npoints))
             return fail(ctx, QMC_E_INVAL, "qmc_plan_run: the plan reads point %d of %d invariants, the kinematics set since "

@@ -87,3 +87,24 @@ def test_changed_kinematics_of_a_two_loop_plan(graph):
         qmc.qmc_plan_destroy(plan)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_a_plan_after_another_integral_was_loaded(graph):
+    g = Gpu()
+    try:
+        I = w.box_massless()
+        iid = g.load(I)
+        qmc.qmc_set_kinematics(g.ctx, np.array([[-3.0, -2.0]]))
+        jobs, nj = qmc.make_jobs(qmc.jobs_for_integral(iid, len(I.sectors), 1, 1009, 2, seed=5))
+        plan = qmc.qmc_plan_create(g.ctx, jobs, nj, -2, 3)
+        qmc.qmc_plan_use_graph(g.ctx, plan, graph)
+        qmc.qmc_plan_run(g.ctx, plan)
+        ref = qmc.qmc_plan_results(g.ctx, plan)[0].copy()
+        for build in (w.double_box_massless, w.box_massive):
+            g.load(build())
+            qmc.qmc_plan_run(g.ctx, plan)
+            assert np.array_equal(qmc.qmc_plan_results(g.ctx, plan)[0], ref)
+        qmc.qmc_plan_destroy(plan)
+    finally:
+        g.close()
