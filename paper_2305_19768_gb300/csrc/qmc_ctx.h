@@ -94,8 +94,12 @@ struct ClassLaunch {
     std::vector<int> orig;               // caller's index of each class-local job
     int block = 128, ppt = 16, grid = 0;
     // jobs for the evaluators of qmc_real.cuh or qmc_deformed.cuh; `general`:
-    // the kinematics set since no longer qualify, the general kernel runs instead
-    bool fx = false, general = false;
+    // the kinematics set since no longer qualify, and the general kernel runs
+    // instead, with the tiles G that it would have had from the start (its job
+    // table is made when it is first needed: `gready`)
+    bool fx = false, general = false, gready = false;
+    QmcLaunch G{};
+    int gblock = 128, gppt = 16;
     struct FxJob {
         int integral, sector, point;
     };

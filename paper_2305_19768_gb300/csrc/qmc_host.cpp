@@ -470,6 +470,36 @@ bool fd_job_ok(const HostSector &S, int cls) {
     return true;
 }
 
+// A job's tiles of tile_k points from tile `begin` of its launch on; returns the
+// tile after its last
+uint64_t retile(QmcJobDev &D, uint64_t tile_k, uint64_t begin) {
+    D.tiles_per_shift = (int32_t)((D.n + tile_k - 1) / tile_k);
+    D.tile_begin = begin;
+    return begin + (uint64_t)D.tiles_per_shift * D.shifts;
+}
+
+// After new kinematics: which launches' jobs still qualify for the integer
+// evaluator; the others take the general kernel, whose job table is made from the
+// launch's own the first time
+int plan_requalify(qmc_plan *plan) {
+    qmc_ctx *ctx = plan->ctx;
+    for (ClassLaunch &c : plan->launches) {
+        c.general = false;
+        for (const ClassLaunch::FxJob &J : c.fx_jobs)
+            c.general = c.general || !fx_job_ok(ctx, ctx->integrals[J.integral].sectors[J.sector], c.cls, J.point);
+        if (!c.general || c.gready) continue;
+        std::vector<QmcJobDev> v(c.orig.size());
+        const size_t bytes = v.size() * sizeof(QmcJobDev);
+        CUDA_TRY(ctx, cudaMemcpy(v.data(), c.L.jobs, bytes, cudaMemcpyDeviceToHost));
+        uint64_t tiles = 0;
+        for (QmcJobDev &D : v) tiles = retile(D, c.G.tile_k, tiles);
+        CUDA_TRY(ctx, cudaMemcpy(const_cast<QmcJobDev *>(c.G.jobs), v.data(), bytes, cudaMemcpyHostToDevice));
+        CUDA_TRY(ctx, cudaStreamSynchronize(cudaStreamLegacy));
+        c.gready = true;
+    }
+    return QMC_OK;
+}
+
 constexpr size_t kStatusBytes = 2 * sizeof(unsigned long long);   // sign failures, non-finite tiles
 constexpr size_t kOneCopy = 4096;   // results up to this many numbers come back with the status (32 KB on the stack)
 
@@ -652,6 +682,10 @@ int qmc_set_kinematics(qmc_ctx *ctx, const double *inv, int npoints, int ninv) {
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
     ctx->npoints = npoints;
     ctx->ninv = ninv;
+    for (qmc_plan *p : ctx->plans) {
+        const int rc = plan_requalify(p);
+        if (rc) return rc;
+    }
     return QMC_OK;
 }
 
@@ -806,6 +840,12 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
         }
         const int prow = prows[slot];
         int occ = 1;
+        uint64_t gtiles = 0;
+        if (!c.fx_jobs.empty()) {
+            c.gblock = c.block;
+            c.gppt = c.ppt;
+            for (QmcJobDev D : v) gtiles += retile(D, (uint64_t)c.gblock * c.gppt, 0);
+        }
         if (c.fx) {
             c.block = qmc_class_dmax(cls) > 3 ? QMC_FX6_BLOCK : QMC_FX3_BLOCK;   // their one block size
             occ = std::max(1, qmc_k_occupancy_real(cls, hi, prow));
@@ -816,11 +856,7 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
         }
         const uint64_t tile_k = (uint64_t)c.block * c.ppt;
         uint64_t tiles = 0;
-        for (QmcJobDev &D : v) {
-            D.tiles_per_shift = (int32_t)((D.n + tile_k - 1) / tile_k);
-            D.tile_begin = tiles;
-            tiles += (uint64_t)D.tiles_per_shift * D.shifts;
-        }
+        for (QmcJobDev &D : v) tiles = retile(D, tile_k, tiles);
         c.grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(tiles, (uint64_t)ctx->sm_count * occ));
         QmcLaunch &L = c.L;
         L.njobs = (int)v.size();
@@ -833,29 +869,35 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
         L.prow = prow;
         L.mone = -1.0;
         L.nzero = -0.0;
+        c.G = L;
+        c.G.ntiles = gtiles;
+        c.G.tile_k = (uint32_t)(c.gblock * c.gppt);
         p->launches.push_back(c);
     }
     // One allocation and one copy for everything a plan holds on the device
     // (six, and a copy or a fill each, took 32 us of a one-shot call's 90 for a
     // plan's set-up and release; with this the call takes 70). In order:
-    //   [jobs]  [queues, failure counts, status | results]  [partial sums]
+    //   [jobs]  [queues, failure counts, status | results]  [partial sums]  [jobs of G]
     // so that one fill clears what a run must find at zero and a small plan's
     // status and results come back in one copy.
     {
         auto up = [](size_t b) { return (b + 255) / 256 * 256; };
         size_t zero = 0, njob_bytes = 0, part = 0;
-        std::vector<size_t> at_queue, at_jobs, at_part;
+        size_t gjob_bytes = 0;
+        std::vector<size_t> at_queue, at_jobs, at_part, at_gjobs;
         for (const ClassLaunch &c : p->launches) {
             at_queue.push_back(zero);
             zero += 16 + (c.orig.size() * sizeof(unsigned int) + 15) / 16 * 16;
             at_jobs.push_back(njob_bytes);
             njob_bytes += up(c.orig.size() * sizeof(QmcJobDev));
             at_part.push_back(part);
-            part += up(std::max<uint64_t>(1, c.L.ntiles) * 2 * norders * sizeof(double));
+            part += up(std::max<uint64_t>(1, std::max(c.L.ntiles, c.G.ntiles)) * 2 * norders * sizeof(double));
+            at_gjobs.push_back(gjob_bytes);
+            if (!c.fx_jobs.empty()) gjob_bytes += up(c.orig.size() * sizeof(QmcJobDev));
         }
         zero = up(zero + kStatusBytes);   // the status ends the cleared part
         const size_t part_at = up(njob_bytes + zero + std::max<size_t>(1, p->out_size) * sizeof(double));
-        PLAN_TRY(cudaMalloc(&p->d_arena, part_at + part));
+        PLAN_TRY(cudaMalloc(&p->d_arena, part_at + part + gjob_bytes));
         p->d_zero = p->d_arena + njob_bytes;
         p->zero_bytes = zero;
         p->d_status = (unsigned long long *)(p->d_zero + zero - kStatusBytes);
@@ -873,6 +915,11 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
             c.L.status = p->d_status;
             c.L.out = p->d_out;
             c.L.job_fail = c.d_jobfail;
+            c.G.queue = c.L.queue;
+            c.G.jobs = (const QmcJobDev *)(p->d_arena + part_at + part + at_gjobs[k]);
+            c.G.partials = c.L.partials;
+            c.G.status = c.L.status;
+            c.G.job_fail = c.L.job_fail;
             ++k;
         }
         PLAN_TRY(cudaMemcpy(p->d_arena, head.data(), head.size(), cudaMemcpyHostToDevice));
@@ -928,25 +975,28 @@ int plan_enqueue(qmc_plan *plan, double *out, cudaStream_t st, bool capturing) {
         ClassLaunch &c = plan->launches[i];
         cudaStream_t cs = i == 0 ? st : plan->side[i - 1];
         if (i > 0) CUDA_TRY(ctx, cudaStreamWaitEvent(cs, plan->fork, 0));
-        c.L.out = out;
-        c.L.sectors = ctx->d_sectors;
-        c.L.monos = ctx->d_monos;
-        c.L.kin = ctx->d_kin;
+        QmcLaunch &L = c.general ? c.G : c.L;
+        L.out = out;
+        L.sectors = ctx->d_sectors;
+        L.monos = ctx->d_monos;
+        L.kin = ctx->d_kin;
         CUDA_TRY(ctx, cudaEventRecordWithFlags(plan->kev[2 * i], cs, evflags));
-        if (c.L.ntiles > 0) {
-            const bool fx = c.fx && !c.general;
-            // the general d <= 6 kernels exist with 128 threads only
-            const int gblock = c.fx && qmc_class_dmax(c.cls) > 3 ? 128 : c.block;
-            const int ggrid = fx || !c.fx ? c.grid
-                                    : (int)std::min<uint64_t>(c.L.ntiles, (uint64_t)ctx->sm_count *
-                                                                std::max(1, qmc_k_occupancy(c.cls, gblock, c.L.prow)));
-            if (fx ? qmc_k_launch_real(c.cls, &c.L, c.grid, cs)
-                   : qmc_k_launch_eval(c.cls, &c.L, gblock, (int)(c.L.tile_k / gblock), ggrid, cs))
+        if (c.general && !c.gready) return fail(ctx, QMC_E_CUDA, "qmc_plan_run: the kinematics were not set completely");
+        if (L.ntiles > 0) {
+            int rc;
+            if (c.general) {
+                const uint64_t fit = (uint64_t)ctx->sm_count * std::max(1, qmc_k_occupancy(c.cls, c.gblock, L.prow));
+                rc = qmc_k_launch_eval(c.cls, &L, c.gblock, c.gppt, (int)std::min(L.ntiles, fit), cs);
+            } else {
+                rc = c.fx ? qmc_k_launch_real(c.cls, &L, c.grid, cs)
+                          : qmc_k_launch_eval(c.cls, &L, c.block, c.ppt, c.grid, cs);
+            }
+            if (rc)
                 return fail(ctx, QMC_E_CUDA, "evaluator launch failed: %s", cudaGetErrorString(cudaGetLastError()));
             ++launches;
         }
         CUDA_TRY(ctx, cudaEventRecordWithFlags(plan->kev[2 * i + 1], cs, evflags));
-        if (qmc_k_launch_finish(&c.L, cs))
+        if (qmc_k_launch_finish(&L, cs))
             return fail(ctx, QMC_E_CUDA, "finish launch failed: %s", cudaGetErrorString(cudaGetLastError()));
         ++launches;
         if (i > 0) {
@@ -969,17 +1019,12 @@ int qmc_plan_run(qmc_plan *plan, double *out_dev, void *stream) {
     cudaStream_t st = stream ? (cudaStream_t)stream : ctx->stream;
     double *out = out_dev ? out_dev : plan->d_out;
     if (plan->kin_version != ctx->kin_version) {
-        // new kinematics: the integer evaluator's jobs must still qualify, and
-        // a captured graph holds the old tables' addresses. The kernels read the
-        // table by the plan's points and invariants: both must still be there
+        // a captured graph holds the old tables' addresses (and launches), and the
+        // kernels read the kinematics by the plan's points and invariants: both
+        // must still be there
         if (plan->max_point >= 0 && (plan->ninv != ctx->ninv || plan->max_point >= ctx->npoints))
             return fail(ctx, QMC_E_INVAL, "qmc_plan_run: the plan reads point %d of %d invariants, the kinematics set since "
                         "hold %d points of %d", plan->max_point, plan->ninv, ctx->npoints, ctx->ninv);
-        for (ClassLaunch &c : plan->launches) {
-            c.general = false;
-            for (const ClassLaunch::FxJob &J : c.fx_jobs)
-                c.general = c.general || !fx_job_ok(ctx, ctx->integrals[J.integral].sectors[J.sector], c.cls, J.point);
-        }
         if (plan->gexec) cudaGraphExecDestroy(plan->gexec);
         plan->gexec = nullptr;
         plan->kin_version = ctx->kin_version;

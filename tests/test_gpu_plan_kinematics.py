@@ -1,6 +1,8 @@
 """A plan run after its kinematics were replaced (GPU): by other values it
 follows them, on the d <= 6 evaluators too; by fewer points, or by points with
 another number of invariants, the run is refused, and runs again when they fit."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -8,6 +10,7 @@ from paper_2305_19768_gb300 import qmc
 from paper_2305_19768_gb300.inputs import workloads as w
 
 from parity import Gpu, assert_close, oracle_sums
+from test_gpu_real_integer import general
 
 pytestmark = pytest.mark.gpu
 
@@ -105,6 +108,36 @@ def test_a_plan_after_another_integral_was_loaded(graph):
             g.load(build())
             qmc.qmc_plan_run(g.ctx, plan)
             assert np.array_equal(qmc.qmc_plan_results(g.ctx, plan)[0], ref)
+        qmc.qmc_plan_destroy(plan)
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("opts", [{}, {"ppt": 5}, {"block": 256}])
+@pytest.mark.parametrize("build,lo,n,step", [(w.box_massless, -2, 1009, 1), (w.box_massless, -2, 20011, 1),
+                                             (w.double_box_massless, -4, 1009, 25)])
+def test_general_kernel_with_its_own_tiles(build, lo, n, step, opts):
+    """Where new kinematics take a plan to the general kernel it has the tiles that
+    a plan of the general kernel has: the same bits as one (whose F carries a
+    negligible negative monomial), also when it comes back a second time."""
+    I = build()
+    g = Gpu(**opts)
+    try:
+        iid, gid = g.load(I), g.load(general(I, Fraction(-1, 10 ** 250)))
+        near, far = np.array([[-3.0, -1.0]]), np.array([[-3000.0, -1.0]])
+        specs = [dict(integral_id=iid, sector=s, point=0, shifts=2, n=n, seed=11, stream=s)
+                 for s in range(0, len(I.sectors), step)]
+        jobs, nj = qmc.make_jobs(specs)
+        qmc.qmc_set_kinematics(g.ctx, near)
+        plan = qmc.qmc_plan_create(g.ctx, jobs, nj, lo, 1 - lo)
+        qmc.qmc_set_kinematics(g.ctx, far)
+        ref, _, rc = g.eval(gid, [dict(sp, integral_id=gid) for sp in specs], lo, 1 - lo)
+        assert rc == 0
+        for kin in (far, near, far):
+            qmc.qmc_set_kinematics(g.ctx, kin)
+            qmc.qmc_plan_run(g.ctx, plan)
+            got = qmc.qmc_plan_results(g.ctx, plan)[0]
+            assert np.array_equal(got, ref) == (kin is far)
         qmc.qmc_plan_destroy(plan)
     finally:
         g.close()
