@@ -115,18 +115,30 @@ PROFILED = {
         "warp_inst_per_eval": 386.3, "issue_busy": 0.529},
 }
 
-# What the roofline counts (flops.py): the specialised evaluators run part of
-# it on the integer pipe, so a fraction of the DFMA peak built on it is
-# FP64-equivalent work and may pass 1
-FLOPS_OF = ("the general evaluator's formulation; qmc_real_kernel and qmc_deformed_kernel run part of it on the "
-            "integer pipe (FP64-equivalent, not a share of the FP64 pipe)")
+# What the roofline counts (flops.py): the FP64 operations that the evaluators of
+# the workload's jobs run. The same sums in the general evaluator's formulation
+# stand beside it as FP64-equivalent work, which may pass the DFMA peak.
+FLOPS_OF = "what the launched evaluators run on the FP64 pipe"
+FORMULATION_OF = ("the general evaluator's formulation of the same sums; part of it runs on the integer pipe "
+                  "(FP64-equivalent, not a share of the FP64 pipe)")
+
+
+def fp64_roofline(flopmod, I, inv, lo, nord, rate, peak_gflops, mixed=False):
+    """achieved and frac from the executed FP64 operations (null where only the
+    general formulation is counted), and that formulation's count beside them."""
+    ran = flopmod.executed_workload(I, inv, lo, nord, mixed)
+    form = flopmod.workload_work(I, lo, nord, mixed=mixed)
+    got = None if ran is None else ran.fp64 * rate / 1e9
+    return {"achieved": got, "peak": peak_gflops, "frac": None if ran is None else got / peak_gflops,
+            "flops_per_eval": None if ran is None else ran.fp64, "flops_of": FLOPS_OF, "unit": "GFLOP/s (fp64)",
+            "formulation": {"flops_per_eval": form.fp64, "achieved": form.fp64 * rate / 1e9, "of": FORMULATION_OF}}, ran or form
 
 
 def kernel_sha1():
     import hashlib
 
     h = hashlib.sha1()
-    for name in ("qmc_kernels.cu", "qmc_real.cuh", "qmc_deformed.cuh"):
+    for name in ("qmc_kernels.cu", "qmc_real.cuh", "qmc_deformed.cuh", "qmc_ilog.h", "qmc_xf.h", "qmc_iarg.h"):
         with open(os.path.join(ROOT, "paper_2305_19768_gb300", "csrc", name), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -279,12 +291,10 @@ def box_extra(device, opts, sptr, flush, peak_gflops, seed):
         ms = timed_plan(qmc, ctx, plan, o.data_ptr(), sptr, flush, 10)
         qmc.qmc_plan_destroy(plan)
         evals = nj * W["m"] * W["n"]
-        fl = flopmod.workload_work(I, W["lo"], W["nord"]).fp64
         rate = evals / (float(np.mean(ms)) * 1e-3)
         out["box1L_massless"] = {
             "workload": W["desc"].format(n=W["n"], m=W["m"]), "evals_per_s": rate, "eval_ms": float(np.mean(ms)),
-            "roofline": {"achieved": fl * rate / 1e9, "peak": peak_gflops, "frac": fl * rate / 1e9 / peak_gflops,
-                         "flops_per_eval": fl, "flops_of": FLOPS_OF, "unit": "GFLOP/s (fp64)"}}
+            "roofline": fp64_roofline(flopmod, I, W["kin"][0], W["lo"], W["nord"], rate, peak_gflops)[0]}
         for prec, key in ((qmc.QMC_PRECISION_FP64, "fp64"), (qmc.QMC_PRECISION_MIXED, "mixed")):
             c2 = qmc.qmc_create(device, precision=prec, **opts)
             try:
@@ -334,12 +344,10 @@ def batch_extra(device, opts, sptr, flush, peak_gflops, seed, n=100003, m=32):
     finally:
         qmc.qmc_destroy(ctx)
     evals = nj * m * n
-    fl = flopmod.workload_work(I, W["lo"], W["nord"]).fp64
     rate = evals / (float(np.mean(ms)) * 1e-3)
     return {"box1L_massive_batch": {
         "workload": W["desc"].format(n=n, m=m), "evals_per_s": rate, "eval_ms": float(np.mean(ms)),
-        "roofline": {"achieved": fl * rate / 1e9, "peak": peak_gflops, "frac": fl * rate / 1e9 / peak_gflops,
-                     "flops_per_eval": fl, "flops_of": FLOPS_OF, "unit": "GFLOP/s (fp64)"}}}
+        "roofline": fp64_roofline(flopmod, I, W["kin"][0], W["lo"], W["nord"], rate, peak_gflops)[0]}}
 
 
 def mixed_extra(device, opts, I, W, kin, jobs, nj, evals_per_step, out_dev, sptr, seed, skip_oracle):
@@ -567,29 +575,26 @@ def main():
         t_e2e += time.perf_counter() - t0
     e2e_val = evals_per_step * n_e2e * world / t_e2e
 
-    # roofline of the evaluator kernels: FP64 flops of the general evaluator's
-    # formulation / their event time, against the DFMA peak measured in this run; FP32 work of the mixed classes
-    # against the FFMA peak; transcendentals per evaluation beside them
-    work = flopmod.workload_work(I, LO, NORD, mixed=args.precision == "mixed")
+    # roofline of the evaluator kernels: the FP64 operations they run / their
+    # event time, against the DFMA peak measured in this run; FP32 work of the
+    # mixed classes against the FFMA peak; transcendentals per evaluation beside them
     avg_eval_ms = float(np.mean(eval_ms))
     rate = evals_per_step / (avg_eval_ms * 1e-3)
-    achieved = work.fp64 * rate / 1e9
     sha = kernel_sha1()
     prof = PROFILED.get((sha, args.workload, args.precision, args.decomposition, args.n), {})
-    roof = {"bound": "alu", "achieved": achieved, "peak": peak_gflops, "unit": "GFLOP/s (fp64)",
-            "frac": achieved / peak_gflops, "traffic": prof.get("traffic"),
-            "flops_per_eval": work.fp64, "flops_of": FLOPS_OF, "peak_source": "DFMA probe in this run (of measured)",
-            "transcendentals_per_eval": {k: getattr(work, k) for k in ("log", "atan2", "rcp", "exp", "rcp_int")},
-            "fp64_executed_flops_per_eval": prof.get("fp64_executed_flops_per_eval"),
-            "fp64_pipe_busy": prof.get("fp64_pipe_busy"),
-            "evals_per_launch": evals_per_step, "eval_ms_per_step": avg_eval_ms,
-            "kernel_sha1": sha}
+    roof, work = fp64_roofline(flopmod, I, W["kin"][0], LO, NORD, rate, peak_gflops, args.precision == "mixed")
+    roof.update({"bound": "alu", "traffic": prof.get("traffic"),
+                 "peak_source": "DFMA probe in this run (of measured)",
+                 "transcendentals_per_eval": {k: getattr(work, k) for k in ("log", "atan2", "rcp", "exp", "rcp_int")},
+                 "fp64_executed_flops_per_eval": prof.get("fp64_executed_flops_per_eval"),
+                 "fp64_pipe_busy": prof.get("fp64_pipe_busy"),
+                 "evals_per_launch": evals_per_step, "eval_ms_per_step": avg_eval_ms,
+                 "kernel_sha1": sha})
     # the same formulation counted as if all of it ran in FP64, the d <= 6 corner
     # stage included: algorithmic, not FP64-pipe work
     eq = flopmod.workload_work(I, LO, NORD, mixed=args.precision == "mixed", fp64_corners=True).fp64
-    if eq != work.fp64:
-        roof["algorithmic_fp64_equivalent"] = {"flops_per_eval": eq, "achieved": eq * rate / 1e9,
-                                               "frac": eq * rate / 1e9 / peak_gflops}
+    if eq != roof["formulation"]["flops_per_eval"]:
+        roof["algorithmic_fp64_equivalent"] = {"flops_per_eval": eq, "achieved": eq * rate / 1e9}
     # the issue roofline: warp instructions per evaluation (ncu, this source)
     # at the measured rate, against 4 warp instructions per SM per clock
     if prof.get("warp_inst_per_eval") and clocks and clocks.get("sm_mhz"):

@@ -14,8 +14,10 @@
 //  * U and F are sums of positive terms, so they are evaluated in fixed
 //    point: t as t 2^64, coefficients scaled so that their sum stays below
 //    2^64, each factor one high product, subset sums over the singular
-//    variables plain 64-bit adds. The error is some 2^-61 of the sum of
-//    coefficients, below 2^-53 of any corner value (all are >= c0);
+//    variables plain 64-bit adds. A monomial may lose a unit, 2^-63 of the sum
+//    of coefficients or less, so at most 2^-55 of any corner value (all are
+//    >= c0, which the rule keeps above 1/128 of that sum); an FP64 monomial may
+//    lose 2^-53 of itself and again of the sum it enters;
 //  * a corner's powers and logarithm follow from those integers directly.
 // FP64 is left with each corner's series (B L^i / i!), their combination and
 // the accumulation. Sectors with three or four singular variables (EX below)

@@ -2,10 +2,11 @@
 
 One evaluation = one lattice point of one sector for one shift, all eps
 orders, all subtraction corners. The count follows the general evaluator's
-formulation of the method (qmc_eval_kernel), operation by operation. The
-specialised evaluators (qmc_real_kernel, qmc_deformed_kernel) need fewer FP64
-operations for the same sums and run more on the integer pipe; at their rates
-this count is FP64-equivalent work, not a share of the FP64 pipe.
+formulation of the method (qmc_eval_kernel), operation by operation; this is
+what `sector_work` and `workload_work` give. The specialised evaluators
+(qmc_real_kernel, qmc_deformed_kernel) need fewer FP64 operations for the same
+sums and run more on the integer pipe: `executed_work` counts what they run, and
+a roofline fraction built on it is a share of the FP64 pipe.
 
 * FP64 flops: add, subtract and multiply count 1, a fused multiply-add 2.
   Steps that the evaluator computes on the integer pipe count 0 FP64 flops:
@@ -586,3 +587,160 @@ def workload_work(integral, lo: int, norders: int, mixed: bool = False, fp64_cor
 def workload_flops(integral, lo: int, norders: int, deform: bool = False) -> float:
     """Mean FP64 flops per evaluation (no credit for integer-pipe steps)."""
     return workload_work(integral, lo, norders).fp64
+
+
+# ------------------------------------------------ the evaluators on integers
+def takes_integer_evaluator(sector, inv, hi: int) -> bool:
+    """Whether a job of the sector at the invariants `inv` runs in
+    qmc_real_kernel or qmc_deformed_kernel (FP64), the rules of the host library."""
+    d, sing, ns, _ = _sector_shape(sector)
+    if any(int(a) <= -2 for a in sector.a) or any(not _is_small_int(x) for x in
+                                                  (sector.u0, sector.u1, sector.f0, sector.f1)):
+        return False
+    if sector.deform:
+        small = all(_is_small_int(b) for b in sector.b)
+        return d <= 3 and hi in (0, 1) and small and all(sum(e) <= 2 for e in sector.F.terms)
+    if not (hi == 0 or (hi == 1 and d <= 3 and ns <= 2)):
+        return False
+    for P in (sector.U, sector.F):
+        c = {e: float(v[0]) + sum(float(x) * y for x, y in zip(v[1:], inv)) for e, v in P.terms.items()}
+        c0, total = c.get((0,) * d, 0.0), sum(c.values())
+        if min(c.values()) < 0.0 or not 1e-100 < c0 <= total < 1e100 or total > 128.0 * c0:
+            return False
+    return True
+
+
+def _fold(ns, hi, V, sub):
+    """FP64 flops of folding the singular variables below ns over the corners
+    with the bits of V: per order the difference of two corner series (sub: it
+    is taken here), then one multiply-add per term."""
+    if ns == 0:
+        return 0
+    n = ns + _popc(V) + hi
+    return ((n if sub else 0) + 2 * (n * (n + 1) // 2) + _fold(ns - 1, hi, V, sub)
+            + _fold(ns - 1, hi, V | (1 << (ns - 1)), sub))
+
+
+def _executed_real(sector, lo, norders, mixed) -> Work:
+    d, sing, ns, emax = _sector_shape(sector)
+    hi = lo + norders - 1
+    w = Work()
+    ex = ns >= 3                                     # the general kernel's roundings
+    regular = [j for j in range(d) if j not in sing and (sector.a[j] > 0 or float(sector.b[j]) != 0.0)]
+    logs_b = any(float(sector.b[j]) != 0.0 for j in regular)
+    if mixed or ex:
+        polys = _powers(d, emax) + _grouped_poly(sector.U, sing, ns) + _grouped_poly(sector.F, sing, ns)
+        if mixed:
+            w.fp32 += polys
+        else:
+            w.fp64 += polys
+    w.fp64 += 2 * ns + 2 * len(regular)              # b / t, b ln t; the regular logarithms' sum
+    w.rcp_int += ns
+    w.log += (ns if ns + hi > 1 else 0) + (len(regular) if ns + hi > 0 else 0)
+    for V in range(1 << ns):
+        lam = hi + _popc(V) >= 1
+        w.log += int(lam)
+        w.rcp_int += int(sector.u0 < 0 or (lam and sector.u1 < 0)) + int(sector.f0 < 0 or (lam and sector.f1 < 0))
+        w.fp64 += 1 if lam and logs_b else 0
+        for i in range(1, hi + _popc(V) + 1):        # B L^i / i!; halves on the exponent
+            w.fp64 += (1 if i == 1 else 2) if ex else (2 if i == 3 else 1)
+    for i in range(1, ns + hi):                      # (b / t) (b ln t)^i / i!
+        w.fp64 += ns * (2 if i == 3 else 1)
+    if ex:                                           # Moebius differences
+        w.fp64 += sum(hi + _popc(P) + 1 for q in range(ns) for P in range(1 << ns) if not P >> q & 1)
+    w.fp64 += _fold(ns, hi, 0, not ex) + 2 * (ns + hi + 1)
+    return w
+
+
+def _executed_deformed(sector, lo, norders) -> Work:
+    d, sing, ns, _ = _sector_shape(sector)
+    hi = lo + norders - 1
+    slot = {j: i for i, j in enumerate(sing + [j for j in range(d) if j not in sing])}
+    pairs, squares = set(), set()
+    for e in sector.F.terms:
+        v = sorted(slot[j] for j in range(d) for _ in range(e[j]))
+        if len(v) == 2:
+            (squares if v[0] == v[1] else pairs).add(v[0] if v[0] == v[1] else tuple(v))
+    coupled = lambda a, b: (min(a, b), max(a, b)) in pairs
+    a_of = {slot[j]: int(sector.a[j]) for j in range(d)}
+    b_of = {slot[j]: int(sector.b[j]) for j in range(d)}
+    u0, f0, u1, f1 = (int(x) for x in (sector.u0, sector.f0, sector.u1, sector.f1))
+    cpow = {1: 0, 2: 4, 3: 10, 4: 8}                 # x^e of a complex x
+    w = Work()
+    w.fp64 += ns * (1 + int(ns + hi > 1) + max(ns + hi - 1, 0))   # b / t, b ln t, their series
+    w.rcp_int += 2 * ns + d                          # 1/t; 1/(t (1 - t)) of every variable
+    w.log += ns if ns + hi > 1 else 0
+    for V in range(1 << ns):
+        lam = hi + _popc(V) >= 1
+        live = [j for j in range(d) if not V >> j & 1]
+        f = 0
+        for j in range(d):                           # gradient
+            if j not in live and not lam:
+                continue
+            near = [k for k in live if k != j and coupled(j, k)]
+            f += 2 * len(near) + (4 if j in live and j in squares else 0)
+        f += 3 * len(live)                           # y, M
+        minor = lambda x, z: 3 if coupled(x, z) else 1
+        if len(live) == 1:
+            f += 1
+        elif len(live) == 2:
+            f += minor(*live) + 3 + 3
+        elif len(live) == 3:
+            f += minor(0, 1) + minor(0, 2) + minor(1, 2) + 1
+            f += 3 * (coupled(0, 1) + coupled(0, 2)) + (3 if len(pairs) == 3 else 0)
+            f += 1 + 8 + 8
+        for i, j in enumerate(live):                 # F on the contour
+            near = sum(1 for k in live if k > j and coupled(j, k))
+            q = (1 if j in squares else 0) + max(2 * near - (0 if j in squares else 1), 0) if near or j in squares else 0
+            f += 2 + q + (2 if near or j in squares else 0) + (1 if i == 0 else 2)
+        need_u = u0 != 0 or (lam and u1 != 0)
+        if need_u:
+            for e in sector.U.terms:
+                if any(e[j] for j in range(d) if slot[j] not in live):
+                    continue
+                deg = sum(e)
+                f += 1 if deg == 0 else 6 * (deg - 1) + 4
+        for j in range(d):
+            if j < ns:
+                if j in live or lam:
+                    f += 3                           # lambda (1 - t) g, 1 + its square
+                f += 4 if j in live else 0
+            elif a_of[j] > 0 or b_of[j]:
+                f += 3 + (cpow[a_of[j]] + 6 if a_of[j] > 0 else 0)
+        f += (3 + (cpow[abs(u0)] + 6 if u0 else 0) if need_u else 0) + 3 + (cpow[abs(f0)] + 6 if f0 else 0)
+        n = hi + _popc(V)
+        f += (2 if ns else 0) + 6 * n + (2 if n >= 3 else 0)
+        w.fp64 += f
+        w.rcp_int += 1 + int(lam)
+        w.log += int(lam)
+        if lam:                                      # arguments, on the integer pipe
+            w.atan2 += sum(1 for j in range(d) if b_of[j]) + int(u1 != 0) + int(f1 != 0)
+    w.fp64 += 2 * _fold(ns, hi, 0, True) + 4 * (ns + hi + 1)
+    return w
+
+
+def executed_work(sector, inv, lo: int, norders: int, mixed: bool = False) -> Work:
+    """FP64 flops that the evaluator of the sector's jobs at the invariants `inv`
+    runs (a product or sum alone counts 1 although it is issued as an FMA), with
+    its integer-pipe logarithms, reciprocals and arctangents beside them. None
+    where only the general formulation's count exists (mixed deformed sectors,
+    the written-out Taylor form)."""
+    hi = lo + norders - 1
+    if any(int(a) <= -2 for a in sector.a):
+        return None
+    if not takes_integer_evaluator(sector, inv, hi):
+        return sector_work(sector, lo, norders, mixed)
+    if sector.deform:
+        return None if mixed else _executed_deformed(sector, lo, norders)
+    return _executed_real(sector, lo, norders, mixed)
+
+
+def executed_workload(integral, inv, lo: int, norders: int, mixed: bool = False):
+    """Mean executed work per evaluation over the sectors, or None."""
+    each = [executed_work(s, inv, lo, norders, mixed) for s in integral.sectors]
+    if any(x is None for x in each):
+        return None
+    tot = Work()
+    for x in each:
+        tot.add(x, 1.0 / len(each))
+    return tot
