@@ -692,7 +692,8 @@ __device__ __forceinline__ void fx_points(const QmcLaunch &Lc, uint64_t k0, uint
             }
             fx_subset_ex<NS>(hU);
             fx_subset_ex<NS>(hF);
-            const double Cd = S.hasC ? fx_pack(Cc) : 1.0;
+            // (a product of t^a may lie below the normal range)
+            const double Cd = S.hasC ? qmc_xf_to_double(qmc_xf{Cc.m, Cc.e, 0}) : 1.0;
 #pragma unroll 1
             for (int V = 0; V < NG; ++V) {
                 const FxCorner c = fx_corner_ex(hU[(NG - 1) ^ V], hF[(NG - 1) ^ V], Cd, Lr, HI > 0 || V != 0);

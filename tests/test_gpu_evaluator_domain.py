@@ -191,3 +191,42 @@ def test_imaginary_parts_of_nearly_real_sums(lam):
             assert top[-1] > 0 and np.all(np.abs(a - b) <= 1e-11 * top), np.abs(a - b).max(axis=0) / top
     finally:
         g.close()
+
+
+FAR = """qmc-sectors 1
+name far
+loops 2 propagators 7 dim 4
+invariants 1 s
+prefactor 0 1 1.0 0.0
+nsectors 1
+sector 0 d 6 deform 0
+a -1 4 -1 4 -1 4
+b -1.0 0.0 -2.0 0.0 1.0 0.0
+U 1.0 3.0 2
+0 0 0 0 0 0 1.0 0.0
+1 1 1 0 0 0 1.0 0.0
+F -2.0 -2.0 3
+0 0 0 0 0 0 0.0 -1.0
+1 0 0 1 1 0 0.0 -1.0
+0 1 1 0 0 1 1.0 0.0
+end
+"""
+
+
+def test_prefactors_below_the_normal_range():
+    """Regular factors t^4 in three variables at the first points of an unshifted
+    lattice with n = 2^24 (t = 35 / n^4 each): their product is below FP64's normal
+    range, and the sums are the general kernel's."""
+    g = Gpu()
+    try:
+        J = Integral.from_text(FAR)
+        iid, gid = g.load(J), g.load(general(J, Fraction(-1, 10 ** 250)))
+        qmc.qmc_set_kinematics(g.ctx, np.array([[-3.0]]))
+        sp = dict(integral_id=iid, sector=0, point=0, shifts=1, n=16777259, z=[1] * 6, seed=3, stream=0,
+                  flags=qmc.QMC_JOB_UNSHIFTED)
+        a, _, ra = g.eval(iid, [sp], -3, 4)
+        b, _, rb = g.eval(gid, [dict(sp, integral_id=gid)], -3, 4)
+        assert ra == rb == 0
+        assert np.all(np.abs(a - b) <= 1e-11 * np.abs(b).max())
+    finally:
+        g.close()
