@@ -59,7 +59,7 @@ struct alignas(16) FdShared {
     int32_t gvar, hvar;              // bits: those that are not
     int32_t perm[QMC_DMAX], slotof[QMC_DMAX], avar[QMC_DMAX], bvar[QMC_DMAX];
     double bd[QMC_DMAX], lam[QMC_DMAX];
-    uint64_t lamm[QMC_DMAX];         // lambda as mantissa, exponent and sign
+    uint64_t lamm[QMC_DMAX];         // lambda as mantissa (0: none, or outside 2^-800 .. 2^1024), exponent and sign
     int32_t lame[QMC_DMAX], lamneg[QMC_DMAX];
     int32_t regular, u0, f0, u1, f1;
     double delta[QMC_DMAX];
@@ -598,6 +598,9 @@ __device__ __forceinline__ void fd_points(const QmcLaunch &Lc, uint64_t k0, uint
             if (lm.m) {
                 P.p[i] = fd_signed(fx_pack(fx_norm(fx_mul(lm, tv))), S.lamneg[i] != 0);
                 if (i < NS) P.s[i] = fd_signed(fx_pack(fx_norm(fx_mul(lm, v))), S.lamneg[i] != 0);
+            } else if (S.lam[i] != 0.0) {               // not finite, or its products may not be normal
+                P.s[i] = S.lam[i] * fx_pack(v);
+                P.p[i] = P.s[i] * td;
             }
             if (c.m) P.k[i] = fd_signed(fx_pack(fx_norm(fx_mul(c, fd_rcp(tv)))), cneg);
             if constexpr (MIXED) {
@@ -842,9 +845,11 @@ __global__ void __launch_bounds__(BLOCK, fd_min_units<MIXED, HI>() * 128 / BLOCK
             S.rz[i] = (uint32_t)rz;
             S.zmod[i] = (uint32_t)zm;
             S.lam[i] = S.job.lambda[j];
+            // (t (1 - t) >= 2^-212: from 2^-800 on its products with lambda are normal)
             const qmc_xf lx = qmc_xf_of(S.job.lambda[j]);
-            S.lamm[i] = lx.m;
-            S.lame[i] = lx.m ? lx.e : 0;
+            const bool usual = lx.m && lx.e > -800 && lx.e < 1024;
+            S.lamm[i] = usual ? lx.m : 0;
+            S.lame[i] = usual ? lx.e : 0;
             S.lamneg[i] = lx.neg;
             if (i == 0) S.minv = minv;
         }

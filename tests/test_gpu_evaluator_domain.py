@@ -230,3 +230,27 @@ def test_prefactors_below_the_normal_range():
         assert np.all(np.abs(a - b) <= 1e-11 * np.abs(b).max())
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("lam", [float("nan"), float("inf"), -float("inf"), 1e-250, -1e-290, 5e-324])
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("name", ["box_massive", "box"])
+def test_lambda_outside_the_usual_range(name, lam, mixed):
+    """A lambda that is not finite gives sums that are not, and the status says
+    so; one whose products leave FP64's normal range gives the undeformed sums."""
+    I, lo = (w.box_massive(), 0) if name == "box_massive" else (w.box_massless(deform=True), -2)
+    g = Gpu(precision=qmc.QMC_PRECISION_MIXED if mixed else qmc.QMC_PRECISION_FP64)
+    try:
+        iid = g.load(I)
+        qmc.qmc_set_kinematics(g.ctx, np.array([[-3.0, -2.0]]))
+        specs = [dict(integral_id=iid, sector=s, point=0, shifts=2, n=1009, seed=3, stream=s, **{"lambda": lam})
+                 for s in range(len(I.sectors))]
+        a, _, ra = g.eval(iid, specs, lo, 1 - lo)
+        if not np.isfinite(lam):
+            assert ra == NONFINITE
+            return
+        b, _, rb = g.eval(iid, [dict(sp, **{"lambda": 0.0}) for sp in specs], lo, 1 - lo)
+        assert ra in (0, -6) and rb == 0            # (-6: a negative lambda's sign check)
+        assert np.all(np.abs(a - b) <= 1e-12 * np.abs(b).max())
+    finally:
+        g.close()
