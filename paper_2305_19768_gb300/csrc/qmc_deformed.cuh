@@ -472,7 +472,8 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
     }
     if (needU) factor(U, fd_norm2(U.re, U.im), S.u0, S.u1, false);
     factor(F, fd_norm2(F.re, F.im), S.f0, S.f1, true);
-    if (max(den.e, max(np.e, nn.e)) > kFdBad / 2) B.re = B.im = __longlong_as_double(0x7FF8000000000000LL);
+    // (den also beyond FP64's range: its reciprocal would vanish beside a finite B)
+    if (den.e > 1020 || max(np.e, nn.e) > kFdBad / 2) B.re = B.im = __longlong_as_double(0x7FF8000000000000LL);
     out.B = B;
     out.q = fd_rcp(den);
     out.L = dc{0.0, 0.0};

@@ -254,3 +254,25 @@ def test_lambda_outside_the_usual_range(name, lam, mixed):
         assert np.all(np.abs(a - b) <= 1e-12 * np.abs(b).max())
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("scale", [1e70, 1e75, 1e78, 1e90, 1e120, 1e-70, 1e-78])
+def test_deformed_coefficients_of_any_size(scale):
+    """F^-2 at large and small kinematics: the general kernel's sums where it has
+    them, and its status where the square of F^2 leaves FP64's range."""
+    I, lo = w.box_massless(deform=True), -2
+    g = Gpu()
+    try:
+        iid, gid = g.load(I), g.load(general(I, Fraction(1, 10 ** 250)))
+        qmc.qmc_set_kinematics(g.ctx, np.array([[7.0 * scale, -2.5 * scale]]))
+        specs = [dict(integral_id=iid, sector=s, point=0, shifts=2, n=1009, seed=3, stream=s,
+                      **{"lambda": 0.5 / scale}) for s in range(len(I.sectors))]
+        a, fa, ra = g.eval(iid, specs, lo, 3)
+        b, fb, rb = g.eval(gid, [dict(sp, integral_id=gid) for sp in specs], lo, 3)
+        assert ra == rb and rb == (0 if 1e-76 < scale < 1e76 else NONFINITE)
+        if rb == 0:
+            a, b = a.reshape(-1, 3, 2), b.reshape(-1, 3, 2)
+            top = np.abs(b).max(axis=(0, 2))
+            assert np.all(top > 0) and np.all(np.abs(a - b).max(axis=(0, 2)) <= 1e-11 * top)
+    finally:
+        g.close()
