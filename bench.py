@@ -110,9 +110,9 @@ PROFILED = {
     # double box, n = 1000003, m = 32 (the default line): traffic from a 1-pass
     # capture of one full launch; instruction counts and pipe activity from the
     # full capture of the same kernel at n = 20011 (per evaluation, the same code)
-    ("d3f921baac652e14754100c686ca113859c905de", "box2L_planar_massless", "fp64", "iterative", 1000003): {
-        "traffic": 111145199104 + 2148485046272, "fp64_executed_flops_per_eval": 269.4, "fp64_pipe_busy": 0.477,
-        "warp_inst_per_eval": 386.3, "issue_busy": 0.529},
+    ("a464297fad1a7504e279cecc8fc60f57c341bbeb", "box2L_planar_massless", "fp64", "iterative", 1000003): {
+        "traffic": 110843129600 + 2146234152448, "fp64_executed_flops_per_eval": 269.4, "fp64_pipe_busy": 0.475,
+        "warp_inst_per_eval": 385.9, "issue_busy": 0.526},
 }
 
 # What the roofline counts (flops.py): the FP64 operations that the evaluators of

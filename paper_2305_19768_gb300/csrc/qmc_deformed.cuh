@@ -35,7 +35,9 @@
 // pipe 87 % busy); massless box, 16 physical points at n = 4001, 5.9e8 (555)
 // -> 1.06e9 (453) with complex logarithms of the factors' product -> 1.86e9
 // (204, 78 %); the massive box in mixed precision, 256 points at n = 1009,
-// 2.85e9 -> 6.6e9.
+// 2.85e9 -> 6.6e9. Arguments and their sums to FP64's relative precision at every
+// size (qmc_iarg.h; 2^-57 fixed point before): the massless box at 60 points
+// 1.94e9 -> 1.87e9.
 // MIXED: derivatives of F and U(z), F(z) from FP32 monomial products in the
 // order of the general mixed kernel, everything after them in FP64.
 
