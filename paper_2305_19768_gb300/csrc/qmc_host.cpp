@@ -711,6 +711,8 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
     // size, and the power-table rows (the largest exponent among the sectors:
     // fewer rows, less shared memory per block, more resident blocks)
     std::vector<std::map<uint64_t, uint64_t>> lattices(2 * QMC_NCLASS);
+    std::map<uint64_t, uint64_t>::value_type *last = nullptr;   // the last job's entry
+    int last_slot = -1;
     std::vector<int> prows(2 * QMC_NCLASS, 1);
     std::vector<int> own(njobs, -1);   // index among the plan's jobs
     int nown = 0, max_point = -1;
@@ -752,7 +754,11 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
             return fail(ctx, QMC_E_INVAL, "job %d: orders %d..%d with %d poles exceed the evaluator's series length %d",
                         i, lo, hi, S.ns, qmc_class_lmax(cls));
         const int slot = 2 * cls + (fx_order_ok(hi, cls) && (fd_job_ok(S, cls) || fx_job_ok(ctx, S, cls, J.point)) ? 1 : 0);
-        lattices[slot][J.n] += (uint64_t)J.shifts;
+        if (slot != last_slot || last->first != J.n) {
+            last = &*lattices[slot].emplace(J.n, 0).first;
+            last_slot = slot;
+        }
+        last->second += (uint64_t)J.shifts;
         prows[slot] = std::max(prows[slot], S.prow);
         if (mine && !mine[i]) continue;
         own[i] = nown++;

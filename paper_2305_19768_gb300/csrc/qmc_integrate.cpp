@@ -389,8 +389,13 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
     std::vector<double> tau(slots.size(), 1.0);
     std::vector<double> amp_val((size_t)npts * namp * norders * 2), amp_var((size_t)npts * namp * norders);
     std::vector<double> amp_vre((size_t)npts * namp * norders), amp_vim((size_t)npts * namp * norders);
-    // evaluate host jobs (this rank's share of `all`, whose members are marked in
-    // `own`): the caller's evaluator or one GPU plan; per-shift sums, per-job
+    auto create_share = [&](const std::vector<qmc_job> &all, const std::vector<unsigned char> &own,
+                            const std::vector<qmc_job> &jobs, qmc_plan **plan) {
+        return world > 1 ? plan_create_share(ctx, all.data(), (int)all.size(), own.data(), slo, sn, plan)
+                         : qmc_plan_create(ctx, jobs.data(), (int)jobs.size(), slo, sn, plan);
+    };
+    // evaluate host jobs (with several ranks this rank's share of `all`, whose
+    // members are marked in `own`): the caller's evaluator or one GPU plan; per-shift sums, per-job
     // sign-check failures, evaluator seconds per class (slot QMC_NCLASS: one
     // figure for all classes, from an evaluator that is not timed per class)
     auto eval_jobs = [&](const std::vector<qmc_job> &all, const std::vector<unsigned char> &own,
@@ -410,7 +415,7 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
             return QMC_OK;
         }
         qmc_plan *plan = nullptr;
-        int rc = plan_create_share(ctx, all.data(), (int)all.size(), own.data(), slo, sn, &plan);
+        int rc = create_share(all, own, jobs, &plan);
         if (rc) return rc;
         rc = qmc_plan_run(plan, nullptr, nullptr);
         uint64_t sf = 0;
@@ -469,8 +474,10 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
                     J.lambda[j] = sl.lambda;
                     J.z[j] = zc[(size_t)c * 6 + j];
                 }
-                all.push_back(J);
-                own.push_back(owner[u] == rank);
+                if (world > 1) {
+                    all.push_back(J);
+                    own.push_back(owner[u] == rank);
+                }
                 if (owner[u] == rank) jobs.push_back(J);
             }
             if (owner[u] != rank) continue;
@@ -489,7 +496,7 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
                 if (rc && rc != QMC_E_SIGN_CHECK) return fail(ctx, rc, "qmc_integrate: the evaluator failed (%d)", rc);
             } else {
                 qmc_plan *plan = nullptr;
-                int rc = plan_create_share(ctx, all.data(), (int)all.size(), own.data(), slo, sn, &plan);
+                int rc = create_share(all, own, jobs, &plan);
                 if (rc) return rc;
                 rc = qmc_plan_run(plan, nullptr, nullptr);
                 if (!rc) rc = qmc_plan_results(plan, est.data(), nullptr);
@@ -558,8 +565,10 @@ int qmc_integrate_ex(qmc_ctx *ctx, const qmc_sum_spec *spec, double epsrel, doub
                         J.lambda[j] = sl.lambda;
                         J.z[j] = median ? sl.z[j] : 0;
                     }
-                    all.push_back(J);
-                    own.push_back(owner[u] == rank);
+                    if (world > 1) {
+                        all.push_back(J);
+                        own.push_back(owner[u] == rank);
+                    }
                     if (owner[u] != rank) continue;
                     jobs.push_back(J);
                     mine.push_back(u);
