@@ -434,7 +434,8 @@ __device__ __forceinline__ FdCorner fd_corner(const FdPoint &P, const FdOps &o, 
         const fc f = fd_polyc<BLOCK>(S.nU, S.nF);
         F = dc{fd_to_double(f.re), fd_to_double(f.im)};
     }
-    if (__double_as_longlong(F.im) > 0) ++signfail;
+    // F.im > 0 on the bits (not for NaN)
+    if ((uint64_t)__double_as_longlong(F.im) - 1ULL < 0x7FF0000000000000ULL) ++signfail;
     // The corner value J / prod rho (kept singular) prod z^a (regular) U^u0
     // F^f0, a factor x^-e as conj(x)^e / |x|^2e: B collects the complex
     // products and q the real ones, in mantissas. Its exponent

@@ -276,3 +276,22 @@ def test_deformed_coefficients_of_any_size(scale):
             assert np.all(top > 0) and np.all(np.abs(a - b).max(axis=(0, 2)) <= 1e-11 * top)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("s", [1e30, 1e60, 1e160])
+def test_sign_failures_where_F_is_not_a_number(s, mixed):
+    """Points whose F is NaN fail no sign check: the same counts as the general
+    kernel's, which serves a window up to eps^2."""
+    I = w.box_massive()
+    g = Gpu(precision=qmc.QMC_PRECISION_MIXED if mixed else qmc.QMC_PRECISION_FP64)
+    try:
+        iid = g.load(I)
+        qmc.qmc_set_kinematics(g.ctx, np.array([[s, -0.3 * s]]))
+        specs = [dict(integral_id=iid, sector=i, point=0, shifts=2, n=1009, seed=3, stream=i, **{"lambda": 0.5})
+                 for i in range(len(I.sectors))]
+        _, fa, ra = g.eval(iid, specs, 0, 1)
+        _, fb, rb = g.eval(iid, specs, 0, 3)
+        assert fa == fb and (ra == rb or not mixed)
+    finally:
+        g.close()
