@@ -110,8 +110,8 @@ PROFILED = {
     # double box, n = 1000003, m = 32 (the default line): traffic from a 1-pass
     # capture of one full launch; instruction counts and pipe activity from the
     # full capture of the same kernel at n = 20011 (per evaluation, the same code)
-    ("a464297fad1a7504e279cecc8fc60f57c341bbeb", "box2L_planar_massless", "fp64", "iterative", 1000003): {
-        "traffic": 110843129600 + 2146234152448, "fp64_executed_flops_per_eval": 269.4, "fp64_pipe_busy": 0.475,
+    ("4daa997a5ae61b5cdafc305f48360037b40f289d", "box2L_planar_massless", "fp64", "iterative", 1000003): {
+        "traffic": 110671104000 + 2144790853376, "fp64_executed_flops_per_eval": 269.4, "fp64_pipe_busy": 0.475,
         "warp_inst_per_eval": 385.9, "issue_busy": 0.526},
 }
 
