@@ -96,9 +96,10 @@ struct ClassLaunch {
     // jobs for the evaluators of qmc_real.cuh or qmc_deformed.cuh; `general`:
     // the kinematics set since no longer qualify, and the general kernel runs
     // instead, with the tiles G that it would have had from the start (its job
-    // table is made when it is first needed: `gready`)
-    bool fx = false, general = false, gready = false;
+    // table and partial sums are made when they are first needed)
+    bool fx = false, general = false;
     QmcLaunch G{};
+    unsigned char *d_general = nullptr;
     int gblock = 128, gppt = 16;
     struct FxJob {
         int integral, sector, point;

@@ -480,22 +480,35 @@ uint64_t retile(QmcJobDev &D, uint64_t tile_k, uint64_t begin) {
 
 // After new kinematics: which launches' jobs still qualify for the integer
 // evaluator; the others take the general kernel, whose job table is made from the
-// launch's own the first time
+// launch's own the first time (with a plan's own allocation it would cost every
+// plan: beyond 1 MB an allocation takes 70 us more)
 int plan_requalify(qmc_plan *plan) {
     qmc_ctx *ctx = plan->ctx;
     for (ClassLaunch &c : plan->launches) {
         c.general = false;
         for (const ClassLaunch::FxJob &J : c.fx_jobs)
             c.general = c.general || !fx_job_ok(ctx, ctx->integrals[J.integral].sectors[J.sector], c.cls, J.point);
-        if (!c.general || c.gready) continue;
+        if (!c.general || c.d_general) continue;
         std::vector<QmcJobDev> v(c.orig.size());
         const size_t bytes = v.size() * sizeof(QmcJobDev);
         CUDA_TRY(ctx, cudaMemcpy(v.data(), c.L.jobs, bytes, cudaMemcpyDeviceToHost));
         uint64_t tiles = 0;
-        for (QmcJobDev &D : v) tiles = retile(D, c.G.tile_k, tiles);
-        CUDA_TRY(ctx, cudaMemcpy(const_cast<QmcJobDev *>(c.G.jobs), v.data(), bytes, cudaMemcpyHostToDevice));
-        CUDA_TRY(ctx, cudaStreamSynchronize(cudaStreamLegacy));
-        c.gready = true;
+        for (QmcJobDev &D : v) tiles = retile(D, (uint64_t)c.gblock * c.gppt, tiles);
+        const size_t part_at = (bytes + 255) / 256 * 256;
+        unsigned char *d = nullptr;
+        CUDA_TRY(ctx, cudaMalloc(&d, part_at + std::max<uint64_t>(1, tiles) * 2 * plan->norders * sizeof(double)));
+        cudaError_t e = cudaMemcpy(d, v.data(), bytes, cudaMemcpyHostToDevice);
+        if (!e) e = cudaStreamSynchronize(cudaStreamLegacy);
+        if (e) {
+            cudaFree(d);
+            return fail(ctx, QMC_E_CUDA, "qmc_set_kinematics: %s", cudaGetErrorString(e));
+        }
+        c.G = c.L;
+        c.G.tile_k = (uint32_t)(c.gblock * c.gppt);
+        c.G.ntiles = tiles;
+        c.G.jobs = (const QmcJobDev *)d;
+        c.G.partials = (double *)(d + part_at);
+        c.d_general = d;
     }
     return QMC_OK;
 }
@@ -506,6 +519,7 @@ constexpr size_t kOneCopy = 4096;   // results up to this many numbers come back
 void free_plan_buffers(qmc_plan *p) {
     if (p->gexec) cudaGraphExecDestroy(p->gexec);
     p->gexec = nullptr;
+    for (ClassLaunch &c : p->launches) cudaFree(c.d_general);
     p->launches.clear();
     cudaFree(p->d_arena);
     if (p->ev0) cudaEventDestroy(p->ev0);
@@ -846,12 +860,8 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
         }
         const int prow = prows[slot];
         int occ = 1;
-        uint64_t gtiles = 0;
-        if (!c.fx_jobs.empty()) {
-            c.gblock = c.block;
-            c.gppt = c.ppt;
-            for (QmcJobDev D : v) gtiles += retile(D, (uint64_t)c.gblock * c.gppt, 0);
-        }
+        c.gblock = c.block;
+        c.gppt = c.ppt;
         if (c.fx) {
             c.block = qmc_class_dmax(cls) > 3 ? QMC_FX6_BLOCK : QMC_FX3_BLOCK;   // their one block size
             occ = std::max(1, qmc_k_occupancy_real(cls, hi, prow));
@@ -875,35 +885,29 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
         L.prow = prow;
         L.mone = -1.0;
         L.nzero = -0.0;
-        c.G = L;
-        c.G.ntiles = gtiles;
-        c.G.tile_k = (uint32_t)(c.gblock * c.gppt);
         p->launches.push_back(c);
     }
     // One allocation and one copy for everything a plan holds on the device
     // (six, and a copy or a fill each, took 32 us of a one-shot call's 90 for a
     // plan's set-up and release; with this the call takes 70). In order:
-    //   [jobs]  [queues, failure counts, status | results]  [partial sums]  [jobs of G]
+    //   [jobs]  [queues, failure counts, status | results]  [partial sums]
     // so that one fill clears what a run must find at zero and a small plan's
     // status and results come back in one copy.
     {
         auto up = [](size_t b) { return (b + 255) / 256 * 256; };
         size_t zero = 0, njob_bytes = 0, part = 0;
-        size_t gjob_bytes = 0;
-        std::vector<size_t> at_queue, at_jobs, at_part, at_gjobs;
+        std::vector<size_t> at_queue, at_jobs, at_part;
         for (const ClassLaunch &c : p->launches) {
             at_queue.push_back(zero);
             zero += 16 + (c.orig.size() * sizeof(unsigned int) + 15) / 16 * 16;
             at_jobs.push_back(njob_bytes);
             njob_bytes += up(c.orig.size() * sizeof(QmcJobDev));
             at_part.push_back(part);
-            part += up(std::max<uint64_t>(1, std::max(c.L.ntiles, c.G.ntiles)) * 2 * norders * sizeof(double));
-            at_gjobs.push_back(gjob_bytes);
-            if (!c.fx_jobs.empty()) gjob_bytes += up(c.orig.size() * sizeof(QmcJobDev));
+            part += up(std::max<uint64_t>(1, c.L.ntiles) * 2 * norders * sizeof(double));
         }
         zero = up(zero + kStatusBytes);   // the status ends the cleared part
         const size_t part_at = up(njob_bytes + zero + std::max<size_t>(1, p->out_size) * sizeof(double));
-        PLAN_TRY(cudaMalloc(&p->d_arena, part_at + part + gjob_bytes));
+        PLAN_TRY(cudaMalloc(&p->d_arena, part_at + part));
         p->d_zero = p->d_arena + njob_bytes;
         p->zero_bytes = zero;
         p->d_status = (unsigned long long *)(p->d_zero + zero - kStatusBytes);
@@ -921,11 +925,6 @@ int plan_create_share(qmc_ctx *ctx, const qmc_job *jobs, int njobs, const unsign
             c.L.status = p->d_status;
             c.L.out = p->d_out;
             c.L.job_fail = c.d_jobfail;
-            c.G.queue = c.L.queue;
-            c.G.jobs = (const QmcJobDev *)(p->d_arena + part_at + part + at_gjobs[k]);
-            c.G.partials = c.L.partials;
-            c.G.status = c.L.status;
-            c.G.job_fail = c.L.job_fail;
             ++k;
         }
         PLAN_TRY(cudaMemcpy(p->d_arena, head.data(), head.size(), cudaMemcpyHostToDevice));
@@ -987,7 +986,7 @@ int plan_enqueue(qmc_plan *plan, double *out, cudaStream_t st, bool capturing) {
         L.monos = ctx->d_monos;
         L.kin = ctx->d_kin;
         CUDA_TRY(ctx, cudaEventRecordWithFlags(plan->kev[2 * i], cs, evflags));
-        if (c.general && !c.gready) return fail(ctx, QMC_E_CUDA, "qmc_plan_run: the kinematics were not set completely");
+        if (c.general && !c.d_general) return fail(ctx, QMC_E_CUDA, "qmc_plan_run: the kinematics were not set completely");
         if (L.ntiles > 0) {
             int rc;
             if (c.general) {
